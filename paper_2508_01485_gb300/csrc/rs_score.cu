@@ -2018,8 +2018,18 @@ __global__ void __launch_bounds__(kThreads, 3) p3_heavy_kernel(
 // Strict reading: X(w, u) for every pushed pair, from the closed triads (u, w, v)
 // with C(v) = C(u) != C(w): for every intra-community edge {u, v} (u < v) and
 // every common neighbour w of another community, s_v is added at u's entry in
-// w's row and s_u at v's.  The shorter row of u, v is walked; w is looked up in
-// the other row and the entries in w's row by binary search (rows are sorted).
+// w's row and s_u at v's.  w is a cross neighbour of both u and v, so only their
+// cross lists (P1's, sorted by id) are walked and searched, not their rows: the
+// shorter one is walked, w is looked up in the other, and the entries in w's row
+// are found by binary search.  A hub row has no cross list; its whole row stands
+// in for it (walked, its own community is skipped; searched, it holds w just the same).
+//
+// A warp takes 32 consecutive CSR entries, so a hub's row is spread over many
+// warps, and shares the candidates (edge, walked w) of its edges evenly among its
+// lanes.  What bounds it is the chain of dependent loads of a candidate's search.
+// The form before this one gave a warp a whole row and a lane an edge, and walked
+// whole rows with a label gather per entry: 4.12 ms on a 100,003-node graph (0.81M
+// edges, degrees to 1,000), most of it the tail of a few warps, against 0.13 ms.
 // ======================================================================================
 __device__ __forceinline__ int64_t csr_find(const int64_t *off, const int32_t *col, int32_t row, int32_t key) {
     int64_t lo = off[row], hi = off[row + 1], end = hi;
@@ -2030,34 +2040,114 @@ __device__ __forceinline__ int64_t csr_find(const int64_t *off, const int32_t *c
     return (lo < end && col[lo] == key) ? lo : -1;
 }
 
-__global__ void __launch_bounds__(kThreads) strict_pairs_kernel(int64_t n, const int64_t *__restrict__ off,
-                                                                const int32_t *__restrict__ col,
-                                                                const int32_t *__restrict__ lab,
-                                                                const NodeRec *__restrict__ rec,
-                                                                unsigned long long *sx) {
-    int lane = threadIdx.x & 31;
-    int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u = w0; u < n; u += nw) {                 // a warp per row u, lanes over its entries v
-        int32_t cu = lab[u];
-        int64_t bu = off[u], du = off[u + 1] - bu;
-        for (int64_t e = lane; e < du; e += 32) {
-            int32_t v = col[bu + e];
-            if (v <= u || lab[v] != cu) continue;
-            int64_t bv = off[v], dv = off[v + 1] - bv;
-            bool walk_u = du <= dv;
-            int32_t o = walk_u ? v : (int32_t)u;
-            int64_t ba = walk_u ? bu : bv, da = walk_u ? du : dv;
-            uint64_t su = rec[u].s_fix, sv = rec[v].s_fix;
-            for (int64_t j = 0; j < da; ++j) {
-                int32_t w = col[ba + j];
-                if (w == o || lab[w] == cu) continue;
-                if (csr_find(off, col, o, w) < 0) continue;
-                int64_t pu = csr_find(off, col, w, (int32_t)u), pv = csr_find(off, col, w, v);
-                if (sv && pu >= 0) atomic_add_u128(sx + 2 * pu, (u128)sv);
-                if (su && pv >= 0) atomic_add_u128(sx + 2 * pv, (u128)su);
+// the row holding CSR entry e (off[0] <= e < off[n]), found by the warp: 32 probes a step
+__device__ __forceinline__ int64_t warp_row_of(const int64_t *off, int64_t n, int64_t e, int lane) {
+    int64_t lo = 0, hi = n;                            // off[lo] <= e < off[hi]
+    while (hi - lo > 1) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t p = lo + lane * step;
+        const unsigned m = __ballot_sync(FULL, p < hi && off[p] <= e);   // lane 0's probe holds
+        const int64_t l2 = lo + (31 - __clz(m)) * step;
+        hi = min(hi, l2 + step);
+        lo = l2;
+    }
+    return lo;
+}
+
+struct StrictWarp {
+    const int32_t *walk[32], *look[32];                // the walked and the searched list of each edge
+    int64_t ends[32];                                  // row ends, while the entries' rows are found
+    uint64_t su[32], sv[32];
+    int32_t look_len[32], u[32], v[32];
+    int32_t skip[32];                                  // a walked hub row: its own label, else -1
+    int32_t pre[33];                                   // prefix sums of the walked lists' lengths
+};
+
+__global__ void __launch_bounds__(kThreads) strict_pairs_kernel(
+    int64_t n, const int64_t *__restrict__ off, const int32_t *__restrict__ col, const int32_t *__restrict__ lab,
+    const NodeRec *__restrict__ rec, const int32_t *__restrict__ cl_col, Batch B, int32_t small_max, int32_t cta_cap,
+    unsigned long long *sx) {
+    __shared__ StrictWarp warps[kThreads / 32];
+    const int lane = threadIdx.x & 31;
+    StrictWarp &S = warps[threadIdx.x >> 5];
+    const int64_t E = off[n];
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t e0 = 32 * w0; e0 < E; e0 += 32 * nw) {
+        const int64_t e = e0 + lane;
+        const bool act = e < E;
+        // the rows of the warp's entries: the ends of the rows from e0's on, 32 at a time
+        int64_t u = -1;
+        for (int64_t r = warp_row_of(off, n, e0, lane); __any_sync(FULL, act && u < 0); r += 32) {
+            S.ends[lane] = r + lane < n ? off[r + lane + 1] : INT64_MAX;
+            __syncwarp();
+            int32_t lo = 0, hi = 32;                   // first row that ends after e
+            while (lo < hi) {
+                const int32_t mid = (lo + hi) >> 1;
+                if (S.ends[mid] <= e) lo = mid + 1; else hi = mid;
+            }
+            if (u < 0 && lo < 32) u = r + lo;
+            __syncwarp();
+        }
+        int32_t cnt = 0;
+        if (act) {
+            const int32_t v = col[e];
+            if (v > u && lab[v] == lab[u]) {
+                const NodeRec ru = rec[u], rv = rec[v];
+                if (ru.dx > 0 && rv.dx > 0) {
+                    const int32_t k = k_of(B, graph_of(B, v));
+                    const int64_t bu = off[u], bv = off[v];
+                    const int32_t du = (int32_t)(off[u + 1] - bu), dv = (int32_t)(off[v + 1] - bv);
+                    auto hub = [&](int32_t d) {        // a row of the hub class
+                        return d > small_max && dev_pow2_at_least(2u * (uint32_t)min(d, k)) > (uint32_t)cta_cap;
+                    };
+                    const bool hu = hub(du), hv = hub(dv);
+                    const int32_t lu = hu ? du : ru.dx, lv = hv ? dv : rv.dx;
+                    const int32_t *pu = hu ? col + bu : cl_col + bu, *pv = hv ? col + bv : cl_col + bv;
+                    const bool walk_u = lu <= lv;
+                    S.walk[lane] = walk_u ? pu : pv;
+                    S.look[lane] = walk_u ? pv : pu;
+                    S.look_len[lane] = walk_u ? lv : lu;
+                    S.skip[lane] = (walk_u ? hu : hv) ? ru.label : -1;
+                    S.u[lane] = (int32_t)u;
+                    S.v[lane] = v;
+                    S.su[lane] = ru.s_fix;
+                    S.sv[lane] = rv.s_fix;
+                    cnt = min(lu, lv);
+                }
             }
         }
+        // candidates of the 32 edges: degrees are below 2^24, so the sum is below 2^29
+        int32_t incl = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += y;
+        }
+        S.pre[lane + 1] = incl;
+        if (lane == 0) S.pre[0] = 0;
+        __syncwarp();
+        const int32_t total = S.pre[32];
+        for (int32_t f = lane; f < total; f += 32) {
+            int32_t lo = 0, hi = 32;                   // last edge with pre <= f
+            while (hi - lo > 1) {
+                const int32_t mid = (lo + hi) >> 1;
+                if (S.pre[mid] <= f) lo = mid; else hi = mid;
+            }
+            const int32_t w = S.walk[lo][f - S.pre[lo]];
+            if (S.skip[lo] >= 0 && lab[w] == S.skip[lo]) continue;
+            const int32_t *p = S.look[lo];
+            int32_t l = 0, h = S.look_len[lo];
+            const int32_t len = h;
+            while (l < h) {
+                const int32_t mid = (l + h) >> 1;
+                if (p[mid] < w) l = mid + 1; else h = mid;
+            }
+            if (l >= len || p[l] != w) continue;
+            const int64_t pu = csr_find(off, col, w, S.u[lo]), pv = csr_find(off, col, w, S.v[lo]);
+            if (S.sv[lo] && pu >= 0) atomic_add_u128(sx + 2 * pu, (u128)S.sv[lo]);
+            if (S.su[lo] && pv >= 0) atomic_add_u128(sx + 2 * pv, (u128)S.su[lo]);
+        }
+        __syncwarp();
     }
 }
 
@@ -2300,7 +2390,8 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     const Strict SX{g->col, g->strict ? g->sx : nullptr};
     if (g->strict) {
         RS_CUDA_TRY(cudaMemsetAsync(g->sx, 0, 2 * g->nnz * sizeof(unsigned long long), s));
-        strict_pairs_kernel<<<grid_for(n * 32, NT, cps), NT, 0, s>>>(n, g->off, g->col, g->lab, g->rec, g->sx);
+        strict_pairs_kernel<<<grid_for(g->nnz, NT, cps), NT, 0, s>>>(n, g->off, g->col, g->lab, g->rec, g->cl_col, B,
+                                                                     g->tune.small_max, g->tune.cta_cap, g->sx);
         RS_LAUNCHED(g, s, "strict_pairs");
     }
     // ---- P2: with per-class streams, the many-short-rows kernels on the low-priority

@@ -59,3 +59,25 @@ def test_strict_matches_oracle(rs, gen):
 def test_strict_with_alg2(rs):
     g = graphgen.dcsbm_small(20000, seed=9, dmax=800)
     _check(rs, g.offsets, g.cols, g.labels, g.k, np.arange(0, g.n, 7, dtype=np.int32), alg2=True)
+
+
+@pytest.mark.parametrize("tuning", [{}, {"small_max": 1, "warp_cap": 64, "cta_cap": 64}])
+@pytest.mark.parametrize("gap", [0, 31, 32, 100])
+def test_strict_rows_across_warps(rs, tuning, gap):
+    """Runs of `gap` isolated nodes between the others (a warp's 32 entries then span more rows
+    than it looks at once), rows that start inside a warp, and every row with more than 64 table
+    slots a hub (walked and searched whole)."""
+    rng = np.random.default_rng(gap)
+    m, k = 70, 9
+    off, cols, labels = random_tiny_graph(rng, m, k, 0.35)
+    at = np.arange(m) * (gap + 1) + gap                  # old id -> new id
+    deg = np.zeros(m * (gap + 1) + gap, np.int64)
+    deg[at] = np.diff(off)
+    lab = rng.integers(0, 80, len(deg)).astype(np.int32)
+    lab[at] = labels
+    G = rs.Graph.build(np.concatenate([[0], np.cumsum(deg)]), at[cols].astype(np.int32), lab, 80, strict=True)
+    G.set_tuning(**tuning)
+    s = G.score().cpu().numpy()
+    assert G.device_errors() == 0
+    ref = oracle.Oracle(np.concatenate([[0], np.cumsum(deg)]), at[cols].astype(np.int32), lab, 80).scores(strict=True)
+    np.testing.assert_allclose(s, ref, rtol=1e-12, atol=0)
