@@ -3,16 +3,26 @@
 //
 // Each node is a unique 96-bit key (bits(score) << 32 | ~id): for scores >= 0
 // the IEEE bit pattern orders like the value, and ~id makes smaller ids rank
-// higher among equal scores.  One cooperative launch (one 1024-thread CTA per
-// SM, grid-wide barriers from cooperative groups) runs a most-significant-digit
-// radix select with 12-bit digits:
-//   per level (three grid-wide barriers): privatised shared-memory histograms
-//   of the digit over the current candidates, merged into a global histogram;
-//   CTA 0 finds the bucket that holds the K-th key; keys of higher buckets are
-//   final ("sure"), keys of that bucket stay candidates, both appended with one
-//   atomic per warp, while the global histogram is cleared for the next level.
-// As soon as the sure keys and the candidates fit a small shared-memory sort
-// (about 2K keys), CTA 0 sorts them (bitonic) and writes the first K.
+// higher among equal scores.  One cooperative launch (at most one 1024-thread
+// CTA per SM, grid-wide barriers from cooperative groups) runs a
+// most-significant-digit radix select with 12-bit digits:
+//   per level (two grid-wide barriers): privatised shared-memory histograms of
+//   the digit over the current candidates, merged into a global histogram; every
+//   CTA finds the bucket that holds the K-th key in it for itself; keys of higher
+//   buckets are final ("sure"), keys of that bucket stay candidates, both appended
+//   with one atomic per warp.  The levels take turns with two global histograms:
+//   one is cleared while the other is read.
+// As soon as the sure keys and the candidates fit the final ranking (16,384 keys
+// at most) the grid ranks them: runs of 256 keys are sorted, a run per CTA, and
+// every key's rank is its place in its own run plus the number of greater keys in
+// each other run (binary searches, the runs spread over the lanes), which is where
+// it is written.
+//
+// Latency bounds it: the passes over the scores are a few microseconds, the rest are
+// barriers and the launch.  Against the form before this one (three barriers a level, a
+// bitonic sort of all the keys by one CTA): 31 -> 22 us for n = 2,000, k = 50 (two plain
+// launches), 52 -> 38 us for n = 1,000,000, k = 1,000, 260 -> 54 us for n = 1,000,000,
+// k = 10,000 and 112 -> 74 us for n = 8,000,000, k = 1,000.
 #include <algorithm>
 #include <cooperative_groups.h>
 
@@ -28,18 +38,14 @@ constexpr int kTkThreads = 1024;
 constexpr int kBits = 12;
 constexpr int kBins = 1 << kBits;
 constexpr int kLevels = 96 / kBits;
-constexpr int kSortMax = 16384;   // largest K, and the size of the final sort
-constexpr size_t kTkSmem = (size_t)kSortMax * (8 + 4);
+constexpr int kSortMax = 16384;   // largest K, and the most keys the final ranking takes
+constexpr int kRun = 256;         // keys per sorted run of the final ranking
 
-enum { C_NEED = 0, C_SURE = 1, C_SEL = 2, C_NEXT = 3 /* and 4: candidate counters of even / odd levels */ };
+enum { C_SURE = 0, C_NEXT = 1 /* and 2: candidate counters of even / odd levels */ };
 
-// keys left when the selection stops and sorts: a bitonic sort costs log^2 of its
-// size in barriers, so another radix level is cheaper than sorting much more than K
-__host__ __device__ __forceinline__ int sort_target(int k) {
-    int p = 2048;
-    while (p < 2 * k && p < kSortMax) p <<= 1;
-    return p;
-}
+// keys left when the selection stops and ranks: ranking 8,192 keys costs less than
+// another radix level does, and 2 K keys are met for every K up to kSortMax / 2
+__host__ __device__ __forceinline__ int rank_target(int k) { return 2 * k > 8192 ? kSortMax : 8192; }
 
 // digit `level` (0 = most significant) of the 96-bit key (key64 : ~id)
 __device__ __forceinline__ uint32_t digit_of(unsigned long long key, uint32_t nid, int level) {
@@ -58,7 +64,7 @@ struct TkArgs {
     int32_t k;
     int32_t *ids_out;
     double *scores_out;
-    uint32_t *hist;                 // kBins
+    uint32_t *hist;                 // 2 x kBins
     int *ctrl;
     unsigned long long *key[2];     // candidate buffers (n each)
     uint32_t *nid[2];
@@ -77,28 +83,6 @@ __device__ __forceinline__ void load_item(const TkArgs &A, int level, int src, i
     }
 }
 
-// descending bitonic sort of (key, nid) pairs in shared memory, P a power of two;
-// the pair of each compare-exchange comes from shifts and masks (st is a power of two)
-__device__ void block_sort_desc(unsigned long long *key, uint32_t *nid, int P) {
-    for (int size = 2; size <= P; size <<= 1)
-        for (int st = size >> 1; st; st >>= 1) {
-            const int lst = __ffs(st) - 1;
-            const bool flip = st == (size >> 1);
-            for (int i = threadIdx.x; i < P / 2; i += blockDim.x) {
-                int base = (i >> lst) << (lst + 1), o = i & (st - 1);
-                int lo = base + o;
-                int hi = flip ? base + 2 * st - 1 - o : lo + st;
-                unsigned long long kl = key[lo], kh = key[hi];
-                uint32_t nl = nid[lo], nh = nid[hi];
-                if (kl < kh || (kl == kh && nl < nh)) {
-                    key[lo] = kh; key[hi] = kl;
-                    nid[lo] = nh; nid[hi] = nl;
-                }
-            }
-            __syncthreads();
-        }
-}
-
 // append the flagged items of a warp to buf at a position drawn with one atomic
 // per warp (every lane of the warp calls; order inside the buffer is free)
 __device__ __forceinline__ void warp_append(bool flag, unsigned long long key, uint32_t nid, int *counter,
@@ -115,60 +99,141 @@ __device__ __forceinline__ void warp_append(bool flag, unsigned long long key, u
     }
 }
 
+// keys of the sorted (descending) run key/nid[0, len) that rank above (k, id)
+__device__ __forceinline__ int greater_in_run(const unsigned long long *key, const uint32_t *nid, int len,
+                                              unsigned long long k, uint32_t id) {
+    int lo = 0, hi = len;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const unsigned long long x = key[mid];
+        if (x > k || (x == k && nid[mid] > id)) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// The final ranking, step 1: the ns sure keys and total - ns items of buffer src (level 0:
+// of the scores), as runs of kRun keys, each sorted by one CTA into the candidate buffer not
+// in use; a key's place is the number of greater keys in its run, counted by four threads.
+// sh: 4 kRun words.
+__device__ __forceinline__ void sort_runs(const TkArgs &A, int level, int src, int ns, int total, uint32_t *sh) {
+    const int tid = threadIdx.x;
+    const int runs = (total + kRun - 1) / kRun;
+    unsigned long long *wkey = (unsigned long long *)sh;
+    uint32_t *wnid = sh + 2 * kRun, *wplace = wnid + kRun;
+    for (int r = blockIdx.x; r < runs; r += gridDim.x) {
+        const int len = min(kRun, total - r * kRun);
+        __syncthreads();
+        if (tid < len) {
+            const int i = r * kRun + tid;
+            unsigned long long key; uint32_t nid;
+            if (i < ns) { key = A.skey[i]; nid = A.snid[i]; }
+            else load_item(A, level, src, i - ns, key, nid);
+            wkey[tid] = key; wnid[tid] = nid; wplace[tid] = 0;
+        }
+        __syncthreads();
+        constexpr int kParts = kTkThreads / kRun;
+        const int i = tid & (kRun - 1), share = tid / kRun;
+        if (i < len) {
+            const unsigned long long key = wkey[i]; const uint32_t nid = wnid[i];
+            uint32_t above = 0;
+            const int hi = min(len, (share + 1) * (kRun / kParts));
+            for (int j = share * (kRun / kParts); j < hi; ++j)
+                above += wkey[j] > key || (wkey[j] == key && wnid[j] > nid);
+            if (above) atomicAdd(&wplace[i], above);
+        }
+        __syncthreads();
+        if (tid < len) {
+            const int p = r * kRun + (int)wplace[tid];
+            A.key[src ^ 1][p] = wkey[tid]; A.nid[src ^ 1][p] = wnid[tid];
+        }
+    }
+}
+
+// step 2: every key's rank, by `lanes` lanes per key, each over every lanes-th run; the keys of
+// rank below K are written at their rank
+__device__ __forceinline__ void rank_runs(const TkArgs &A, int src, int total) {
+    const unsigned long long *rkey = A.key[src ^ 1];
+    const uint32_t *rnid = A.nid[src ^ 1];
+    const int runs = (total + kRun - 1) / kRun, lane = threadIdx.x & 31;
+    int lanes = 1;
+    while (lanes < runs && lanes < 32) lanes <<= 1;
+    const int sub = lane & (lanes - 1);
+    const int64_t gsize = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; t0 < (int64_t)total * lanes; t0 += gsize) {
+        const int i = (int)((t0 + lane) / lanes);
+        const bool in = i < total;
+        unsigned long long key = 0; uint32_t nid = 0;
+        int rank = 0;
+        if (in) {
+            const int own = i / kRun;
+            key = rkey[i]; nid = rnid[i];
+            for (int r = sub; r < runs; r += lanes)
+                rank += r == own ? i - own * kRun
+                                 : greater_in_run(rkey + r * kRun, rnid + r * kRun, min(kRun, total - r * kRun), key, nid);
+        }
+        for (int o = lanes >> 1; o; o >>= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, o);
+        if (in && sub == 0 && rank < A.k) {
+            A.ids_out[rank] = (int32_t)~nid;
+            if (A.scores_out) A.scores_out[rank] = __longlong_as_double((long long)key);
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kTkThreads) tk_select_kernel(TkArgs A) {
     cg::grid_group grid = cg::this_grid();
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint32_t *sh_hist = (uint32_t *)smem;                      // kBins (levels)
+    __shared__ __align__(16) uint32_t sh_hist[kBins];
     __shared__ uint32_t part[32];
     __shared__ int sh_sel;
-    __shared__ int64_t sh_above;
-    int tid = threadIdx.x;
-    int64_t gtid = (int64_t)blockIdx.x * blockDim.x + tid;
-    int64_t gsize = (int64_t)gridDim.x * blockDim.x;
+    __shared__ int sh_above;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + tid;
+    const int64_t gsize = (int64_t)gridDim.x * blockDim.x;
     // every warp walks the same trip count, so warp-wide ballots see whole warps
-    int64_t wbase = gtid & ~31ll;
+    const int64_t wbase = gtid & ~31ll;
     int *ctrl = A.ctrl;
-    if (gtid == 0) {
-        ctrl[C_SURE] = 0; ctrl[C_NEXT] = 0; ctrl[C_NEXT + 1] = 0;
-    }
-    for (int64_t b = gtid; b < kBins; b += gsize) A.hist[b] = 0;
     // the state every thread derives alike: candidates m in buffer src, rank need among them
     int src = 0;
     int64_t m = A.n;
     int64_t need = A.k;
-    bool done = A.n <= sort_target(A.k);                        // everything fits the final sort
+    bool done = false;                                          // n > rank_target(k)
+    if (gtid == 0) { ctrl[C_SURE] = 0; ctrl[C_NEXT] = 0; ctrl[C_NEXT + 1] = 0; }
+    for (int64_t b = gtid; b < 2 * kBins; b += gsize) A.hist[b] = 0;
     grid.sync();
     int level = 0;
     for (; level < kLevels && !done; ++level) {
+        uint32_t *hist = A.hist + (level & 1) * kBins, *other = A.hist + ((level + 1) & 1) * kBins;
         // histogram of this level's digit (the global one was cleared before)
         for (int b = tid; b < kBins; b += blockDim.x) sh_hist[b] = 0;
         __syncthreads();
-        // lanes with the same digit add once (the top digits of real scores crowd a
-        // few bins, where per-lane shared atomics would serialise)
-        for (int64_t i0 = wbase; i0 < m; i0 += gsize) {
-            int64_t i = i0 + (tid & 31);
-            bool in = i < m;
-            uint32_t dg = kBins;                                // no bin: lanes past the end
-            if (in) {
-                unsigned long long key; uint32_t nid;
-                load_item(A, level, src, i, key, nid);
-                dg = digit_of(key, nid, level);
+        // four items per lane and trip, loaded together; lanes with the same digit add
+        // once (the top digits of real scores crowd a few bins, where per-lane shared
+        // atomics would serialise)
+        for (int64_t i0 = wbase; i0 < m; i0 += 4 * gsize) {
+            uint32_t dg[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t i = i0 + j * gsize + lane;
+                unsigned long long key = 0; uint32_t nid = 0;
+                dg[j] = kBins;                                  // no bin: lanes past the end
+                if (i < m) { load_item(A, level, src, i, key, nid); dg[j] = digit_of(key, nid, level); }
             }
-            unsigned same = __match_any_sync(0xFFFFFFFFu, dg);
-            if (in && (tid & 31) == __ffs(same) - 1) atomicAdd(&sh_hist[dg], (uint32_t)__popc(same));
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const unsigned same = __match_any_sync(0xFFFFFFFFu, dg[j]);
+                if (dg[j] < kBins && lane == __ffs(same) - 1) atomicAdd(&sh_hist[dg[j]], (uint32_t)__popc(same));
+            }
         }
         __syncthreads();
         for (int b = tid; b < kBins; b += blockDim.x)
-            if (sh_hist[b]) atomicAdd(&A.hist[b], sh_hist[b]);
+            if (sh_hist[b]) atomicAdd(&hist[b], sh_hist[b]);
         grid.sync();
-        // CTA 0: the bucket holding the need-th largest key
-        if (blockIdx.x == 0) {
+        // every CTA: the bucket holding the need-th largest key
+        {
             constexpr int per = kBins / kTkThreads;             // 4 bins per thread, from the top
-            int top = kBins - per * tid;
-            uint32_t sacc = 0;
-            for (int j = 1; j <= per; ++j) sacc += A.hist[top - j];
+            const int top = kBins - per * tid;
+            uint32_t f[per], sacc = 0;
+            for (int j = 0; j < per; ++j) { f[j] = __ldcg(&hist[top - 1 - j]); sacc += f[j]; }
             // inclusive scan over the threads: within warps by shuffles, then over the warp sums
-            const int lane = tid & 31, wid = tid >> 5;
             uint32_t incl = sacc;
             for (int o = 1; o < 32; o <<= 1) {
                 uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
@@ -177,7 +242,7 @@ __global__ void __launch_bounds__(kTkThreads) tk_select_kernel(TkArgs A) {
             if (lane == 31) part[wid] = incl;
             __syncthreads();
             if (wid == 0) {
-                uint32_t w = lane < kTkThreads / 32 ? part[lane] : 0;
+                uint32_t w = part[lane];
                 for (int o = 1; o < 32; o <<= 1) {
                     uint32_t v = __shfl_up_sync(0xFFFFFFFFu, w, o);
                     if (lane >= o) w += v;
@@ -185,73 +250,61 @@ __global__ void __launch_bounds__(kTkThreads) tk_select_kernel(TkArgs A) {
                 part[lane] = w;                                 // inclusive sums of the warp sums
             }
             __syncthreads();
-            const uint32_t mine = incl + (wid ? part[wid - 1] : 0u);
-            int64_t before = (int64_t)mine - sacc;
-            if (before < need && need <= (int64_t)mine) {
+            const int64_t mine = (int64_t)incl + (wid ? part[wid - 1] : 0u);
+            const int64_t before = mine - sacc;
+            if (before < need && need <= mine) {
                 int64_t acc = before;
-                for (int j = 1; j <= per; ++j) {
-                    int b = top - j;
-                    if (acc + A.hist[b] >= need) { sh_sel = b; sh_above = acc; break; }
-                    acc += A.hist[b];
+                for (int j = 0; j < per; ++j) {
+                    if (acc + f[j] >= need) { sh_sel = top - 1 - j; sh_above = (int)acc; break; }
+                    acc += f[j];
                 }
             }
             __syncthreads();
-            if (tid == 0) {
-                ctrl[C_SEL] = sh_sel;
-                ctrl[C_NEED] = (int)(need - sh_above);
-            }
         }
-        grid.sync();
-        // compact: higher buckets are sure, the selected bucket stays; the global
-        // histogram is cleared for the next level, and the candidate counter of
-        // the next level (last read before this level's first barrier) reset
-        const uint32_t sel = (uint32_t)ctrl[C_SEL];
-        need = ctrl[C_NEED];
+        // compact: higher buckets are sure, the selected bucket stays; the other global
+        // histogram is cleared for the next level (last read before this level's barrier),
+        // and the candidate counter of the next level reset (likewise)
+        const uint32_t sel = (uint32_t)sh_sel;
+        need -= sh_above;
         const int dst = src ^ 1;
         int *next = &ctrl[C_NEXT + (level & 1)];
-        for (int64_t b = gtid; b < kBins; b += gsize) A.hist[b] = 0;
+        for (int64_t b = gtid; b < kBins; b += gsize) other[b] = 0;
         if (gtid == 0) ctrl[C_NEXT + ((level + 1) & 1)] = 0;
-        for (int64_t i0 = wbase; i0 < m; i0 += gsize) {
-            int64_t i = i0 + (tid & 31);
-            unsigned long long key = 0; uint32_t nid = 0, dg = 0;
-            bool in = i < m;
-            if (in) {
-                load_item(A, level, src, i, key, nid);
-                dg = digit_of(key, nid, level);
+        for (int64_t i0 = wbase; i0 < m; i0 += 4 * gsize) {
+            unsigned long long key[4]; uint32_t nid[4], dg[4];
+            bool in[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t i = i0 + j * gsize + lane;
+                key[j] = 0; nid[j] = 0; dg[j] = 0;
+                in[j] = i < m;
+                if (in[j]) { load_item(A, level, src, i, key[j], nid[j]); dg[j] = digit_of(key[j], nid[j], level); }
             }
-            warp_append(in && dg > sel, key, nid, &ctrl[C_SURE], A.skey, A.snid);
-            warp_append(in && dg == sel, key, nid, next, A.key[dst], A.nid[dst]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                warp_append(in[j] && dg[j] > sel, key[j], nid[j], &ctrl[C_SURE], A.skey, A.snid);
+                warp_append(in[j] && dg[j] == sel, key[j], nid[j], next, A.key[dst], A.nid[dst]);
+            }
         }
         grid.sync();
-        m = *(volatile int *)next;
+        m = __ldcg(next);
         src = dst;
-        done = m <= need || *(volatile int *)&ctrl[C_SURE] + m <= sort_target(A.k);
+        done = m <= need || __ldcg(&ctrl[C_SURE]) + m <= rank_target(A.k);
     }
-    // CTA 0: sort the sure keys and the candidates left, write the first K
-    if (blockIdx.x != 0) return;
-    unsigned long long *key = (unsigned long long *)smem;
-    uint32_t *nid = (uint32_t *)(key + sort_target(A.k));      // the launch sized the sort for k
-    bool from_scores = level == 0;                              // nothing was compacted: n fits the sort
-    int ns = ctrl[C_SURE];
-    int nc = (int)m;
-    int total = ns + nc;
-    int P = 1;
-    while (P < total) P <<= 1;
-    for (int i = tid; i < P; i += blockDim.x) {
-        if (i < ns) { key[i] = A.skey[i]; nid[i] = A.snid[i]; }
-        else if (i < total) {
-            int64_t j = i - ns;
-            if (from_scores) { key[i] = (unsigned long long)__double_as_longlong(A.scores[j]); nid[i] = ~(uint32_t)j; }
-            else { key[i] = A.key[src][j]; nid[i] = A.nid[src][j]; }
-        } else { key[i] = 0; nid[i] = 0; }                     // padding sorts last
-    }
-    __syncthreads();
-    block_sort_desc(key, nid, P);
-    for (int i = tid; i < A.k; i += blockDim.x) {
-        A.ids_out[i] = (int32_t)~nid[i];
-        if (A.scores_out) A.scores_out[i] = __longlong_as_double((long long)key[i]);
-    }
+    // the sure keys and the candidates left
+    const int ns = __ldcg(&ctrl[C_SURE]);
+    sort_runs(A, level, src, ns, ns + (int)m, sh_hist);
+    grid.sync();
+    rank_runs(A, src, ns + (int)m);
 }
+
+// n <= rank_target(k): every score goes to the final ranking, as two plain launches (the
+// barrier between them costs less than a cooperative launch does)
+__global__ void __launch_bounds__(kTkThreads) tk_runs_kernel(TkArgs A) {
+    __shared__ __align__(16) uint32_t sh[4 * kRun];
+    sort_runs(A, 0, 0, 0, (int)A.n, sh);
+}
+__global__ void __launch_bounds__(kTkThreads) tk_rank_kernel(TkArgs A) { rank_runs(A, 0, (int)A.n); }
 
 }  // namespace
 
@@ -261,7 +314,7 @@ static int ensure_topk_workspace(rs_graph *g, int64_t n) {
     RS_CUDA_TRY(pool_free_many(old, 4));
     g->tk_hist = nullptr; g->tk_ctrl = nullptr; g->tk_keys = nullptr; g->tk_ids = nullptr;
     int64_t cap = n > 1 ? n : 1;
-    RS_CUDA_TRY(pool_malloc((void **)&g->tk_hist, kBins * sizeof(uint32_t)));
+    RS_CUDA_TRY(pool_malloc((void **)&g->tk_hist, 2 * kBins * sizeof(uint32_t)));
     RS_CUDA_TRY(pool_malloc((void **)&g->tk_ctrl, 8 * sizeof(int)));
     RS_CUDA_TRY(pool_malloc((void **)&g->tk_keys, (2 * cap + kSortMax) * sizeof(unsigned long long)));
     RS_CUDA_TRY(pool_malloc((void **)&g->tk_ids, (2 * cap + kSortMax) * sizeof(uint32_t)));
@@ -270,19 +323,18 @@ static int ensure_topk_workspace(rs_graph *g, int64_t n) {
     return 0;
 }
 
-static int tk_grid = 0;   // one CTA per SM (or what fits), found once per process
+static int tk_grid = 0;   // one CTA per SM, found once per process
 
 // workspace for n scores and the selection kernel's launch shape
 int rs::topk_prepare(rs_graph *g, int64_t n) {
     if (int rc = ensure_topk_workspace(g, n)) return rc;
     if (!tk_grid) {
-        RS_CUDA_TRY(cudaFuncSetAttribute(tk_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTkSmem));
         int dev = 0, sms = 0, per_sm = 0;
         RS_CUDA_TRY(cudaGetDevice(&dev));
         RS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        RS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tk_select_kernel, kTkThreads, kTkSmem));
+        RS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tk_select_kernel, kTkThreads, 0));
         if (per_sm < 1) return fail(RS_ECUDA, "rs_topk: selection kernel does not fit an SM");
-        tk_grid = sms * per_sm;
+        tk_grid = sms;
     }
     return 0;
 }
@@ -292,7 +344,6 @@ int rs::topk_scores(rs_graph *g, const double *scores, int64_t n, int32_t k, int
     if (k > kSortMax) return fail(RS_EINVAL, "rs_topk: k above 16384 is not supported");
     if (n > 2147483647LL) return fail(RS_EINVAL, "rs_topk: n too large");
     if (int rc = topk_prepare(g, n)) return rc;
-    const int grid = tk_grid;
     int64_t cap = g->tk_cap;
     TkArgs A;
     A.scores = scores; A.n = n; A.k = k; A.ids_out = ids; A.scores_out = out_scores;
@@ -302,11 +353,19 @@ int rs::topk_scores(rs_graph *g, const double *scores, int64_t n, int32_t k, int
     A.key[0] = kb; A.key[1] = kb + cap; A.skey = kb + 2 * cap;
     A.nid[0] = ib; A.nid[1] = ib + cap; A.snid = ib + 2 * cap;
     prof_begin(g, s);
+    if (n <= rank_target(k)) {
+        const int runs = (int)((n + kRun - 1) / kRun);
+        tk_runs_kernel<<<runs, kTkThreads, 0, s>>>(A);
+        RS_LAUNCHED(g, s, "tk_runs");
+        tk_rank_kernel<<<std::min(tk_grid, (int)((n * std::min(runs, 32) + kTkThreads - 1) / kTkThreads) + 1),
+                         kTkThreads, 0, s>>>(A);
+        RS_LAUNCHED(g, s, "tk_rank");
+        return 0;
+    }
+    // a CTA for every 2,048 scores of the levels' passes, or every run of the ranking
+    const int grid = (int)std::min<int64_t>(tk_grid, std::max<int64_t>((n + 2047) / 2048, rank_target(k) / kRun));
     void *args[] = {&A};
-    // dynamic shared memory: the level histograms, or the final sort of up to sort_target(k)
-    // keys, whichever is larger (24 KB for k <= 1024; the attribute allows kTkSmem)
-    const size_t smem = std::max((size_t)kBins * sizeof(uint32_t), (size_t)sort_target(k) * (8 + 4));
-    RS_CUDA_TRY(cudaLaunchCooperativeKernel((void *)tk_select_kernel, dim3(grid), dim3(kTkThreads), args, smem, s));
+    RS_CUDA_TRY(cudaLaunchCooperativeKernel((void *)tk_select_kernel, dim3(grid), dim3(kTkThreads), args, 0, s));
     RS_LAUNCHED(g, s, "tk_select");
     return 0;
 }

@@ -52,3 +52,19 @@ def test_topk_equals_stable_sort(rs, n, dist):
         np.testing.assert_array_equal(ids.cpu().numpy(), want)
         np.testing.assert_array_equal(vals.cpu().numpy().view(np.uint64), s[want].view(np.uint64))
     G.close()
+
+
+@pytest.mark.parametrize("n", [255, 256, 257, 8191, 8192, 8193, 16385, 40001])
+def test_topk_at_the_edges_of_the_ranking(rs, n):
+    """One run of keys more or less than full, the sizes at which the scores are ranked without a
+    radix level, and the K at which that size doubles."""
+    rng = np.random.default_rng(n)
+    G = _isolated(rs, n)
+    for s in (rng.random(n), rng.choice(np.array([0.0, 0.5, 1.0]), n)):
+        d = torch.as_tensor(s, device="cuda")
+        for K in sorted({min(n, k) for k in (1, 255, 256, 257, 4096, 4097, 8193)}):
+            ids, vals = G.topk(d, K)
+            want = oracle.topk(s, K)
+            np.testing.assert_array_equal(ids.cpu().numpy(), want)
+            np.testing.assert_array_equal(vals.cpu().numpy().view(np.uint64), s[want].view(np.uint64))
+    G.close()
