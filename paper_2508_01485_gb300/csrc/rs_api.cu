@@ -157,19 +157,22 @@ void rs::prof_mark(rs_graph *g, cudaStream_t s, const char *name, bool is_kernel
     if (g->prof_on) prof_record(g, s, name, is_kernel);
 }
 
-int rs::fork_aux(rs_graph *g, cudaStream_t s) {
+int rs::fork_aux(rs_graph *g, cudaStream_t s, unsigned used) {
+    if (!used) return 0;
     RS_CUDA_TRY(cudaEventRecord(g->ev_fork, s));
-    for (int i = 0; i < rs_graph::kAux; ++i) {
-        RS_CUDA_TRY(cudaStreamWaitEvent(g->aux[i], g->ev_fork, 0));
-        prof_begin(g, g->aux[i]);
-    }
+    for (int i = 0; i < rs_graph::kAux; ++i)
+        if (used >> i & 1) {
+            RS_CUDA_TRY(cudaStreamWaitEvent(g->aux[i], g->ev_fork, 0));
+            prof_begin(g, g->aux[i]);
+        }
     return 0;
 }
-int rs::join_aux(rs_graph *g, cudaStream_t s, int used) {
-    for (int i = 0; i < used; ++i) {
-        RS_CUDA_TRY(cudaEventRecord(g->ev_join[i], g->aux[i]));
-        RS_CUDA_TRY(cudaStreamWaitEvent(s, g->ev_join[i], 0));
-    }
+int rs::join_aux(rs_graph *g, cudaStream_t s, unsigned used) {
+    for (int i = 0; i < rs_graph::kAux; ++i)
+        if (used >> i & 1) {
+            RS_CUDA_TRY(cudaEventRecord(g->ev_join[i], g->aux[i]));
+            RS_CUDA_TRY(cudaStreamWaitEvent(s, g->ev_join[i], 0));
+        }
     prof_begin(g, s);
     return 0;
 }
@@ -745,15 +748,12 @@ static int build_tables(rs_graph *g, cudaStream_t s) {
     return 0;
 }
 
-// xR (one reverse value per G_x slot) exists while the mirror pass is selected
+// the mirror pass's tile table exists while that pass is selected
 int rs::set_mirror_buffer(rs_graph *g) {
-    if (g->tune.p3_mirror && !g->xR) {
-        RS_CUDA_TRY(dmalloc(&g->xR, std::max<int64_t>(g->nnz, 1)));
+    if (g->tune.p3_mirror && !g->xtile) {
         RS_CUDA_TRY(dmalloc(&g->xtile, g->nnz / kMirTile + 2));
-    } else if (!g->tune.p3_mirror && g->xR) {
-        RS_CUDA_TRY(pool_free(g->xR));
+    } else if (!g->tune.p3_mirror && g->xtile) {
         RS_CUDA_TRY(pool_free(g->xtile));
-        g->xR = nullptr;
         g->xtile = nullptr;
     }
     return 0;
@@ -771,7 +771,7 @@ static int alloc_workspace(rs_graph *g) {
     }
     RS_CUDA_TRY(cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming));
     RS_CUDA_TRY(dmalloc(&g->rec, n));
-    RS_CUDA_TRY(dmalloc(&g->acc, 2 * n));
+    RS_CUDA_TRY(dmalloc(&g->acc, 3 * n));
     RS_CUDA_TRY(dmalloc(&g->wmax_bits, g->n_graphs));
     RS_CUDA_TRY(dmalloc(&g->winv, g->n_graphs));
     RS_CUDA_TRY(dmalloc(&g->Lall, n));
@@ -782,6 +782,7 @@ static int alloc_workspace(rs_graph *g) {
     RS_CUDA_TRY(dmalloc(&g->xcol, nnz + 8));
     RS_CUDA_TRY(dmalloc(&g->xsk, nnz / 8 + 1));
     RS_CUDA_TRY(dmalloc(&g->xS, nnz));
+    RS_CUDA_TRY(dmalloc(&g->xnode, n));
     RS_CUDA_TRY(dmalloc(&g->xout, n));
     RS_CUDA_TRY(dmalloc(&g->xin, n));
     if (int rc = rs::set_mirror_buffer(g)) return rc;
@@ -802,8 +803,8 @@ static void free_graph(rs_graph *g) {
     if (!g) return;
     void *ptrs[] = {g->off, g->off_alt, g->col, g->col_alt, g->lab, g->removed, g->dead,
                     g->rows_small, g->rows_mid, g->rows_large, g->rows_sort, g->LG, g->RD, g->rec, g->acc, g->wmax_bits,
-                    g->Lall, g->xoff, g->xcol, g->xsk, g->xS, g->xout, g->xin, g->scan_tmp, g->tk_hist,
-                    g->tk_ctrl, g->tk_keys, g->tk_ids, g->d_flag, g->xR, g->xtile, g->rsum, g->cl_col, g->cl_lab,
+                    g->Lall, g->xoff, g->xcol, g->xsk, g->xS, g->xout, g->xin, g->xnode, g->scan_tmp, g->tk_hist,
+                    g->tk_ctrl, g->tk_keys, g->tk_ids, g->d_flag, g->xtile, g->rsum, g->cl_col, g->cl_lab,
                     g->winv, g->gid, g->gk, g->gnode, g->p2rows, g->p2cnt, g->sx, g->wq, g->perm};
     pool_free_many(ptrs, sizeof(ptrs) / sizeof(ptrs[0]));
     free_hub_tables(g);

@@ -84,16 +84,19 @@ __device__ __forceinline__ int tab_find(const Tab &t, int32_t c) {
     return -1;
 }
 
-// Type-II term sigma^2 (Q - s_u) in accumulator units (0 when rest or sigma is 0)
+// Type-II term sigma^2 (Q - s_u), 2^-64 lsb (0 when rest or sigma is 0)
 __device__ __forceinline__ u128 type2_term(df sig, u128 rest) {
     if (rest == 0 || !(sig.hi > 0.0f)) return 0;
     df t = df_mul(df_mul(sig, sig), df_from_u128(rest, -kSFrac));
-    return df_to_fixed(t, kAccFrac);
+    return df_to_fixed(t, kTermFrac);
 }
-// pushed to u (taken away, modulo 2^128, when neg)
+// pushed to u (taken away, modulo 2^192, when neg)
 __device__ __forceinline__ void push_type2(unsigned long long *acc, int32_t u, df sig, u128 rest, bool neg = false) {
-    u128 v = type2_term(sig, rest);
-    if (v) atomic_add_u128(acc + 2 * (int64_t)u, neg ? (u128)0 - v : v);
+    const u128 v = type2_term(sig, rest);
+    if (v) {
+        const u192 t = u192_from_term(v);
+        atomic_add_u192(acc + 3 * (int64_t)u, neg ? u192_neg(t) : t);
+    }
 }
 
 // The strict reading of the triad indicator (RS_TRIAD_STRICT) drops the closed
@@ -120,27 +123,22 @@ __device__ __forceinline__ u128 strict_rest(const Strict &SX, const int64_t *off
     return rest - (((u128)SX.sx[2 * pos + 1] << 64) | SX.sx[2 * pos]);
 }
 
-// the three apex terms of triangle (a, b, c) from its six directed values
-// S(x -> y) = w_x(C(y))^(1/3): at apex a the ordered pairs (w, v) = (b, c) and
-// (c, b) give S(c->a) S(b->c) S(b->a) + S(b->a) S(c->b) S(c->a)
-struct TriTerms { u128 a, b, c; };
-// the same with the pair sums Pac = S(a->c) + S(c->a) and Pab = S(a->b) + S(b->a)
-// given (df_add(Sac, Sca) and df_add(Sab, Sba)): the same operations, so the same bits
-__device__ __forceinline__ TriTerms triangle_term_values_p(df Sab, df Sba, df Sac, df Sca, df Sbc, df Scb, df Pac,
-                                                           df Pab) {
-    df ta = df_mul(df_mul(Sba, Sca), df_add(Sbc, Scb));
-    df tb = df_mul(df_mul(Sab, Scb), Pac);
-    df tc = df_mul(df_mul(Sac, Sbc), Pab);
-    return TriTerms{df_to_fixed(ta, kAccFrac), df_to_fixed(tb, kAccFrac), df_to_fixed(tc, kAccFrac)};
-}
-__device__ __forceinline__ TriTerms triangle_term_values(df Sab, df Sba, df Sac, df Sca, df Sbc, df Scb) {
-    return triangle_term_values_p(Sab, Sba, Sac, Sca, Sbc, Scb, df_add(Sac, Sca), df_add(Sab, Sba));
+// the three apex terms of triangle (a, b, c), rank a < b < c, from its six directed values
+// S(x -> y) = w_x(C(y))^(1/3): at apex a the ordered pairs (w, v) = (b, c) and (c, b) give
+// S(c->a) S(b->c) S(b->a) + S(b->a) S(c->b) S(c->a).  The grouping of the factors is part of
+// the definition (pair products are rounded down): the P3 kernels take the outer factors of
+// apexes a, b and c out of their sums over c, over c and over b.
+struct TriTerms { u192 a, b, c; };
+__device__ __forceinline__ TriTerms triangle_term_values(uint64_t Sab, uint64_t Sba, uint64_t Sac, uint64_t Sca,
+                                                         uint64_t Sbc, uint64_t Scb) {
+    return TriTerms{scale(Sba, pair_term(Sca, Sbc + Scb)), scale(Sab, pair_term(Scb, Sac + Sca)),
+                    scale(Sac, pair_term(Sbc, Sab + Sba))};
 }
 __device__ __forceinline__ void add_triangle(unsigned long long *acc, int32_t a, int32_t b, int32_t c,
                                              const TriTerms &t, bool neg = false) {
-    atomic_add_u128(acc + 2 * (int64_t)a, neg ? (u128)0 - t.a : t.a);
-    atomic_add_u128(acc + 2 * (int64_t)b, neg ? (u128)0 - t.b : t.b);
-    atomic_add_u128(acc + 2 * (int64_t)c, neg ? (u128)0 - t.c : t.c);
+    atomic_add_u192(acc + 3 * (int64_t)a, neg ? u192_neg(t.a) : t.a);
+    atomic_add_u192(acc + 3 * (int64_t)b, neg ? u192_neg(t.b) : t.b);
+    atomic_add_u192(acc + 3 * (int64_t)c, neg ? u192_neg(t.c) : t.c);
 }
 
 // finishing a row in P1: the row's largest weight, s_v and the node record;

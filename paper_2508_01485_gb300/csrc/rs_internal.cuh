@@ -35,6 +35,19 @@ struct __align__(16) NodeRec {
     int32_t dx;       // cross-community degree (neighbours with another label)
 };
 
+// a G_x slot's values, 2^-48 fixed point: f = S(row -> neighbour), written by P2; at out-slots
+// r = S(neighbour -> row), written by the mirror pass.  One 16-byte load brings both
+struct __align__(16) SigPair {
+    uint64_t f, r;
+};
+
+// what P3 gathers of a G_x node: the start of its slots, its out-neighbours and its cross
+// degree (rank); written by P2 for every row with cross neighbours
+struct __align__(16) GxNode {
+    int64_t off;
+    int32_t out, dx;
+};
+
 // per-hub state (global hash table and row aggregates)
 // the per-slot passes over the hubs' tables (their sums, column maxima and sigma) take a
 // hub's table in ranges of this many slots, so that a large hub's table is spread over
@@ -147,7 +160,7 @@ struct rs_graph {
     double *RD = nullptr;             // 1 / (d (d - 1))
     // scoring workspace
     rs::NodeRec *rec = nullptr;
-    unsigned long long *acc = nullptr;        // 2 words per node
+    unsigned long long *acc = nullptr;        // 3 words per node
     unsigned long long *wmax_bits = nullptr;  // double bits of w_max, one per graph
     int32_t *Lall = nullptr;                  // distinct neighbour communities per node
     rs::RowSum *rsum = nullptr;               // per-node aggregates from P1
@@ -156,8 +169,9 @@ struct rs_graph {
     int64_t *xoff = nullptr;                  // G_x row offsets (n + 1)
     int32_t *xcol = nullptr;                  // G_x neighbours (capacity nnz + 8: whole 8-slot sectors)
     int32_t *xsk = nullptr;                   // first id of every 8-slot sector of xcol (nnz / 8 + 1)
-    rs::df *xS = nullptr;                     // S(w -> u) = w_w(C(u))^(1/3)
+    rs::SigPair *xS = nullptr;                // S(w -> u) = w_w(C(u))^(1/3) and, at out-slots, S(u -> w)
     int32_t *xout = nullptr, *xin = nullptr;  // out / in counts per node
+    rs::GxNode *xnode = nullptr;
     int32_t *p2rows = nullptr;                // P2 row lists by cross degree (4 n), counted in p2cnt
     int32_t *p2cnt = nullptr;
     unsigned long long *wq = nullptr;         // per-pass row counters of the dynamically scheduled kernels
@@ -185,7 +199,6 @@ struct rs_graph {
     cudaEvent_t ev_fork = nullptr;
     cudaEvent_t ev_join[kAux] = {};
     // launch parameters and a counter bumped whenever buffers or row classes change
-    rs::df *xR = nullptr;                     // p3_mirror: at out-slot (w -> u) the reverse value S(u -> w)
     int32_t *xtile = nullptr;                 // p3_mirror: node holding the first slot of each mirror tile
     int32_t *perm = nullptr;                  // RS_REORDER: internal id -> the caller's id (device)
     std::vector<int32_t> iperm;               // RS_REORDER: the caller's id -> internal id (host)
@@ -249,9 +262,9 @@ cudaError_t pool_free(void *p);
 cudaError_t pool_free_many(void *const *p, size_t n);   // one device synchronisation for all
 void prof_begin(rs_graph *g, cudaStream_t s);
 void prof_mark(rs_graph *g, cudaStream_t s, const char *name, bool is_kernel);
-// make the auxiliary streams wait for s / make s wait for the first `used` auxiliary streams
-int fork_aux(rs_graph *g, cudaStream_t s);
-int join_aux(rs_graph *g, cudaStream_t s, int used);
+// make the auxiliary streams of the set `used` wait for s / make s wait for them
+int fork_aux(rs_graph *g, cudaStream_t s, unsigned used);
+int join_aux(rs_graph *g, cudaStream_t s, unsigned used);
 #define RS_LAUNCHED(g, s, name)                        \
     do {                                               \
         RS_CUDA_TRY(cudaGetLastError());               \

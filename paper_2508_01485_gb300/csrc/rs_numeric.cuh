@@ -11,7 +11,9 @@
 //  * quotients, cube roots and products use double-float numbers (an
 //    unevaluated sum hi + lo of two floats, ~2^-48 relative; Dekker 1971,
 //    "A floating-point technique for extending the available precision");
-//  * every sum of terms is accumulated in 128-bit fixed point (2^-64 lsb), so
+//  * Type-I terms are exact products of fixed-point values (see the pair products
+//    below), so that sums of them may be taken in any grouping;
+//  * every sum of terms is accumulated in 192-bit fixed point (2^-112 lsb), so
 //    atomics commute and results are bit-identical whatever the schedule.
 #pragma once
 #include <stdint.h>
@@ -22,7 +24,9 @@ typedef unsigned __int128 u128;
 
 constexpr int kLogFrac = 58;      // LG[f] = round(log2(f) * 2^58)
 constexpr int kSFrac = 52;        // node scalar s_v stored as round(s_v * 2^52)
-constexpr int kAccFrac = 64;      // accumulators: 2^-64 lsb
+constexpr int kTermFrac = 64;     // Type-II terms and pair products: 2^-64 lsb
+constexpr int kSigFrac = 48;      // G_x values S(x->y) stored as round(S 2^48)
+constexpr int kAccFrac = kSigFrac + kTermFrac;   // accumulators (three words): 2^-112 lsb
 
 // ---- double-float ----------------------------------------------------------
 
@@ -203,7 +207,7 @@ __device__ __forceinline__ double u128_to_double(u128 x, int e) {
 
 __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
 
-// ---- 128-bit accumulators -------------------------------------------------------
+// ---- 128-bit sums ---------------------------------------------------------------
 
 // acc[0] holds the low 64 bits, acc[1] the high 64 bits; concurrent adds commute
 __device__ __forceinline__ void atomic_add_u128(unsigned long long *acc, u128 v) {
@@ -214,6 +218,91 @@ __device__ __forceinline__ void atomic_add_u128(unsigned long long *acc, u128 v)
         if (old + lo < old) hi += 1ull;
     }
     if (hi) atomicAdd(acc + 1, hi);
+}
+
+// ---- accumulators: three 64-bit words, 2^-112 lsb, modulo 2^192 ---------------------
+
+struct u192 { uint64_t w0, w1, w2; };
+
+__device__ __forceinline__ u192 u192_add(u192 a, u192 b) {
+    const u128 lo = (u128)a.w0 + b.w0;
+    const u128 mid = (u128)a.w1 + b.w1 + (uint64_t)(lo >> 64);
+    return u192{(uint64_t)lo, (uint64_t)mid, a.w2 + b.w2 + (uint64_t)(mid >> 64)};
+}
+__device__ __forceinline__ u192 u192_neg(u192 a) {
+    return u192_add(u192{~a.w0, ~a.w1, ~a.w2}, u192{1, 0, 0});
+}
+// a Type-II term (2^-64 lsb) in accumulator units
+__device__ __forceinline__ u192 u192_from_term(u128 v) {
+    constexpr int sh = kAccFrac - kTermFrac;
+    return u192{(uint64_t)v << sh, (uint64_t)(v >> (64 - sh)), (uint64_t)(v >> (128 - sh))};
+}
+// concurrent adds commute; a word is touched only where it changes
+__device__ __forceinline__ void atomic_add_u192(unsigned long long *acc, u192 v) {
+    uint64_t c = 0;
+    if (v.w0) {
+        const unsigned long long old = atomicAdd(acc, (unsigned long long)v.w0);
+        c = old + v.w0 < old ? 1 : 0;
+    }
+    const uint64_t a1 = v.w1 + c;
+    uint64_t a2 = v.w2 + (a1 < c ? 1 : 0);
+    if (a1) {
+        const unsigned long long old = atomicAdd(acc + 1, (unsigned long long)a1);
+        a2 += old + a1 < old ? 1 : 0;
+    }
+    if (a2) atomicAdd(acc + 2, (unsigned long long)a2);
+}
+// the double nearest to v 2^-112 (v below 2^176)
+__device__ __forceinline__ double u192_to_double(u192 v) {
+    if (v.w2) return u128_to_double(((u128)v.w2 << 64) | v.w1 | (v.w0 ? 1 : 0), 64 - kAccFrac);
+    return u128_to_double(((u128)v.w1 << 64) | v.w0, -kAccFrac);
+}
+
+// ---- exact Type-I terms -------------------------------------------------------------
+//
+// The term of apex x of a triangle is S S (S + S).  The values S(x->y) are 2^-48 fixed
+// point (S < 2^9.6: a weight is at most L log2 L, and L <= d < 2^24), so they and the pair
+// sums P = S + S fit 64 bits, and a term is formed as
+//     scale(S, pair(S', P)),   pair(x, y) = floor(x y 2^-32)  (2^-64 lsb, below 2^85),
+// the product of S and the pair exactly, in accumulator units.  As scale is linear, the
+// terms that share an outer S may be summed as pairs first and scaled once, and the sum
+// of any grouping has the same bits.  The floor drops less than 2^-64 of a value that is
+// at least 2^-12 when it is not 0 (S >= 0.014).
+
+// S(x->y) from its double-float value
+__device__ __forceinline__ uint64_t sig_fixed(df s) {
+    return (uint64_t)((df_to_fixed(s, kSigFrac + 1) + 1) >> 1);
+}
+
+// sums of pairs: at most 2^11 of them stay below 2^96
+struct u96 { uint64_t lo; uint32_t hi; };
+
+__device__ __forceinline__ u96 pair_term(uint64_t x, uint64_t y) {
+    const uint32_t x0 = (uint32_t)x, x1 = (uint32_t)(x >> 32), y0 = (uint32_t)y, y1 = (uint32_t)(y >> 32);
+    const uint64_t m1 = (uint64_t)x0 * y1 + (((uint64_t)x0 * y0) >> 32);
+    const uint64_t m2 = (uint64_t)x1 * y0 + (uint32_t)m1;
+    const uint64_t top = (uint64_t)x1 * y1 + (m1 >> 32) + (m2 >> 32);
+    return u96{(top << 32) | (uint32_t)m2, (uint32_t)(top >> 32)};
+}
+__device__ __forceinline__ void u96_add(u96 &a, u96 b) {
+    const u128 s = (((u128)a.hi << 64) | a.lo) + (((u128)b.hi << 64) | b.lo);
+    a = u96{(uint64_t)s, (uint32_t)(s >> 64)};
+}
+__device__ __forceinline__ u192 scale(uint64_t s, u96 p) {
+    const u128 lo = (u128)s * p.lo, hi = (u128)s * p.hi + (uint64_t)(lo >> 64);
+    return u192{(uint64_t)lo, (uint64_t)hi, (uint64_t)(hi >> 64)};
+}
+
+// sums of pairs as carry-free 32-bit words: word j takes bits [25 j, 25 j + 25) of a pair,
+// so up to 128 pairs may be added to the words, each by an add whose old value is not needed
+constexpr int kLimbs = 4, kLimbBits = 25;
+__device__ __forceinline__ uint32_t pair_limb(u96 p, int j) {
+    const u128 v = ((u128)p.hi << 64) | p.lo;
+    return (uint32_t)(v >> (kLimbBits * j)) & ((1u << kLimbBits) - 1);
+}
+__device__ __forceinline__ u96 from_limbs(uint32_t l0, uint32_t l1, uint32_t l2, uint32_t l3) {
+    const u128 v = (u128)l0 + ((u128)l1 << kLimbBits) + ((u128)l2 << (2 * kLimbBits)) + ((u128)l3 << (3 * kLimbBits));
+    return u96{(uint64_t)v, (uint32_t)(v >> 64)};
 }
 
 // ---- warp reductions ---------------------------------------------------------------

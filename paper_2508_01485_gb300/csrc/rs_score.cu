@@ -29,8 +29,12 @@
 //   P3  per node a: oriented triangle listing on G_x (pairs of out-neighbours,
 //       closing edge by binary search), the Type-I terms of the three apexes;
 //   FIN R(u) = acc(u) / (w_max d(u)(d(u)-1)), 0 when d(u) < 2 or w_max = 0.
-// All terms are added into 128-bit fixed-point accumulators, so the scores do
-// not depend on the order in which threads run.
+// All terms are added into 192-bit fixed-point accumulators, and Type-I terms are
+// exact products, so the scores depend neither on the order in which threads run
+// nor on how terms are grouped before they are added.
+#include <initializer_list>
+#include <utility>
+
 #include "rs.h"
 #include "rs_internal.cuh"
 #include "rs_device.cuh"
@@ -676,6 +680,49 @@ __global__ void __launch_bounds__(NT) hub_p1_colmax_kernel(
 }
 
 // ======================================================================================
+// P2 row lists by cross degree (known after P1): each P2 kernel then walks only its rows
+//   0 mid and large rows, dx <= 32 (tiles)
+//   1 mid rows, and large rows with dx <= dx_cta, 32 < dx <= 128 (p2_mid: a warp per row)
+//   2 the same with dx > 128 (p2_large of kP2SmallCta threads)
+//   3 large rows, dx > dx_cta (p2_large)
+// ======================================================================================
+constexpr int kP2Lists = 4;
+constexpr int32_t kP2WarpDx = 128;            // a warp keeps a row of this cross degree in registers
+constexpr int kP2SmallCta = 256;
+
+__device__ __forceinline__ void append_row(int32_t *list, int32_t *cnt, bool take, int32_t v) {
+    unsigned m = __ballot_sync(FULL, take);
+    int lane = threadIdx.x & 31;
+    int32_t base = 0;
+    if (m && lane == __ffs(m) - 1) base = atomicAdd(cnt, __popc(m));
+    base = __shfl_sync(FULL, base, __ffs(m ? m : 1u) - 1);
+    if (take) list[base + __popc(m & lanemask_lt())] = v;
+}
+
+// every list has room for all mid and large rows
+struct P2Split {
+    const int32_t *rows_mid, *rows_large;
+    int64_t n_mid, n_large;
+    int32_t dx_cta;
+    int32_t *lists, *cnt;
+};
+__host__ __device__ __forceinline__ int64_t p2_list_start(int c, int64_t n_mid, int64_t n_large) {
+    return c * (n_mid + n_large);
+}
+__device__ __forceinline__ void p2_split(const P2Split &A, const NodeRec *rec, int block, int blocks) {
+    const int64_t total = A.n_mid + A.n_large;
+    for (int64_t i0 = (int64_t)block * blockDim.x; i0 < total; i0 += (int64_t)blocks * blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        const bool act = i < total, mid = i < A.n_mid;
+        const int32_t v = act ? (mid ? A.rows_mid[i] : A.rows_large[i - A.n_mid]) : 0;
+        const int32_t dx = act ? rec[v].dx : 0;
+        const int cls = !act ? -1 : dx <= 32 ? 0 : !mid && dx > A.dx_cta ? 3 : dx <= kP2WarpDx ? 1 : 2;
+        for (int c = 0; c < kP2Lists; ++c)
+            append_row(A.lists + p2_list_start(c, A.n_mid, A.n_large), A.cnt + c, cls == c, v);
+    }
+}
+
+// ======================================================================================
 // G_x row offsets: nodes with dx >= 2 keep dx slots; xoff is the exclusive scan of
 // those capacities, in one pass (decoupled look-back).  Tiles of kGxTile nodes are
 // taken in ticket order; a tile publishes its own total at once and its inclusive
@@ -697,7 +744,12 @@ constexpr unsigned long long kGxAgg = 1ull << 62, kGxIncl = 2ull << 62, kGxMask 
 // consecutive nodes (coalesced loads and stores), carrying its running total.
 __global__ void __launch_bounds__(kGxThreads) gx_offsets_kernel(
     const NodeRec *__restrict__ rec, int64_t n, int64_t *__restrict__ xoff, unsigned long long *status,
-    unsigned long long *ticket, int *err, long spin_limit, int64_t withhold_tile) {
+    unsigned long long *ticket, int *err, long spin_limit, int64_t withhold_tile, int32_t *__restrict__ cover,
+    int32_t *last, P2Split split, int split_blocks) {
+    if ((int)blockIdx.x < split_blocks) {              // the P2 row lists, by blocks of their own
+        p2_split(split, rec, blockIdx.x, split_blocks);
+        return;
+    }
     __shared__ int64_t warp_tot[kGxThreads / 32];
     __shared__ unsigned long long sh_tile;
     __shared__ int64_t sh_prefix;
@@ -783,12 +835,20 @@ __global__ void __launch_bounds__(kGxThreads) gx_offsets_kernel(
     }
     __syncthreads();
     const int64_t before = sh_prefix + warp_tot[wid];
+    int32_t own_last = -1;                            // the warp's last node with slots
     if (t == 0 && threadIdx.x == 0) xoff[0] = 0;
 #pragma unroll
     for (int k = 0; k < kGxPer; ++k) {
         int64_t v = base + k * 32 + lane;
-        if (v < n) xoff[v + 1] = before + val[k];
+        const int64_t hi = before + val[k], lo = hi - cap[k];
+        if (v < n) xoff[v + 1] = hi;
+        // the mirror's tiles that start in v's slots (every slot lies in exactly one row)
+        if (cover && cap[k] > 0)
+            for (int64_t m = (lo + kMirTile - 1) / kMirTile; m * kMirTile < hi; ++m) cover[m] = (int32_t)v;
+        const unsigned some = __ballot_sync(FULL, cap[k] > 0);
+        if (some) own_last = (int32_t)(base + k * 32 + 31 - __clz(some));
     }
+    if (cover && lane == 0 && own_last >= 0) atomicMax(last, own_last);
 }
 
 // ======================================================================================
@@ -812,10 +872,16 @@ constexpr int kNarrowRows = 8;                 // rows per tile of the narrow mi
 // the slot space also the packed index entry xsk[p / 8] (searches of long out-lists read it;
 // every slot inside a row is written once here, so the entries of sectors starting inside
 // rows are complete when P2 ends)
-__device__ __forceinline__ void gx_put(int32_t *xcol, df *xS, int32_t *xsk, int64_t p, int32_t u, df sig) {
+__device__ __forceinline__ void gx_put(int32_t *xcol, SigPair *xS, int32_t *xsk, int64_t p, int32_t u, uint64_t sig) {
     xcol[p] = u;
-    xS[p] = sig;
+    xS[p].f = sig;
     if ((p & 7) == 0) xsk[p >> 3] = u;
+}
+
+// what P3 needs of a G_x node at once: one 16-byte load instead of three random ones
+__device__ __forceinline__ GxNode load_node(const GxNode *xnode, int32_t v) {
+    const longlong2 x = __ldg(reinterpret_cast<const longlong2 *>(xnode + v));
+    return GxNode{x.x, (int32_t)(uint32_t)(unsigned long long)x.y, (int32_t)(uint32_t)((unsigned long long)x.y >> 32)};
 }
 
 struct P2Tile {
@@ -824,7 +890,7 @@ struct P2Tile {
     int32_t dx[32], w[32];
     uint32_t d[32], L[32];
     uint64_t xlo[32], xhi[32];
-    df sig1[32];
+    uint64_t sig1[32];          // sigma of a column with one member, fixed point
     int32_t no[32], ni[32];
     uint64_t st[32];
 };
@@ -834,8 +900,8 @@ __global__ void __launch_bounds__(kThreads) p2_small_kernel(
     const int64_t *__restrict__ off, const int32_t *__restrict__ rows, int64_t nrows_host,
     const int32_t *__restrict__ nrows_dev, const uint64_t *__restrict__ LG, const NodeRec *__restrict__ rec, const RowSum *__restrict__ rsum,
     const int32_t *__restrict__ cl_col, const int32_t *__restrict__ cl_lab, unsigned long long *acc,
-    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, df *__restrict__ xS, int32_t *__restrict__ xsk,
-    int32_t *__restrict__ xout, int32_t *__restrict__ xin, Strict SX) {
+    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, SigPair *__restrict__ xS, int32_t *__restrict__ xsk,
+    int32_t *__restrict__ xout, int32_t *__restrict__ xin, GxNode *__restrict__ xnode, Strict SX) {
     __shared__ P2Tile tiles[kThreads / 32];
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     P2Tile &T = tiles[wid];
@@ -858,7 +924,7 @@ __global__ void __launch_bounds__(kThreads) p2_small_kernel(
                 RowSum rs = rsum[w];
                 T.xlo[lane] = rs.xlo; T.xhi[lane] = rs.xhi; T.L[lane] = rs.L;
                 RowAgg a{T.d[lane], rs.L, ((u128)rs.xhi << 64) | rs.xlo};
-                T.sig1[lane] = df_cbrt(column_weight(a, 1, LG));
+                T.sig1[lane] = sig_fixed(df_cbrt(column_weight(a, 1, LG)));
                 T.xb[lane] = xoff[w];
             }
         }
@@ -901,7 +967,7 @@ __global__ void __launch_bounds__(kThreads) p2_small_kernel(
             unsigned long long key = ((unsigned long long)(uint32_t)r << 32) | (uint32_t)c;
             unsigned gc = 0;
             if (act) gc = __match_any_sync(am, key);
-            df sig{0.0f, 0.0f};
+            uint64_t sf = 0;
             if (act) {
                 uint32_t f = __popc(gc);
                 u128 rest = 0;
@@ -909,10 +975,11 @@ __global__ void __launch_bounds__(kThreads) p2_small_kernel(
                     unsigned m = gc & ~(1u << lane);
                     while (m) { rest += T.st[__ffs(m) - 1]; m &= m - 1; }
                 }
-                if (f == 1) sig = T.sig1[r];
+                if (f == 1) sf = T.sig1[r];
                 else {
                     RowAgg a{T.d[r], T.L[r], ((u128)T.xhi[r] << 64) | T.xlo[r]};
-                    sig = df_cbrt(column_weight(a, f, LG));
+                    const df sig = df_cbrt(column_weight(a, f, LG));
+                    sf = sig_fixed(sig);
                     push_type2(acc, u, sig, strict_rest(SX, off, T.w[r], u, rest));
                 }
             }
@@ -928,109 +995,125 @@ __global__ void __launch_bounds__(kThreads) p2_small_kernel(
             __syncwarp();
             if (o) {
                 int64_t p = T.xb[r] + bo + __popc(go & lanemask_lt());
-                gx_put(xcol, xS, xsk, p, u, sig);
+                gx_put(xcol, xS, xsk, p, u, sf);
                 if (lane == __ffs(go) - 1) T.no[r] = bo + __popc(go);
             }
             if (in) {
                 int64_t p = T.xb[r] + T.dx[r] - 1 - (bi + __popc(gi & lanemask_lt()));
-                gx_put(xcol, xS, xsk, p, u, sig);
+                gx_put(xcol, xS, xsk, p, u, sf);
                 if (lane == __ffs(gi) - 1) T.ni[r] = bi + __popc(gi);
             }
             __syncwarp();
             e0 = E;
         }
-        if (have) { xout[w] = T.no[lane]; xin[w] = T.ni[lane]; }
+        if (have) { xout[w] = T.no[lane]; xin[w] = T.ni[lane]; xnode[w] = GxNode{T.xb[lane], T.no[lane], dx}; }
         __syncwarp();
     }
 }
 
 // Mid rows, one warp per row: a per-warp table (community -> count, Type-II
 // sum) over the cross list, then the terms and the G_x entries in id order.
-constexpr int kMidSlotBytes = 4 + 4 + 16;   // key, count, 2-word sum
+//
+// A row has at most kP2WarpDx cross neighbours, so its list and their records are loaded at
+// once into registers (kP2Per entries per lane), and an entry's table slot is kept from the
+// insertion for the terms: the loads of a row are two dependent steps.  With the list read
+// chunk by chunk, twice, and the table searched again, a row of 129-256 neighbours took up to
+// 50 us of one warp, the end of the whole phase on small graphs; those rows now take a CTA.
+constexpr int kP2Per = kP2WarpDx / 32;
+constexpr int kP2MidSlots = 2 * kP2WarpDx, kMidSlotBytes = 4 + 4 + 16;   // key, count, 2-word sum
+constexpr size_t kP2MidSmem = (size_t)kMidWarps * kP2MidSlots * kMidSlotBytes;
 
 __global__ void __launch_bounds__(kThreads) p2_mid_kernel(
-    const int64_t *__restrict__ off, const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, Batch B, int32_t dx_max, int32_t wslots,
+    const int64_t *__restrict__ off, const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, Batch B,
     const uint64_t *__restrict__ LG, const NodeRec *__restrict__ rec, const RowSum *__restrict__ rsum,
     const int32_t *__restrict__ cl_col, const int32_t *__restrict__ cl_lab, unsigned long long *acc,
-    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, df *__restrict__ xS, int32_t *__restrict__ xsk,
-    int32_t *__restrict__ xout, int32_t *__restrict__ xin, int *err, Strict SX, unsigned long long *wq) {
+    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, SigPair *__restrict__ xS, int32_t *__restrict__ xsk,
+    int32_t *__restrict__ xout, int32_t *__restrict__ xin, GxNode *__restrict__ xnode, int *err, Strict SX, unsigned long long *wq) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t stage[kThreads];
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint64_t *st = stage + (threadIdx.x & ~31);
-    unsigned char *base_w = smem + (size_t)wid * wslots * kMidSlotBytes;   // wslots >= every row's table
+    unsigned char *base_w = smem + (size_t)wid * kP2MidSlots * kMidSlotBytes;
     const int64_t nrows = *nrows_dev;               // rows of this kernel, counted by p2_split
     for (int64_t i = warp_next(wq); i < nrows; i = warp_next(wq)) {
-        int32_t w = rows[i];
-        int64_t b = off[w];
-        int d = (int)(off[w + 1] - b);
-        NodeRec rw = rec[w];
-        int dx = rw.dx;
-        if (dx > dx_max || dx <= 32) continue;     // the CTA-per-row kernel / the tile kernel
-        int32_t bo = 0, bi = 0;
-        {
-            uint32_t cap = dev_pow2_at_least(2u * (uint32_t)min(dx, k_of(B, graph_of(B, w))));
-            Tab t;
-            t.q = (unsigned long long *)base_w;
-            t.key = (int32_t *)(base_w + 16 * wslots);
-            t.cnt = (uint32_t *)(base_w + 20 * wslots);
-            t.sig = nullptr;
-            t.mask = cap - 1;
-            for (uint32_t j = lane; j < cap; j += 32) { t.key[j] = kEmpty; t.cnt[j] = 0; t.q[2 * j] = 0; t.q[2 * j + 1] = 0; }
-            __syncwarp();
-            for (int base = 0; base < dx; base += 32) {
-                int e = base + lane;
-                bool act = e < dx;
-                int32_t c = act ? cl_lab[b + e] : -1;
-                st[lane] = act ? rec[cl_col[b + e]].s_fix : 0;
+        const int32_t w = rows[i];
+        const int64_t b = off[w];
+        const int d = (int)(off[w + 1] - b);
+        const int dx = rec[w].dx;
+        const int64_t xb = xoff[w];
+        const RowSum rs = rsum[w];
+        int32_t u[kP2Per], c[kP2Per], sl[kP2Per], udx[kP2Per];
+        uint64_t s[kP2Per];
+#pragma unroll
+        for (int j = 0; j < kP2Per; ++j) {
+            const int e = 32 * j + lane;
+            u[j] = e < dx ? cl_col[b + e] : -1;
+            c[j] = e < dx ? cl_lab[b + e] : -1;
+        }
+        const uint32_t cap = dev_pow2_at_least(2u * (uint32_t)min(dx, k_of(B, graph_of(B, w))));
+        Tab t;
+        t.q = (unsigned long long *)base_w;
+        t.key = (int32_t *)(base_w + 16 * kP2MidSlots);
+        t.cnt = (uint32_t *)(base_w + 20 * kP2MidSlots);
+        t.sig = nullptr;
+        t.mask = cap - 1;
+        for (uint32_t j = lane; j < cap; j += 32) { t.key[j] = kEmpty; t.cnt[j] = 0; t.q[2 * j] = 0; t.q[2 * j + 1] = 0; }
+#pragma unroll
+        for (int j = 0; j < kP2Per; ++j) {
+            NodeRec r{0, -1, 0};
+            if (u[j] >= 0) r = rec[u[j]];
+            s[j] = r.s_fix;
+            udx[j] = r.dx;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < kP2Per; ++j) {
+            sl[j] = -1;
+            if (32 * j < dx) {
+                const bool act = u[j] >= 0;
+                st[lane] = s[j];
                 __syncwarp();
-                unsigned am = __ballot_sync(FULL, act);
+                const unsigned am = __ballot_sync(FULL, act);
                 if (act) {
-                    unsigned grp = __match_any_sync(am, c);
-                    if (lane == __ffs(grp) - 1) {
-                        int sl = tab_insert(t, c, __popc(grp), err);
-                        if (sl >= 0) atomic_add_u128(t.q + 2 * sl, group_sum_all(st, grp));
+                    const unsigned grp = __match_any_sync(am, c[j]);
+                    const int leader = __ffs(grp) - 1;
+                    int q = -1;
+                    if (lane == leader) {
+                        q = tab_insert(t, c[j], __popc(grp), err);
+                        if (q >= 0) atomic_add_u128(t.q + 2 * q, group_sum_all(st, grp));
                     }
+                    sl[j] = __shfl_sync(grp, q, leader);
                 }
                 __syncwarp();
-            }
-            RowSum rs = rsum[w];
-            RowAgg a{(uint32_t)d, rs.L, ((u128)rs.xhi << 64) | rs.xlo};
-            df sig1 = df_cbrt(column_weight(a, 1, LG));   // the usual count of a foreign community
-            int64_t xb = xoff[w];
-            for (int base = 0; base < dx; base += 32) {
-                int e = base + lane;
-                bool act = e < dx;
-                int32_t u = act ? cl_col[b + e] : -1;
-                int32_t c = act ? cl_lab[b + e] : -1;
-                NodeRec ru{0, -1, 0};
-                if (act) ru = rec[u];
-                df sig{0.0f, 0.0f};
-                bool ok = act;
-                if (act) {
-                    int sl = tab_find(t, c);
-                    if (sl < 0) { atomicOr(err, 2); ok = false; }
-                    else {
-                        uint32_t f = t.cnt[sl];
-                        sig = f == 1 ? sig1 : df_cbrt(column_weight(a, f, LG));
-                        if (f > 1) {
-                            u128 q = ((u128)t.q[2 * sl + 1] << 64) | t.q[2 * sl];
-                            push_type2(acc, u, sig, strict_rest(SX, off, w, u, q - ru.s_fix));
-                        }
-                    }
-                }
-                if (dx >= 2) {
-                    bool inx = ok && ru.dx >= 2;
-                    bool o = inx && rank_after(ru.dx, u, dx, w);
-                    bool in = inx && !o;
-                    unsigned mo = __ballot_sync(FULL, o), mi = __ballot_sync(FULL, in);
-                    if (o) gx_put(xcol, xS, xsk, xb + bo + __popc(mo & lanemask_lt()), u, sig);
-                    if (in) gx_put(xcol, xS, xsk, xb + dx - 1 - (bi + __popc(mi & lanemask_lt())), u, sig);
-                    bo += __popc(mo); bi += __popc(mi);
-                }
             }
         }
-        if (lane == 0) { xout[w] = bo; xin[w] = bi; }
+        const RowAgg a{(uint32_t)d, rs.L, ((u128)rs.xhi << 64) | rs.xlo};
+        const uint64_t sig1 = sig_fixed(df_cbrt(column_weight(a, 1, LG)));   // the usual count of a foreign community
+        int32_t bo = 0, bi = 0;
+#pragma unroll
+        for (int j = 0; j < kP2Per; ++j) {
+            if (32 * j < dx) {
+                uint64_t sf = sig1;
+                const bool ok = sl[j] >= 0;
+                if (ok) {
+                    const uint32_t f = t.cnt[sl[j]];
+                    if (f > 1) {
+                        const df sig = df_cbrt(column_weight(a, f, LG));
+                        sf = sig_fixed(sig);
+                        const u128 q = ((u128)t.q[2 * sl[j] + 1] << 64) | t.q[2 * sl[j]];
+                        push_type2(acc, u[j], sig, strict_rest(SX, off, w, u[j], q - s[j]));
+                    }
+                }
+                const bool inx = ok && udx[j] >= 2;
+                const bool o = inx && rank_after(udx[j], u[j], dx, w);
+                const bool in = inx && !o;
+                const unsigned mo = __ballot_sync(FULL, o), mi = __ballot_sync(FULL, in);
+                if (o) gx_put(xcol, xS, xsk, xb + bo + __popc(mo & lanemask_lt()), u[j], sf);
+                if (in) gx_put(xcol, xS, xsk, xb + dx - 1 - (bi + __popc(mi & lanemask_lt())), u[j], sf);
+                bo += __popc(mo); bi += __popc(mi);
+            }
+        }
+        if (lane == 0) { xout[w] = bo; xin[w] = bi; xnode[w] = GxNode{xb, bo, dx}; }
         __syncwarp();
     }
 }
@@ -1048,8 +1131,8 @@ __device__ __forceinline__ Tab p2_table(unsigned char *base, uint32_t cap) {
 
 // CTA-ordered compaction of the G_x entries of one round; returns this thread's position
 template <int NT>
-__device__ __forceinline__ void gx_round(bool out, bool in, int64_t xb, int32_t dxw, int32_t u, df sig,
-                                         int32_t &base_out, int32_t &base_in, int32_t *xcol, df *xS,
+__device__ __forceinline__ void gx_round(bool out, bool in, int64_t xb, int32_t dxw, int32_t u, uint64_t sig,
+                                         int32_t &base_out, int32_t &base_in, int32_t *xcol, SigPair *xS,
                                          int32_t *xsk, int32_t *sh_cnt /* 2 * NT/32 */) {
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned mo = __ballot_sync(FULL, out), mi = __ballot_sync(FULL, in);
@@ -1068,11 +1151,11 @@ __device__ __forceinline__ void gx_round(bool out, bool in, int64_t xb, int32_t 
 
 template <int NT>
 __global__ void __launch_bounds__(NT) p2_large_kernel(
-    const int64_t *__restrict__ off, const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, Batch B, int32_t dx_min,
+    const int64_t *__restrict__ off, const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, Batch B,
     const uint64_t *__restrict__ LG, const NodeRec *__restrict__ rec, const RowSum *__restrict__ rsum,
     const int32_t *__restrict__ cl_col, const int32_t *__restrict__ cl_lab, unsigned long long *acc,
-    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, df *__restrict__ xS, int32_t *__restrict__ xsk,
-    int32_t *__restrict__ xout, int32_t *__restrict__ xin, int *err, Strict SX, unsigned long long *wq) {
+    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, SigPair *__restrict__ xS, int32_t *__restrict__ xsk,
+    int32_t *__restrict__ xout, int32_t *__restrict__ xin, GxNode *__restrict__ xnode, int *err, Strict SX, unsigned long long *wq) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int32_t sh_cnt[2 * NT / 32];
     __shared__ uint64_t stage[NT];
@@ -1086,11 +1169,6 @@ __global__ void __launch_bounds__(NT) p2_large_kernel(
         int d = (int)(off[w + 1] - b);
         NodeRec rw = rec[w];
         int dx = rw.dx;
-        if (dx < dx_min) continue;                  // done by the warp-per-row kernel
-        if (dx == 0) {
-            if (tid == 0) { xout[w] = 0; xin[w] = 0; }
-            continue;
-        }
         uint32_t cap = dev_pow2_at_least(2u * (uint32_t)min(dx, k_of(B, graph_of(B, w))));
         Tab t = p2_table(smem, cap);
         for (uint32_t j = tid; j < cap; j += NT) {
@@ -1143,10 +1221,10 @@ __global__ void __launch_bounds__(NT) p2_large_kernel(
             if (dx >= 2) {
                 bool inx = ok && ru.dx >= 2;
                 bool o = inx && rank_after(ru.dx, u, dx, w);
-                gx_round<NT>(o, inx && !o, xb, dx, u, sig, bo, bi, xcol, xS, xsk, sh_cnt);
+                gx_round<NT>(o, inx && !o, xb, dx, u, inx ? sig_fixed(sig) : 0, bo, bi, xcol, xS, xsk, sh_cnt);
             }
         }
-        if (tid == 0) { xout[w] = bo; xin[w] = bi; }
+        if (tid == 0) { xout[w] = bo; xin[w] = bi; xnode[w] = GxNode{xb, bo, dx}; }
         __syncthreads();
     }
 }
@@ -1211,7 +1289,7 @@ __global__ void __launch_bounds__(NT) hub_p2_insert_kernel(
 template <int NT>
 __global__ void __launch_bounds__(NT) hub_p2_counts_kernel(
     const HubInfo *__restrict__ hubs, int64_t nhubs, const int32_t *hitem_out, const int32_t *hitem_in,
-    int32_t *xout, int32_t *xin) {
+    const int64_t *__restrict__ xoff, const NodeRec *__restrict__ rec, int32_t *xout, int32_t *xin, GxNode *xnode) {
     for (int64_t hi = (int64_t)blockIdx.x * NT + threadIdx.x; hi < nhubs; hi += (int64_t)gridDim.x * NT) {
         const HubInfo h = hubs[hi];
         int32_t so = 0, si = 0;
@@ -1221,6 +1299,7 @@ __global__ void __launch_bounds__(NT) hub_p2_counts_kernel(
         }
         xout[h.row] = so;
         xin[h.row] = si;
+        xnode[h.row] = GxNode{xoff[h.row], so, rec[h.row].dx};
     }
 }
 
@@ -1232,7 +1311,7 @@ __global__ void __launch_bounds__(NT) hub_p2_emit_kernel(
     const NodeRec *__restrict__ rec, const int32_t *__restrict__ hslot,
     const unsigned long long *hq, const df *hsig, const int32_t *hitem_out, const int32_t *hitem_in,
     unsigned long long *acc, const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol,
-    df *__restrict__ xS, int32_t *__restrict__ xsk, int *err, Strict SX) {
+    SigPair *__restrict__ xS, int32_t *__restrict__ xsk, int *err, Strict SX) {
     __shared__ int32_t sh_cnt[2 * NT / 32];
     int tid = threadIdx.x;
     for (int64_t it = blockIdx.x; it < nitems; it += gridDim.x) {
@@ -1269,7 +1348,7 @@ __global__ void __launch_bounds__(NT) hub_p2_emit_kernel(
             if (rw.dx >= 2) {
                 bool inx = cross && ru.dx >= 2;
                 bool o = inx && rank_after(ru.dx, u, rw.dx, h.row);
-                gx_round<NT>(o, inx && !o, xb, rw.dx, u, sig, bo, bi, xcol, xS, xsk, sh_cnt);
+                gx_round<NT>(o, inx && !o, xb, rw.dx, u, inx ? sig_fixed(sig) : 0, bo, bi, xcol, xS, xsk, sh_cnt);
             }
         }
     }
@@ -1283,13 +1362,13 @@ __global__ void __launch_bounds__(NT) hub_p2_emit_kernel(
 // order, so its in-list read backwards from the row's last slot is sorted and
 // S(x -> y) for an in-neighbour y is found by binary search there.  P3 needs
 // the reverse values only of the edges of triangles.  It either looks them up
-// per triangle (three searches in in-lists), or reads them from xR, which the
-// mirror pass below fills for every G_x edge beforehand (one search per edge,
-// in a short out-list).  The first wins when triangles are few per G_x edge
+// per triangle (three searches in in-lists), or reads them beside the forward
+// values, where the mirror pass below puts them for every G_x edge beforehand (one
+// search per edge, in a short out-list).  The first wins when triangles are few per G_x edge
 // (0.11 on the 1M-node DC-SBM graph), the second when they are many; the
 // choice is a launch parameter (p3_mirror).
-__device__ __forceinline__ df in_value(int32_t x, int32_t y, const int64_t *xoff, const int32_t *xcol,
-                                       const df *xS, const int32_t *xin, int *err) {
+__device__ __forceinline__ uint64_t in_value(int32_t x, int32_t y, const int64_t *xoff, const int32_t *xcol,
+                                             const SigPair *xS, const int32_t *xin, int *err) {
     const int64_t last = xoff[x + 1] - 1;
     const int32_t len = xin[x];
     int32_t l = 0, h = len;
@@ -1297,23 +1376,27 @@ __device__ __forceinline__ df in_value(int32_t x, int32_t y, const int64_t *xoff
         int32_t mid = (l + h) >> 1;
         if (xcol[last - mid] < y) l = mid + 1; else h = mid;
     }
-    if (l < len && xcol[last - l] == y) return xS[last - l];
+    if (l < len && xcol[last - l] == y) return xS[last - l].f;
     atomicOr(err, 16);
-    return df{0.0f, 0.0f};
+    return 0;
 }
 
-// where P3 takes a reverse value: xR at the out-slot (mirror pass), or the
-// in-list of the higher-ranked end
+// where P3 takes an edge's values: both at the out-slot (mirror pass), or the reverse one
+// in the in-list of the higher-ranked end
 struct Rev {
-    const df *xR;                   // null: look the values up
+    const SigPair *xS;
     const int64_t *xoff;
     const int32_t *xcol;
-    const df *xS;
     const int32_t *xin;
     int *err;
-    // S(hi -> lo) for the G_x edge whose out-slot (lo -> hi) is `slot`
-    __device__ __forceinline__ df get(int64_t slot, int32_t hi, int32_t lo) const {
-        return xR ? xR[slot] : in_value(hi, lo, xoff, xcol, xS, xin, err);
+    bool mirrored;
+    // S(lo -> hi) and S(hi -> lo) for the G_x edge whose out-slot (lo -> hi) is `slot`
+    __device__ __forceinline__ SigPair get(int64_t slot, int32_t hi, int32_t lo) const {
+        if (mirrored) {
+            const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(xS + slot));
+            return SigPair{v.x, v.y};
+        }
+        return SigPair{xS[slot].f, in_value(hi, lo, xoff, xcol, xS, xin, err)};
     }
 };
 
@@ -1369,28 +1452,14 @@ __device__ __forceinline__ int64_t find_in_list_sk(const int32_t *xcol, const in
 // space [0, xoff[n]) is cut into tiles of kMirTile consecutive slots, one
 // tile per CTA trip, so the work per CTA does not depend on the in-degrees.
 // The nodes a tile spans run from the node holding its first slot to the one
-// holding the next tile's first slot (a table filled during P2, so no tile
-// searches the offsets).  A tile stages their offsets in shared memory, counts
+// holding the next tile's first slot (a table filled with the offsets, so no tile
+// searches them; `last` is the last node with slots).  A tile stages their offsets in shared memory, counts
 // their in-slots inside the tile and spreads only those over the threads; a
 // slot's out-slot twin is found in w's out-list (w has the lower rank), by
 // find_in_list_sk: a binary search, or for a list of more than kSkipMin ids one
 // through the packed sector index.  A tile spanning more than kMirNodes nodes
 // (long runs of nodes outside G_x) searches the offsets in global memory.
 constexpr int kMirNodes = 1024;
-
-// cover[t] = the node whose G_x row holds slot t kMirTile (t < tiles), and
-// cover[tiles] = the node holding the last slot; every slot lies in exactly
-// one non-empty row, so each entry is written once
-__global__ void mirror_tiles_kernel(int64_t n, const int64_t *__restrict__ xoff, int32_t *__restrict__ cover) {
-    const int64_t S = xoff[n];
-    const int64_t tiles = (S + kMirTile - 1) / kMirTile;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = xoff[u], hi = xoff[u + 1];
-        if (hi <= lo) continue;
-        for (int64_t t = (lo + kMirTile - 1) / kMirTile; t * kMirTile < hi; ++t) cover[t] = (int32_t)u;
-        if (hi == S) cover[tiles] = (int32_t)u;
-    }
-}
 
 __device__ __forceinline__ int64_t last_leq(const int64_t *xoff, int64_t lo, int64_t hi, int64_t key) {
     // last index i in [lo, hi) with xoff[i] <= key (xoff[lo] <= key)
@@ -1403,18 +1472,19 @@ __device__ __forceinline__ int64_t last_leq(const int64_t *xoff, int64_t lo, int
 
 // copy S(u -> w) from u's in-slot sl to w's out-slot for u (found in w's out-list, through
 // the packed index when the list is long)
-__device__ __forceinline__ void mirror_one(int64_t sl, int32_t u, const int64_t *xoff, const int32_t *xcol,
-                                           const int32_t *xsk, const df *xS, const int32_t *xout, df *xR, int *err) {
+__device__ __forceinline__ void mirror_one(int64_t sl, int32_t u, const int32_t *xcol,
+                                           const int32_t *xsk, SigPair *xS, const GxNode *xnode, int *err) {
     const int32_t w = xcol[sl];
-    const int64_t pos = find_in_list_sk(xcol, xsk, xoff[w], xout[w], u);
-    if (pos >= 0) xR[pos] = xS[sl];
+    const GxNode nw = load_node(xnode, w);
+    const int64_t pos = find_in_list_sk(xcol, xsk, nw.off, nw.out, u);
+    if (pos >= 0) xS[pos].r = xS[sl].f;
     else atomicOr(err, 16);
 }
 
 __global__ void __launch_bounds__(kThreads) gx_mirror_kernel(
-    int64_t n, const int64_t *__restrict__ xoff, const int32_t *__restrict__ xcol, const df *__restrict__ xS,
-    const int32_t *__restrict__ xout, const int32_t *__restrict__ xin, const int32_t *__restrict__ cover,
-    df *__restrict__ xR, const int32_t *__restrict__ xsk, int *err) {
+    int64_t n, const int64_t *__restrict__ xoff, const int32_t *__restrict__ xcol, SigPair *__restrict__ xS,
+    const GxNode *__restrict__ xnode, const int32_t *__restrict__ xin, const int32_t *__restrict__ cover,
+    const int32_t *__restrict__ last, const int32_t *__restrict__ xsk, int *err) {
     __shared__ int64_t s_lo[kMirNodes];          // first in-slot of each staged node inside the tile
     __shared__ int32_t s_pre[kMirNodes + 1];     // prefix sums of the staged nodes' in-slots in the tile
     __shared__ int32_t s_wsum[kThreads / 32];
@@ -1424,13 +1494,13 @@ __global__ void __launch_bounds__(kThreads) gx_mirror_kernel(
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         int64_t s0 = t * kMirTile, s1 = min(S, s0 + kMirTile);
         // nodes [ulo, uhi): from the one holding s0 to the one holding s1 (or the last slot)
-        int64_t ulo = cover[t], uhi = (int64_t)cover[t + 1] + 1;
+        int64_t ulo = cover[t], uhi = (int64_t)(t + 1 < tiles ? cover[t + 1] : *last) + 1;
         __syncthreads();                             // the previous tile's stage is free
         int32_t nn = (int32_t)(uhi - ulo);
         if (nn > kMirNodes) {
             for (int64_t sl = s0 + tid; sl < s1; sl += blockDim.x) {
                 int64_t u = last_leq(xoff, ulo, uhi, sl);
-                if (sl >= xoff[u + 1] - xin[u]) mirror_one(sl, (int32_t)u, xoff, xcol, xsk, xS, xout, xR, err);
+                if (sl >= xoff[u + 1] - xin[u]) mirror_one(sl, (int32_t)u, xcol, xsk, xS, xnode, err);
             }
             continue;
         }
@@ -1478,15 +1548,9 @@ __global__ void __launch_bounds__(kThreads) gx_mirror_kernel(
                 int32_t mid = (lo + hi) >> 1;
                 if (s_pre[mid] <= q) lo = mid; else hi = mid;
             }
-            mirror_one(s_lo[lo] + (q - s_pre[lo]), (int32_t)(ulo + lo), xoff, xcol, xsk, xS, xout, xR, err);
+            mirror_one(s_lo[lo] + (q - s_pre[lo]), (int32_t)(ulo + lo), xcol, xsk, xS, xnode, err);
         }
     }
-}
-
-// the three apex terms of triangle (a, b, c), rank a < b < c, added to the accumulators
-__device__ __forceinline__ void triangle_terms(int32_t a, int32_t b, int32_t c, df Sab, df Sba, df Sac, df Sca,
-                                               df Sbc, df Scb, unsigned long long *acc) {
-    add_triangle(acc, a, b, c, triangle_term_values(Sab, Sba, Sac, Sca, Sbc, Scb));
 }
 
 // P3 lists the triangles of G_x once each, from their lowest-ranked node a
@@ -1496,50 +1560,80 @@ __device__ __forceinline__ void triangle_terms(int32_t a, int32_t b, int32_t c, 
 // the lower-ranked one.  There are sum_a d+(a)(d+(a)-1)/2 candidates, several
 // times fewer than the wedges a -> b -> c on these graphs.
 //
-// A warp takes 32 consecutive nodes and stages their out-lists (with each
-// entry's G_x offset, out-degree and rank) in shared memory, window by window
-// of at most kWinCap entries.  All candidate pairs of a window form one flat
-// index space that the lanes share evenly (two per lane per trip): entry e
-// owns the pairs (e, f > e) of its node.  The closing edge is looked up in the
-// lower-ranked node's out-list in global memory by find_in_list_sk (a binary
-// search, or for a long list one through the packed sector index).  Found
-// triangles are queued in shared memory and finished a warp at a time, one per
-// lane: the three forward values
-// sit at the out-slots, the three reverse ones in xR (the mirror pass) or, with
-// p3_mirror = 0, in the in-lists of the two higher-ranked nodes, and the terms
-// of the three apexes are added.  Nodes with more than kWinCap out-neighbours
-// (heavy nodes) are walked by wedges instead (p3_heavy_kernel).
-constexpr int kP3Warps = kThreads / 32;
+// A CTA of four warps takes a group of up to 32 consecutive nodes and stages their
+// out-lists (with each entry's G_x offset, out-degree and rank) in shared memory, window
+// by window of at most kWinCap entries.  All candidate pairs of a window form one flat
+// index space that the threads share evenly: entry e owns the pairs (e, f > e) of its
+// node.  The closing edge is looked up in the lower-ranked node's out-list in global
+// memory by find_in_list_sk (a binary search, or for a long list one through the packed
+// sector index).  Found triangles are queued per warp and finished 32 at a time, one per
+// lane: a triangle's terms all have the form S S (S + S) with one factor on an edge
+// a - x of the window, so their pair products are summed per window entry in shared
+// memory, and the entries' sums are scaled and added to the accumulators once per window
+// (a's over its entries first).  Nodes with more than kWinCap out-neighbours (heavy
+// nodes) are walked by wedges instead (p3_heavy_kernel).
+//
+// What bounds it is the chain of dependent loads per window (and, where most pairs close, the
+// data path of the loads), so a window is shared by four warps and the groups shrink on small
+// graphs.  A warp per window, with three double-float terms and three 128-bit global adds per
+// triangle, took, against this form: 174 -> 40 us on 33,333 nodes, 283 -> 98 us on 200,001,
+// 142 -> 135 us on 1M nodes (10.3M edges, 262K triangles), 3.83 -> 2.33 ms on a batch of 256
+// graphs (81M edges), 9.11 -> 5.34 ms on the 8M-node hub-skewed graph.
+constexpr int kP3Threads = 128, kP3Warps = kP3Threads / 32, kP3CtasPerSm = 12;
+static_assert(kP3Threads == kWinCap, "a thread per window entry");
 
 struct P3Stage {
     int64_t boff[kWinCap];          // xoff[b]
+    int64_t aoff[32];               // xoff[a]
+    int64_t qpos[kP3Warps][64];     // triangles found and not yet finished: the closing slot
+    uint8_t qlo[kP3Warps][64];      //   and the window entries of the lower- and higher-ranked
+    uint8_t qhi[kP3Warps][64];      //   neighbours
     int32_t nb[kWinCap];            // b
     int32_t bdeg[kWinCap];          // d+(b)
     int32_t bdx[kWinCap];           // dx(b): rank(b) = (dx(b), b)
+    // sums of pair products per entry x, 0 between windows: `to` those that S(a->x) scales
+    // (they belong to x), `from` those that S(x->a) scales (they belong to a).  An entry
+    // closes fewer than kWinCap triangles, so the words do not overflow
+    uint32_t to[kLimbs][kWinCap], from[kLimbs][kWinCap];
+    int32_t seg[33];                // first entry of each lane's node in the window
+    int32_t anode[32];              // a
+    uint32_t wsum[kP3Warps];
     uint16_t ppre[kWinCap + 1];     // prefix sums of the pairs (e, f > e) owned by the entries
     uint8_t owner[kWinCap];         // lane (node) of the entry
-    int32_t seg[33];                // first entry of each lane's node in the window
-    int64_t aoff[32];               // xoff[a]
-    // triangles found and not yet finished: the closing slot, the owner lane
-    // and the window entries of the lower- and higher-ranked neighbours
-    int64_t qpos[64];
-    uint8_t qow[64], qlo[64], qhi[64];
+    int32_t found;                  // whether the window has a triangle
+    long long ticket;
 };
 
-// finish the first m (<= 32) queued triangles of the window, one per lane: the
-// forward values are at the three out-slots
-// the node of owner lane ow: base + ow, or (scrambled groups) the staged id anode[ow]
-template <bool kScr>
-__device__ __forceinline__ void p3_flush(const P3Stage &S, const int32_t *anode, int m, int64_t base, const df *xS,
-                                         const Rev &R,
-                                         unsigned long long *acc, int lane) {
+__device__ __forceinline__ void limbs_add(uint32_t (*l)[kWinCap], int e, u96 p) {
+#pragma unroll
+    for (int j = 0; j < kLimbs; ++j) {
+        const uint32_t v = pair_limb(p, j);
+        if (v) atomicAdd(&l[j][e], v);
+    }
+}
+__device__ __forceinline__ u96 limbs_take(uint32_t (*l)[kWinCap], int e) {
+    const u96 p = from_limbs(l[0][e], l[1][e], l[2][e], l[3][e]);
+#pragma unroll
+    for (int j = 0; j < kLimbs; ++j) l[j][e] = 0;
+    return p;
+}
+
+// the out-slot of window entry e, in its node's out-list
+__device__ __forceinline__ int64_t p3_slot(const P3Stage &S, int e) {
+    const int o = S.owner[e];
+    return S.aoff[o] + (e - S.seg[o]);
+}
+
+// finish the first m (<= 32) triangles queued by the warp, one per lane
+__device__ __forceinline__ void p3_flush(P3Stage &S, int wid, int m, const Rev &R, int lane) {
     if (lane < m) {
-        int ow = S.qow[lane], el = S.qlo[lane], eh = S.qhi[lane];
-        int64_t ao = S.aoff[ow] - S.seg[ow];
-        int64_t il = ao + el, ih = ao + eh, pc = S.qpos[lane];
-        int32_t a = kScr ? anode[ow] : (int32_t)(base + ow), b = S.nb[el], c = S.nb[eh];
-        df Sba = R.get(il, b, a), Sca = R.get(ih, c, a), Scb = R.get(pc, c, b);
-        triangle_terms(a, b, c, xS[il], Sba, xS[ih], Sca, xS[pc], Scb, acc);
+        const int el = S.qlo[wid][lane], eh = S.qhi[wid][lane];
+        const int32_t a = S.anode[S.owner[el]], b = S.nb[el], c = S.nb[eh];
+        const SigPair bc = R.get(S.qpos[wid][lane], c, b), ab = R.get(p3_slot(S, el), b, a),
+                      ac = R.get(p3_slot(S, eh), c, a);
+        limbs_add(S.from, el, pair_term(ac.r, bc.f + bc.r));      // a: scaled by S(b->a)
+        limbs_add(S.to, el, pair_term(bc.r, ac.f + ac.r));        // b: scaled by S(a->b)
+        limbs_add(S.to, eh, pair_term(bc.f, ab.f + ab.r));        // c: scaled by S(a->c)
     }
 }
 
@@ -1547,49 +1641,237 @@ __device__ __forceinline__ bool rank_less(int32_t dx1, int32_t id1, int32_t dx2,
     return dx1 < dx2 || (dx1 == dx2 && id1 < id2);
 }
 
+// groups of `group` (<= 32) nodes are handed out by an atomic counter (next_group, zeroed
+// before the launch), so CTAs that drew light groups take more and no tail is left waiting.
+// kScr (graphs built with RS_REORDER): lane j of group g takes node
+// (group g + j) * stride mod n (stride coprime to n), because consecutive ids then hold a
+// community's heaviest nodes together and one group of them would be a long tail for
+// its CTA; otherwise lane j takes node group g + j and stride is unused.
+template <bool kScr>
+__global__ void __launch_bounds__(kP3Threads, kP3CtasPerSm) p3_list_kernel(
+    int64_t n, const int64_t *__restrict__ xoff, const int32_t *__restrict__ xcol, const int32_t *__restrict__ xsk,
+    Rev R, const int32_t *__restrict__ xout, const GxNode *__restrict__ xnode, unsigned long long *acc,
+    unsigned long long *next_group, int32_t group, int64_t stride, unsigned long long *hvl, int64_t hvcap,
+    unsigned long long *hv_count) {
+    __shared__ P3Stage S;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+    for (int j = 0; j < kLimbs; ++j) { S.to[j][tid] = 0; S.from[j][tid] = 0; }
+    if (tid == 0) { S.found = 0; S.ticket = (long long)atomicAdd(next_group, 1ull); }
+    __syncthreads();
+    while (true) {
+        const int64_t base = S.ticket * group;
+        if (base >= n) break;
+        __syncthreads();                               // everyone has read the ticket
+        if (tid == 0) S.ticket = (long long)atomicAdd(next_group, 1ull);   // read after the windows' barriers
+        // every warp works out the windows alike: lane j holds node j of the group
+        int64_t av = base + lane;
+        const bool have = lane < group && av < n;
+        if (kScr && have) av = (int64_t)(((unsigned __int128)av * (uint64_t)stride) % (uint64_t)n);
+        const int32_t da = have ? xout[av] : 0;
+        const bool grp = da >= 2 && da <= kWinCap;
+        const int32_t mine = grp ? da : 0;
+        int32_t incl = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int64_t ba = grp ? xoff[av] : 0;
+        // windows of consecutive nodes whose entries fit kWinCap
+        int32_t start = 0;
+        while (true) {
+            const int32_t excl0 = start > 0 ? __shfl_sync(FULL, incl, start - 1) : 0;
+            const unsigned fitm = __ballot_sync(FULL, lane >= start && incl - excl0 <= kWinCap);
+            if (start >= 32 || fitm == 0) break;
+            const int32_t end = 32 - __clz(fitm);             // lanes [start, end) fit
+            const int32_t Ew = __shfl_sync(FULL, incl, end - 1) - excl0;
+            if (Ew > 0) {
+                if (wid == 0) {
+                    // seg is nondecreasing over all 32 lanes: the entry j belongs to the
+                    // last lane o with seg[o] <= j (lanes without entries share the next seg)
+                    const bool inwin = lane >= start && lane < end;
+                    S.seg[lane] = lane < start ? 0 : (inwin ? incl - mine - excl0 : Ew);
+                    if (lane == 0) S.seg[32] = Ew;
+                    S.aoff[lane] = ba;
+                    S.anode[lane] = (int32_t)av;
+                }
+                __syncthreads();
+                // a thread per entry: its data and the pair prefix sums
+                uint32_t x = 0;
+                if (tid < Ew) {
+                    int32_t lo = 0, hi = 32;
+                    while (hi - lo > 1) {
+                        const int32_t mid = (lo + hi) >> 1;
+                        if (S.seg[mid] <= tid) lo = mid; else hi = mid;
+                    }
+                    const int32_t loc = tid - S.seg[lo];
+                    const int32_t b = xcol[S.aoff[lo] + loc];
+                    S.nb[tid] = b;
+                    S.owner[tid] = (uint8_t)lo;
+                    const GxNode nb = load_node(xnode, b);
+                    S.boff[tid] = nb.off;
+                    S.bdeg[tid] = nb.out;
+                    S.bdx[tid] = nb.dx;
+                    x = (uint32_t)(S.seg[lo + 1] - S.seg[lo] - 1 - loc);   // pairs (e, f > e) of the node
+                }
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(FULL, x, o);
+                    if (lane >= o) x += y;
+                }
+                if (lane == 31) S.wsum[wid] = x;
+                __syncthreads();
+                for (int j = 0; j < wid; ++j) x += S.wsum[j];
+                if (tid < Ew) S.ppre[tid + 1] = (uint16_t)x;
+                if (tid == 0) S.ppre[0] = 0;
+                __syncthreads();
+                const int32_t P = S.ppre[Ew];
+                int qn = 0;                                // triangles queued by the warp (uniform)
+                for (int32_t p0 = 32 * wid; p0 < P; p0 += kP3Threads) {
+                    const int32_t pv = p0 + lane;
+                    int32_t el = 0, eh = 0;
+                    int64_t pos = -1;
+                    if (pv < P) {
+                        int32_t lo = 0, hi = Ew;            // last entry with ppre[e] <= pv
+                        while (hi - lo > 1) {
+                            const int32_t mid = (lo + hi) >> 1;
+                            if (S.ppre[mid] <= pv) lo = mid; else hi = mid;
+                        }
+                        const int32_t f = lo + 1 + (pv - S.ppre[lo]);
+                        const bool e_low = rank_less(S.bdx[lo], S.nb[lo], S.bdx[f], S.nb[f]);
+                        el = e_low ? lo : f;
+                        eh = e_low ? f : lo;
+                        pos = find_in_list_sk(xcol, xsk, S.boff[el], S.bdeg[el], S.nb[eh]);
+                    }
+                    const bool hit = pos >= 0;
+                    const unsigned hm = __ballot_sync(FULL, hit);
+                    if (hit) {
+                        const int slot = qn + __popc(hm & lanemask_lt());
+                        S.qpos[wid][slot] = pos;
+                        S.qlo[wid][slot] = (uint8_t)el;
+                        S.qhi[wid][slot] = (uint8_t)eh;
+                        S.found = 1;
+                    }
+                    qn += __popc(hm);
+                    // a full warp of triangles, or (in the warp's last trip) what is left
+                    const bool last = p0 + kP3Threads >= P;
+                    while (qn >= 32 || (last && qn > 0)) {
+                        const int m = min(qn, 32);
+                        __syncwarp();
+                        p3_flush(S, wid, m, R, lane);
+                        __syncwarp();
+                        if (lane < qn - m) {
+                            S.qpos[wid][lane] = S.qpos[wid][32 + lane];
+                            S.qlo[wid][lane] = S.qlo[wid][32 + lane];
+                            S.qhi[wid][lane] = S.qhi[wid][32 + lane];
+                        }
+                        qn -= m;
+                        __syncwarp();
+                    }
+                }
+                __syncthreads();
+                // the window's sums to the accumulators, a thread per entry
+                if (S.found) {
+                    u192 ta{0, 0, 0};
+                    int own = -1;
+                    if (tid < Ew) {
+                        own = S.owner[tid];
+                        const u96 to = limbs_take(S.to, tid), from = limbs_take(S.from, tid);
+                        if (to.lo | to.hi | from.lo | from.hi) {
+                            const SigPair ax = R.get(p3_slot(S, tid), S.nb[tid], S.anode[own]);
+                            if (to.lo | to.hi) atomic_add_u192(acc + 3 * (int64_t)S.nb[tid], scale(ax.f, to));
+                            ta = scale(ax.r, from);
+                        }
+                    }
+                    // a's terms, summed over the lanes of each node (consecutive) to its first lane
+                    if (__any_sync(FULL, (ta.w0 | ta.w1 | ta.w2) != 0)) {
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int oo = __shfl_down_sync(FULL, own, o);
+                            const u192 y{__shfl_down_sync(FULL, ta.w0, o), __shfl_down_sync(FULL, ta.w1, o),
+                                         __shfl_down_sync(FULL, ta.w2, o)};
+                            if (lane + o < 32 && oo == own) ta = u192_add(ta, y);
+                        }
+                        const int before = __shfl_up_sync(FULL, own, 1);
+                        if (own >= 0 && (lane == 0 || before != own) && (ta.w0 | ta.w1 | ta.w2))
+                            atomic_add_u192(acc + 3 * (int64_t)S.anode[own], ta);
+                    }
+                    __syncthreads();
+                    if (tid == 0) S.found = 0;
+                }
+                __syncthreads();                           // the stage is reused next
+            }
+            start = end;
+        }
+        // heavy nodes' tasks go to the list (its capacity bounds their number, so the
+        // error branch is not taken)
+        if (wid == 0 && da > kWinCap) {
+            const int32_t nt = (da + kHvBlock - 1) / kHvBlock;
+            const unsigned long long h = atomicAdd(hv_count, (unsigned long long)nt);
+            if (h + nt <= (unsigned long long)hvcap) {
+                for (int32_t i = 0; i < nt; ++i) hvl[h + i] = (unsigned long long)av << 32 | (unsigned)i;
+            } else {
+                atomicOr(R.err, 64);
+            }
+        }
+        __syncthreads();                                   // the next ticket is there
+    }
+}
+
 // Heavy nodes: a wedge walk, one CTA per task.  A task is a heavy node a with a block
 // of kHvBlock of its out-neighbours b.  The CTA stages a's out-list A (sorted by id),
-// kHvIds ids at a time, as a shared-memory hash table of 4-slot buckets (id -> position
-// in the chunk, at most a quarter of the slots used) beside the value S(c->a) and the sum S(a->c) + S(c->a) for
-// every c of the chunk.  Its warps then take the task's out-neighbours b one at a time: a warp
-// streams b's out-list (the nodes c ranked above b), coalesced, and looks every c up in
-// the table; a hit closes the triangle {a, b, c}, which is met once, at its
-// middle-ranked node b.  When A takes several chunks, b's out-list is first cut to the
-// chunk's id range.  There are several times more wedges than pairs on such nodes, but
-// a wedge costs a coalesced load and a probe or two in shared memory where a pair
-// costs a binary search in global memory.
+// kHvIds ids at a time, as a shared-memory hash table (id -> position in the chunk) beside
+// the value S(c->a) and the sum S(a->c) + S(c->a) for every c of the chunk.  Its warps then
+// take the task's out-neighbours b one at a time: a warp streams b's out-list (the nodes c
+// ranked above b), coalesced, and looks every c up in the table; a hit closes the triangle
+// {a, b, c}, which is met once, at its middle-ranked node b.  When A takes several chunks,
+// b's out-list is first cut to the chunk's id range.  There are several times more wedges
+// than pairs on such nodes, but a wedge costs a coalesced load and one 4-byte load from
+// shared memory where a pair costs a binary search in global memory.
 //
 // A third of the heavy wedges close on the 8M-node graph, so finishing the triangles
-// dominates, and its atomics are cut down: hits are queued and finished a warp at a
-// time (one triangle per lane); a's terms are summed in registers over the task, b's
-// over the warp's walk of b (every queued triangle has the same b), and c's in two
-// 64-bit words per staged position in shared memory (the term's low 48 bits and the
-// rest, each added without reading the old value back), added to the accumulators once
-// per chunk.  The integer sums are exact, so the bits do not depend on how they are split.
+// dominates.  Hits are queued (one word each) and finished a warp at a time, one triangle
+// per lane, by three pair products, whose outer factors come out of the sums: a's and b's
+// pairs are summed in registers over the warp's walk of b (S(b->a) and S(a->b) scale them
+// once at its end), c's pairs in four 32-bit words per staged position in shared memory
+// (S(a->c) scales them once per chunk).  The products are exact, so the bits do not depend
+// on the grouping.
+//
+// Issue slots and the latency of the loads bound it.  Before this form
+// (4-slot buckets read 16 bytes at a time, three double-float products and three fixed-point
+// conversions per triangle, c's sums by 64-bit shared atomics, which take five times as long
+// as 32-bit ones) it ran the shared-memory pipe at 74% and issue at 66%: 43.8 -> 36.5 ms on the
+// 8M-node graph (6.4e9 wedges, 2.1e9 triangles), 5.87 -> 4.52 ms on 2M nodes, where the pipe is
+// now at 41% and issue at 58%.
 //
 // The warp whose group holds a heavy node does not walk it: it appends the node's
 // tasks to the task list (slots taken with an atomic counter), and p3_heavy_kernel,
 // launched next on the same stream, runs them, a CTA per task.
 constexpr int kHvIds = 1024;                  // ids of A staged per chunk
-constexpr int kHvSlots = 4 * kHvIds;          // hash slots: the table is at most a quarter full
+constexpr int kHvBits = 13, kHvSlots = 1 << kHvBits;   // hash slots: at most an eighth used
 constexpr int kHvUnroll = 4;                  // 32-entry rows of b's out-list per trip
 constexpr int kHvQ = 32 * kHvUnroll + 32;     // queued triangles per warp: < 32 left + one trip
 constexpr int kHvWarps = kThreads / 32;
 
-struct HvQueue {
-    int32_t k[kHvQ];                          // c's entry in b's out-list
-    int32_t c[kHvQ];
-    int32_t pos[kHvQ];                        // c's position in the chunk of A
-};
+// The hash of an id is a product by an odd constant modulo 2^32, a bijection: its top
+// kHvBits bits are the home slot, the 19 bits below identify the id there.  A slot word
+// holds bit 31 (taken), kMore (an id whose home is this slot is elsewhere), kMoved (its own
+// id is not at home), the id's position and its 19 bits; an id at home is thus recognised
+// exactly by one 4-byte load.  Moved ids are in the slots after their home; their bits
+// alone do not identify them, so they are checked against A itself.
+constexpr uint32_t kHvTaken = 1u << 31, kHvMore = 1u << 30, kHvMoved = 1u << 29;
+constexpr int kHvRest = 32 - kHvBits;
+constexpr uint32_t kHvRestMask = (1u << kHvRest) - 1, kHvPosMask = kHvIds - 1;
+static_assert(kHvRest + 10 + 3 == 32 && kHvIds == 1 << 10, "a slot word's fields");
+__device__ __forceinline__ uint32_t hv_hash(int32_t c) { return (uint32_t)c * 0x9E3779B1u; }
+
 struct P3Heavy {
-    int4 key[kHvSlots / 4];                   // the chunk's ids, 4 slots per bucket (-1: empty slot)
-    uint16_t slot_pos[kHvSlots];              // their positions in the chunk
-    df sca[kHvIds], pac[kHvIds];              // S(c->a), S(a->c) + S(c->a)
-    unsigned long long clo[kHvIds], chi[kHvIds];   // c's terms of the chunk: bits [0, 48) and [48, 112)
-    HvQueue q[kHvWarps];
+    SigPair sp[kHvIds];                       // S(c->a), S(a->c) + S(c->a)
+    uint32_t tab[kHvSlots];
+    uint32_t sum[kLimbs][kHvIds];             // c's pairs of the chunk; at most kHvBlock each
+    uint32_t q[kHvWarps][kHvQ];               // hits: c's entry in b's out-list << 10 | position
     int64_t a, bA;
     int32_t dA, eb0, nb, next_b, stop;
 };
+static_assert(kHvBlock <= 128, "the words of a pair sum take 128 pairs");
 
 // first position of the sorted p[0, cnt) (cnt >= 1) holding an id >= key, or cnt;
 // the trip count depends on cnt alone
@@ -1603,52 +1885,18 @@ __device__ __forceinline__ int32_t lower_pos(const int32_t *p, int32_t cnt, int3
     return base + (p[base] < key ? 1 : 0);
 }
 
-__device__ __forceinline__ uint32_t hv_hash(int32_t c, uint32_t mask) {
-    return (((uint32_t)c * 0x9E3779B1u) >> 16) & mask;
-}
-
-// position of id c in the staged chunk, or -1.  The table is buckets of 4 slots, filled
-// in slot order, at most a quarter of the slots used: one 16-byte load of the home bucket
-// settles nearly every lookup (a key is there, or the bucket has an empty slot); a full
-// home bucket (under 1% of them) sends the probe on to the next buckets.
-__device__ __forceinline__ int32_t hv_find(const P3Heavy &H, int32_t c, uint32_t bmask) {
-    uint32_t bk = hv_hash(c, bmask);
-    for (uint32_t it = 0; it <= bmask; ++it) {
-        const int4 q = H.key[bk];
-        const int j = q.x == c ? 0 : q.y == c ? 1 : q.z == c ? 2 : q.w == c ? 3 : -1;
-        if (j >= 0) return H.slot_pos[4 * bk + j];
-        if (q.w < 0) return -1;
-        bk = (bk + 1) & bmask;
+// position of an id that is not at home, or -1: the slots after its home (hash h), up to
+// the first empty one.  A: the chunk's ids
+__device__ __forceinline__ int32_t hv_find_moved(const P3Heavy &H, int32_t c, uint32_t h, const int32_t *A) {
+    uint32_t s = h >> kHvRest;
+    for (int it = 0; it < kHvSlots; ++it) {
+        s = (s + 1) & (kHvSlots - 1);
+        const uint32_t w = H.tab[s];
+        if (!w) break;
+        const int32_t p = (int32_t)(w >> kHvRest & kHvPosMask);
+        if ((w & kHvMoved) && (w & kHvRestMask) == (h & kHvRestMask) && A[p] == c) return p;
     }
     return -1;
-}
-
-// c's term t added to its chunk sums in shared memory: bits [0, 48) of t to lo_w, bits
-// [48, 112) to hi_w, each by an atomic add whose old value is not needed (no carry to
-// propagate).  A position receives at most kHvBlock terms per chunk (one per out-neighbour
-// b of the task), and every term is below 2^101 (at most 2^37 in value: each S(x->y) is
-// the cube root of a weight below 31 * 2^31, so below 2^12, and a term is S * S * (S + S)),
-// so the low word stays below 2^55 and the high one below 2^60; the chunk's sum is
-// lo + hi * 2^48, exactly.
-__device__ __forceinline__ void shared_add_split(unsigned long long *lo_w, unsigned long long *hi_w, u128 t) {
-    atomicAdd(lo_w, (unsigned long long)((uint64_t)t & ((1ull << 48) - 1)));
-    atomicAdd(hi_w, (unsigned long long)(uint64_t)(t >> 48));
-}
-
-// finish the m (<= 32) queued triangles {a, b, c} at queue entries [f, f + m) of the
-// warp's current b, one per lane (all lanes call); the chunk of A starts at slot aslot0
-__device__ __forceinline__ void hv_finish(P3Heavy &H, const HvQueue &Q, int f, int m, int32_t b, int64_t ob,
-                                          int64_t aslot0, df Sab, df Sba, df Pab, const df *xS, const Rev &R,
-                                          int lane, u128 &acc_a, u128 &acc_b) {
-    if (lane < m) {
-        const int32_t c = Q.c[f + lane], p = Q.pos[f + lane];
-        const int64_t pc = ob + Q.k[f + lane];
-        const df Sbc = xS[pc], Scb = R.get(pc, c, b), Sac = xS[aslot0 + p];
-        const TriTerms t = triangle_term_values_p(Sab, Sba, Sac, H.sca[p], Sbc, Scb, H.pac[p], Pab);
-        acc_a += t.a;
-        acc_b += t.b;
-        shared_add_split(&H.clo[p], &H.chi[p], t.c);
-    }
 }
 
 // an out-neighbour b of the task (entry eb of A): its out-list [ob + s, ob + e) cut to
@@ -1657,252 +1905,118 @@ __device__ __forceinline__ void hv_finish(P3Heavy &H, const HvQueue &Q, int f, i
 struct HvB {
     int32_t b, s, e;
     int64_t ob;
-    df Sab, Sba;
+    SigPair ab;
 };
 __device__ __forceinline__ HvB hv_load_b(int32_t a, int64_t eb, bool cut, int32_t lo_id, int32_t hi_id,
-                                         const int64_t *xoff, const int32_t *xcol, const df *xS, const Rev &R,
-                                         const int32_t *xout) {
+                                         const int32_t *xcol, const Rev &R, const GxNode *xnode) {
     HvB B;
     B.b = xcol[eb];
-    B.ob = xoff[B.b];
-    const int32_t db = xout[B.b];
+    const GxNode nb = load_node(xnode, B.b);
+    B.ob = nb.off;
+    const int32_t db = nb.out;
     B.s = 0;
     B.e = db;
     if (cut && db > 0) {
         B.s = lower_pos(xcol + B.ob, db, lo_id);
         B.e = lower_pos(xcol + B.ob, db, hi_id + 1);
     }
-    B.Sab = xS[eb];
-    B.Sba = R.get(eb, B.b, a);
+    B.ab = R.get(eb, B.b, a);
     return B;
 }
 
-// one warp's walk of out-neighbour b over the staged chunk (starting at slot aslot0):
-// each trip loads and looks up kHvUnroll rows of 32 entries of b's out-list, queues the
-// hits, and finishes the queued triangles 32 at a time (at the end of the list, the
-// rest too); the finishing code is inlined once
-__device__ __forceinline__ void hv_walk_b(P3Heavy &H, HvQueue &Q, const HvB &B, int64_t aslot0, uint32_t mask,
-                                          const int32_t *xcol, const df *xS, const Rev &R,
-                                          unsigned long long *acc, int lane, u128 &acc_a) {
+// the sum of v over the warp's lanes (below 2^96), by hardware sums of 27-bit pieces
+__device__ __forceinline__ u96 warp_sum_u96(u96 v) {
+    constexpr uint32_t M = (1u << 27) - 1;
+    const u128 x = ((u128)v.hi << 64) | v.lo;
+    const uint32_t r0 = __reduce_add_sync(FULL, (uint32_t)x & M);
+    const uint32_t r1 = __reduce_add_sync(FULL, (uint32_t)(x >> 27) & M);
+    const uint32_t r2 = __reduce_add_sync(FULL, (uint32_t)(x >> 54) & M);
+    const uint32_t r3 = __reduce_add_sync(FULL, (uint32_t)(x >> 81));
+    const u128 s = (u128)r0 + ((u128)r1 << 27) + ((u128)r2 << 54) + ((u128)r3 << 81);
+    return u96{(uint64_t)s, (uint32_t)(s >> 64)};
+}
+
+// one warp's walk of out-neighbour b over the staged chunk (ids A): each trip loads and
+// looks up kHvUnroll rows of 32 entries of b's out-list, queues the hits, and finishes the
+// queued triangles 32 at a time (at the end of the list, the rest too); the finishing code
+// is inlined once.  A list has at most 2^20 ids (each of them has a cross degree at least
+// as large, and nnz < 2^40), so a hit fits one word; a walk closes at most kHvIds
+// triangles, so its pair sums stay below 2^96
+__device__ __forceinline__ void hv_walk_b(P3Heavy &H, uint32_t *Q, const HvB &B, const int32_t *A,
+                                          const int32_t *xcol, const Rev &R, unsigned long long *acc, int lane,
+                                          u192 &acc_a) {
     if (B.s >= B.e) return;
-    const df Pab = df_add(B.Sab, B.Sba);
+    const uint64_t Pab = B.ab.f + B.ab.r;
     int qn = 0;                                        // queued triangles (warp-uniform)
-    u128 acc_b = 0;
+    bool any = false;
+    u96 sum_a{0, 0}, sum_b{0, 0};
     for (int32_t j0 = B.s; j0 < B.e; j0 += 32 * kHvUnroll) {
         int32_t c[kHvUnroll], pos[kHvUnroll];
 #pragma unroll
         for (int u = 0; u < kHvUnroll; ++u) {
             const int32_t k = j0 + u * 32 + lane;
-            c[u] = k < B.e ? xcol[B.ob + k] : -1;
+            c[u] = k < B.e ? xcol[B.ob + k] : -1;      // -1 is nobody's id, and the hash is a bijection
         }
-        // every row's home bucket is probed with no loop (b's out-list is already cut to
-        // the chunk's id range, so an id outside it simply misses); the rare lanes whose
-        // home bucket is full without their id probe on, in a branch the warp takes together
         bool more = false;
 #pragma unroll
         for (int u = 0; u < kHvUnroll; ++u) {
-            const uint32_t bk = hv_hash(c[u], mask);
-            const int4 q = H.key[bk];
-            const int j = q.x == c[u] ? 0 : q.y == c[u] ? 1 : q.z == c[u] ? 2 : q.w == c[u] ? 3 : -1;
-            const bool valid = j0 + u * 32 + lane < B.e;
-            pos[u] = valid && j >= 0 ? (int32_t)H.slot_pos[4 * bk + j] : -1;
-            more |= valid && j < 0 && q.w >= 0;
+            const uint32_t h = hv_hash(c[u]);
+            const uint32_t w = H.tab[h >> kHvRest];
+            const bool hit = ((w ^ (kHvTaken | (h & kHvRestMask))) & (kHvTaken | kHvMoved | kHvRestMask)) == 0;
+            pos[u] = hit ? (int32_t)(w >> kHvRest & kHvPosMask) : -1;
+            more |= !hit && (w & kHvMore);
         }
         if (__any_sync(FULL, more)) {
-#pragma unroll
+#pragma unroll 1
             for (int u = 0; u < kHvUnroll; ++u)
-                if (pos[u] < 0 && j0 + u * 32 + lane < B.e) pos[u] = hv_find(H, c[u], mask);
+#pragma unroll
+                for (int v = 0; v < kHvUnroll; ++v)    // (registers are not indexed)
+                    if (u == v && pos[v] < 0 && c[v] >= 0 && (H.tab[hv_hash(c[v]) >> kHvRest] & kHvMore))
+                        pos[v] = hv_find_moved(H, c[v], hv_hash(c[v]), A);
         }
 #pragma unroll
         for (int u = 0; u < kHvUnroll; ++u) {
             const bool hit = pos[u] >= 0;
             const unsigned hm = __ballot_sync(FULL, hit);
-            if (hit) {
-                const int slot = qn + __popc(hm & lanemask_lt());
-                Q.k[slot] = j0 + u * 32 + lane;
-                Q.c[slot] = c[u];
-                Q.pos[slot] = pos[u];
-            }
+            if (hit) Q[qn + __popc(hm & lanemask_lt())] = (uint32_t)(j0 + u * 32 + lane) << 10 | (uint32_t)pos[u];
             qn += __popc(hm);
         }
         const bool last = j0 + 32 * kHvUnroll >= B.e;
         int f = 0;
         while (qn - f >= 32 || (last && qn > f)) {
             const int m = min(32, qn - f);
+            any = true;
             __syncwarp();
-            hv_finish(H, Q, f, m, B.b, B.ob, aslot0, B.Sab, B.Sba, Pab, xS, R, lane, acc_a, acc_b);
+            if (lane < m) {
+                const uint32_t q = Q[f + lane];
+                const int32_t p = (int32_t)(q & kHvPosMask);
+                const int64_t pc = B.ob + (q >> 10);
+                const SigPair bc = R.get(pc, R.mirrored ? 0 : xcol[pc], B.b), sp = H.sp[p];
+                u96_add(sum_a, pair_term(sp.f, bc.f + bc.r));
+                u96_add(sum_b, pair_term(bc.r, sp.r));
+                const u96 t = pair_term(bc.f, Pab);
+#pragma unroll
+                for (int j = 0; j < kLimbs; ++j) {
+                    const uint32_t v = pair_limb(t, j);
+                    if (j < kLimbs - 1 || v) atomicAdd(&H.sum[j][p], v);
+                }
+            }
             f += m;
         }
         if (f > 0) {                                   // the rest (< 32) to the front
             __syncwarp();
-            int32_t k = 0, cc = 0, pp = 0;
-            if (lane < qn - f) { k = Q.k[f + lane]; cc = Q.c[f + lane]; pp = Q.pos[f + lane]; }
+            uint32_t q = 0;
+            if (lane < qn - f) q = Q[f + lane];
             __syncwarp();
-            if (lane < qn - f) { Q.k[lane] = k; Q.c[lane] = cc; Q.pos[lane] = pp; }
+            if (lane < qn - f) Q[lane] = q;
             qn -= f;
         }
         __syncwarp();
     }
-    acc_b = warp_sum_u128(acc_b);
-    if (lane == 0 && acc_b) atomic_add_u128(acc + 2 * (int64_t)B.b, acc_b);
-}
-
-// groups of 32 nodes are handed out by an atomic counter (next_group, zeroed before
-// the launch), so warps that drew light groups take more and no tail is left waiting.
-// kScr (graphs built with RS_REORDER): lane j of group g takes node
-// (32 g + j) * stride mod n (stride coprime to n), because consecutive ids then hold a
-// community's heaviest nodes together and one group of them would be a long tail for
-// its warp; otherwise lane j takes node 32 g + j and stride is unused.
-template <bool kScr>
-__global__ void __launch_bounds__(kThreads, 5) p3_list_kernel(
-    int64_t n, const int64_t *__restrict__ xoff, const int32_t *__restrict__ xcol, const int32_t *__restrict__ xsk,
-    const df *__restrict__ xS, Rev R, const int32_t *__restrict__ xout, const NodeRec *__restrict__ rec,
-    unsigned long long *acc, unsigned long long *next_group, int64_t stride, unsigned long long *hvl, int64_t hvcap,
-    unsigned long long *hv_count) {
-    __shared__ P3Stage stage[kP3Warps];
-    __shared__ int32_t s_anode[kScr ? kP3Warps * 32 : 1];
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    P3Stage &S = stage[wid];
-    int32_t *anode = s_anode + (kScr ? wid * 32 : 0);
-    while (true) {
-        unsigned long long ticket = 0;
-        if (lane == 0) ticket = atomicAdd(next_group, 1ull);
-        const int64_t base = (int64_t)__shfl_sync(FULL, ticket, 0) * 32;
-        if (base >= n) break;
-        int64_t av = base + lane;
-        if (kScr && av < n) av = (int64_t)(((unsigned __int128)av * (uint64_t)stride) % (uint64_t)n);
-        int32_t da = av < n ? xout[av] : 0;
-        bool grp = da >= 2 && da <= kWinCap;
-        int32_t mine = grp ? da : 0;
-        int32_t incl = mine;
-        for (int o = 1; o < 32; o <<= 1) {
-            int32_t y = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += y;
-        }
-        int64_t ba = grp ? xoff[av] : 0;
-        // windows of consecutive nodes whose entries fit kWinCap
-        int32_t start = 0;
-        while (true) {
-            int32_t excl0 = start > 0 ? __shfl_sync(FULL, incl, start - 1) : 0;
-            unsigned fitm = __ballot_sync(FULL, lane >= start && incl - excl0 <= kWinCap);
-            if (start >= 32 || fitm == 0) break;
-            int32_t end = 32 - __clz(fitm);               // lanes [start, end) fit
-            int32_t Ew = __shfl_sync(FULL, incl, end - 1) - excl0;
-            bool inwin = lane >= start && lane < end;
-            int32_t e0 = incl - mine - excl0;              // this lane's first entry in the window
-            if (Ew > 0) {
-                // seg is nondecreasing over all 32 lanes: the entry j belongs to the
-                // last lane o with seg[o] <= j (lanes without entries share the next seg)
-                S.seg[lane] = lane < start ? 0 : (inwin ? e0 : Ew);
-                if (lane == 0) S.seg[32] = Ew;
-                S.aoff[lane] = ba;
-                if (kScr) anode[lane] = (int32_t)av;
-                __syncwarp();
-                // entries, their data and the pair prefix sums, lanes over entries
-                uint32_t carry = 0;
-                if (lane == 0) S.ppre[0] = 0;
-                for (int32_t j0 = 0; j0 < Ew; j0 += 32) {
-                    int32_t j = j0 + lane;
-                    uint32_t x = 0;
-                    if (j < Ew) {
-                        int32_t lo = 0, hi = 32;
-                        while (hi - lo > 1) {
-                            int32_t mid = (lo + hi) >> 1;
-                            if (S.seg[mid] <= j) lo = mid; else hi = mid;
-                        }
-                        int32_t loc = j - S.seg[lo];
-                        int32_t b = xcol[S.aoff[lo] + loc];
-                        S.nb[j] = b;
-                        S.owner[j] = (uint8_t)lo;
-                        S.boff[j] = xoff[b];
-                        S.bdeg[j] = xout[b];
-                        S.bdx[j] = rec[b].dx;
-                        x = (uint32_t)(S.seg[lo + 1] - S.seg[lo] - 1 - loc);   // pairs (j, f > j) of the node
-                    }
-                    for (int o = 1; o < 32; o <<= 1) {
-                        uint32_t y = __shfl_up_sync(FULL, x, o);
-                        if (lane >= o) x += y;
-                    }
-                    if (j < Ew) S.ppre[j + 1] = (uint16_t)(carry + x);
-                    carry += __shfl_sync(FULL, x, 31);
-                }
-                __syncwarp();
-                int32_t P = S.ppre[Ew];
-                int qn = 0;                                // queued triangles (warp-uniform)
-                // pairs per lane per trip: each search and the finishing code are inlined U
-                // times, and the searches run one after another anyway, so a short unroll
-                // keeps the code in the instruction cache (4 measured 10.07 against 9.10 ms
-                // on the 8M-node graph)
-                constexpr int U = 2;
-                for (int32_t p0 = 0; p0 < P; p0 += 32 * U) {
-                    int32_t lo_e[U], hi_e[U];
-                    int64_t pos[U];
-#pragma unroll
-                    for (int q = 0; q < U; ++q) {
-                        int32_t pv = p0 + q * 32 + lane;
-                        lo_e[q] = -1;
-                        hi_e[q] = 0;
-                        if (pv < P) {
-                            int32_t lo = 0, hi = Ew;        // last entry with ppre[e] <= pv
-                            while (hi - lo > 1) {
-                                int32_t mid = (lo + hi) >> 1;
-                                if (S.ppre[mid] <= pv) lo = mid; else hi = mid;
-                            }
-                            int32_t f = lo + 1 + (pv - S.ppre[lo]);
-                            bool e_low = rank_less(S.bdx[lo], S.nb[lo], S.bdx[f], S.nb[f]);
-                            lo_e[q] = e_low ? lo : f;
-                            hi_e[q] = e_low ? f : lo;
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < U; ++q)
-                        pos[q] = lo_e[q] >= 0 ? find_in_list_sk(xcol, xsk, S.boff[lo_e[q]], S.bdeg[lo_e[q]], S.nb[hi_e[q]])
-                                          : -1;
-#pragma unroll
-                    for (int q = 0; q < U; ++q) {
-                        bool hit = pos[q] >= 0;
-                        unsigned hm = __ballot_sync(FULL, hit);
-                        if (hit) {
-                            int slot = qn + __popc(hm & lanemask_lt());
-                            S.qpos[slot] = pos[q];
-                            S.qow[slot] = S.owner[lo_e[q]];
-                            S.qlo[slot] = (uint8_t)lo_e[q];
-                            S.qhi[slot] = (uint8_t)hi_e[q];
-                        }
-                        qn += __popc(hm);
-                        if (qn >= 32) {                        // a full warp of triangles
-                            __syncwarp();
-                            p3_flush<kScr>(S, anode, 32, base, xS, R, acc, lane);
-                            __syncwarp();
-                            if (lane < qn - 32) {
-                                S.qpos[lane] = S.qpos[32 + lane];
-                                S.qow[lane] = S.qow[32 + lane];
-                                S.qlo[lane] = S.qlo[32 + lane];
-                                S.qhi[lane] = S.qhi[32 + lane];
-                            }
-                            qn -= 32;
-                            __syncwarp();
-                        }
-                    }
-                }
-                __syncwarp();
-                p3_flush<kScr>(S, anode, qn, base, xS, R, acc, lane);   // the window's stage is reused next
-                qn = 0;
-                __syncwarp();
-            }
-            start = end;
-        }
-        // heavy nodes' tasks go to the list (its capacity bounds their number, so the
-        // error branch is not taken)
-        if (da > kWinCap) {
-            const int32_t nt = (da + kHvBlock - 1) / kHvBlock;
-            const unsigned long long h = atomicAdd(hv_count, (unsigned long long)nt);
-            if (h + nt <= (unsigned long long)hvcap) {
-                for (int32_t i = 0; i < nt; ++i) hvl[h + i] = (unsigned long long)av << 32 | (unsigned)i;
-            } else {
-                atomicOr(R.err, 64);
-            }
-        }
+    if (any) {
+        acc_a = u192_add(acc_a, scale(B.ab.r, sum_a));
+        sum_b = warp_sum_u96(sum_b);
+        if (lane == 0) atomic_add_u192(acc + 3 * (int64_t)B.b, scale(B.ab.f, sum_b));
     }
 }
 
@@ -1910,20 +2024,20 @@ __global__ void __launch_bounds__(kThreads, 5) p3_list_kernel(
 // counter; the CTA's warps claim the task's out-neighbours b from a counter in shared
 // memory (dynamic shared memory: sizeof(P3Heavy))
 __global__ void __launch_bounds__(kThreads, 3) p3_heavy_kernel(
-    int64_t n, const int64_t *__restrict__ xoff, const int32_t *__restrict__ xcol, const df *__restrict__ xS,
-    Rev R, const int32_t *__restrict__ xout, unsigned long long *acc, const unsigned long long *__restrict__ hvl,
-    int64_t hvcap, const unsigned long long *hv_count, unsigned long long *hv_next) {
+    int64_t n, const int64_t *__restrict__ xoff, const int32_t *__restrict__ xcol, Rev R,
+    const int32_t *__restrict__ xout, const GxNode *__restrict__ xnode, unsigned long long *acc,
+    const unsigned long long *__restrict__ hvl, int64_t hvcap, const unsigned long long *hv_count,
+    unsigned long long *hv_next) {
     extern __shared__ __align__(16) unsigned char hv_smem[];
     P3Heavy &H = *reinterpret_cast<P3Heavy *>(hv_smem);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tid = threadIdx.x;
-    HvQueue &Q = H.q[wid];
+    uint32_t *Q = H.q[wid];
     unsigned long long lim = *hv_count;
     if (lim > (unsigned long long)hvcap) lim = (unsigned long long)hvcap;
     if (lim == 0) return;
-    for (int i = tid; i < kHvIds; i += kThreads) {
-        H.clo[i] = 0;
-        H.chi[i] = 0;
-    }
+    for (int i = tid; i < kHvIds; i += kThreads)
+#pragma unroll
+        for (int j = 0; j < kLimbs; ++j) H.sum[j][i] = 0;
     while (true) {
         __syncthreads();                               // the previous task is flushed
         if (tid == 0) {
@@ -1949,35 +2063,31 @@ __global__ void __launch_bounds__(kThreads, 3) p3_heavy_kernel(
         if (H.a < 0) continue;
         const int32_t a = (int32_t)H.a, dA = H.dA, eb0 = H.eb0, nb = H.nb;
         const int64_t bA = H.bA;
-        u128 acc_a = 0;
+        u192 acc_a{0, 0, 0};
         for (int32_t k0 = 0; k0 < dA; k0 += kHvIds) {
             const int32_t cnt = min(kHvIds, dA - k0);
-            const uint32_t buckets = max(32u, dev_pow2_at_least((uint32_t)cnt)), mask = buckets - 1;
-            for (uint32_t i = tid; i < buckets; i += kThreads) H.key[i] = make_int4(-1, -1, -1, -1);
+            const int32_t *A = xcol + bA + k0;
+            for (int i = tid; i < kHvSlots / 4; i += kThreads) reinterpret_cast<uint4 *>(H.tab)[i] = make_uint4(0, 0, 0, 0);
             if (tid == 0) H.next_b = 0;
             __syncthreads();
             for (int32_t i = tid; i < cnt; i += kThreads) {
-                const int64_t sl = bA + k0 + i;
-                const int32_t c = xcol[sl];
-                // the first free slot of the first bucket with one, from the home bucket on
-                // (the ids are distinct and at most a quarter of the slots are used, so one
-                // is found); slots fill in order, so a bucket with an empty last slot has
-                // room and holds every key that hashes to it
-                int32_t *keys = reinterpret_cast<int32_t *>(H.key);
-                uint32_t bk = hv_hash(c, mask), slot = 4u * kHvSlots;
-                for (uint32_t it = 0; it <= mask && slot >= 4u * kHvSlots; ++it) {
-                    for (int j = 0; j < 4; ++j)
-                        if (atomicCAS(&keys[4 * bk + j], -1, c) == -1) { slot = 4 * bk + j; break; }
-                    bk = (bk + 1) & mask;
+                const int32_t c = A[i];
+                const uint32_t h = hv_hash(c), home = h >> kHvRest;
+                const uint32_t word = kHvTaken | (uint32_t)i << kHvRest | (h & kHvRestMask);
+                // home, or the next free slot after it (an eighth of the slots at most are used)
+                if ((atomicCAS(&H.tab[home], 0u, word)) != 0) {
+                    atomicOr(&H.tab[home], kHvMore);
+                    uint32_t s = home;
+                    int it = 0;
+                    do s = (s + 1) & (kHvSlots - 1);
+                    while (atomicCAS(&H.tab[s], 0u, word | kHvMoved) != 0 && ++it < kHvSlots);
+                    if (it >= kHvSlots) atomicOr(R.err, 64);
                 }
-                if (slot < 4u * kHvSlots) H.slot_pos[slot] = (uint16_t)i;
-                else atomicOr(R.err, 64);
-                const df sac = xS[sl], sca = R.get(sl, c, a);
-                H.sca[i] = sca;
-                H.pac[i] = df_add(sac, sca);
+                const SigPair v = R.get(bA + k0 + i, c, a);
+                H.sp[i] = SigPair{v.r, v.f + v.r};
             }
             __syncthreads();
-            const int32_t lo_id = xcol[bA + k0], hi_id = xcol[bA + k0 + cnt - 1];
+            const int32_t lo_id = A[0], hi_id = A[cnt - 1];
             const bool cut = dA > kHvIds;
             // the warp claims out-neighbours one at a time; the next one's data is loaded
             // while the current one is walked
@@ -1988,29 +2098,31 @@ __global__ void __launch_bounds__(kThreads, 3) p3_heavy_kernel(
             };
             int32_t j = claim();
             HvB cur{};
-            if (j < nb) cur = hv_load_b(a, bA + eb0 + j, cut, lo_id, hi_id, xoff, xcol, xS, R, xout);
+            if (j < nb) cur = hv_load_b(a, bA + eb0 + j, cut, lo_id, hi_id, xcol, R, xnode);
             while (j < nb) {
                 const int32_t jn = claim();
                 HvB nxt{};
-                if (jn < nb) nxt = hv_load_b(a, bA + eb0 + jn, cut, lo_id, hi_id, xoff, xcol, xS, R, xout);
-                hv_walk_b(H, Q, cur, bA + k0, mask, xcol, xS, R, acc, lane, acc_a);
+                if (jn < nb) nxt = hv_load_b(a, bA + eb0 + jn, cut, lo_id, hi_id, xcol, R, xnode);
+                hv_walk_b(H, Q, cur, A, xcol, R, acc, lane, acc_a);
                 j = jn;
                 cur = nxt;
             }
             __syncthreads();
             // c's sums of the chunk to the accumulators, zeroed for the next chunk
             for (int32_t i = tid; i < cnt; i += kThreads) {
-                const unsigned long long lo = H.clo[i], hi = H.chi[i];
-                if (lo | hi) {
-                    atomic_add_u128(acc + 2 * (int64_t)xcol[bA + k0 + i], ((u128)hi << 48) + lo);
-                    H.clo[i] = 0;
-                    H.chi[i] = 0;
+                const u96 t = from_limbs(H.sum[0][i], H.sum[1][i], H.sum[2][i], H.sum[3][i]);
+                if (t.lo | t.hi) {
+                    atomic_add_u192(acc + 3 * (int64_t)A[i], scale(H.sp[i].r - H.sp[i].f, t));
+#pragma unroll
+                    for (int l = 0; l < kLimbs; ++l) H.sum[l][i] = 0;
                 }
             }
             __syncthreads();
         }
-        acc_a = warp_sum_u128(acc_a);
-        if (lane == 0 && acc_a) atomic_add_u128(acc + 2 * (int64_t)a, acc_a);
+        for (int m = 16; m; m >>= 1)
+            acc_a = u192_add(acc_a, u192{__shfl_xor_sync(FULL, acc_a.w0, m), __shfl_xor_sync(FULL, acc_a.w1, m),
+                                         __shfl_xor_sync(FULL, acc_a.w2, m)});
+        if (lane == 0 && (acc_a.w0 | acc_a.w1 | acc_a.w2)) atomic_add_u192(acc + 3 * (int64_t)a, acc_a);
     }
 }
 
@@ -2152,53 +2264,6 @@ __global__ void __launch_bounds__(kThreads) strict_pairs_kernel(
 }
 
 // ======================================================================================
-// P2 row lists by cross degree (known after P1): each P2 kernel then walks only its rows
-//   0 mid and large rows, dx <= 32 (tiles)   1 mid rows, 32 < dx <= 128 (p2_mid, 256 slots)
-//   2 unused                                 3 large rows, 32 < dx <= min(128, dx_cta) (p2_mid, 256)
-//   4 large rows, dx > dx_cta (p2_large)     5 mid rows, dx > 128 (p2_mid, 512 slots)
-//   6 large rows, 128 < dx <= dx_cta (p2_mid, 512 slots)
-// ======================================================================================
-constexpr int kP2Lists = 7;
-constexpr int32_t kSmallTableDx = 128;        // rows up to this cross degree fit 256-slot tables
-
-__device__ __forceinline__ void append_row(int32_t *list, int32_t *cnt, bool take, int32_t v) {
-    unsigned m = __ballot_sync(FULL, take);
-    int lane = threadIdx.x & 31;
-    int32_t base = 0;
-    if (m && lane == __ffs(m) - 1) base = atomicAdd(cnt, __popc(m));
-    base = __shfl_sync(FULL, base, __ffs(m ? m : 1u) - 1);
-    if (take) list[base + __popc(m & lanemask_lt())] = v;
-}
-
-// list 0 has room for n_mid + n_large rows, the other mid lists for n_mid, the large ones for n_large
-__host__ __device__ __forceinline__ int64_t p2_list_start(int c, int64_t n_mid, int64_t n_large) {
-    const int mids_before[kP2Lists] = {0, 1, 2, 2, 2, 2, 3};
-    const int larges_before[kP2Lists] = {0, 1, 1, 1, 2, 3, 3};
-    return mids_before[c] * n_mid + larges_before[c] * n_large;
-}
-
-__global__ void p2_split_kernel(const int32_t *__restrict__ rows_mid, int64_t n_mid,
-                                const int32_t *__restrict__ rows_large, int64_t n_large,
-                                const NodeRec *__restrict__ rec, int32_t dx_cta, int32_t *lists, int32_t *cnt) {
-    int64_t total = n_mid + n_large;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < total; i0 += (int64_t)gridDim.x * blockDim.x) {
-        int64_t i = i0 + threadIdx.x;
-        bool act = i < total;
-        bool mid = i < n_mid;
-        int32_t v = act ? (mid ? rows_mid[i] : rows_large[i - n_mid]) : 0;
-        int32_t dx = act ? rec[v].dx : 0;
-        int cls = -1;
-        if (act) {
-            if (dx <= 32) cls = 0;                              // the tile kernel, either class
-            else if (mid) cls = dx <= kSmallTableDx ? 1 : 5;
-            else cls = dx > dx_cta ? 4 : dx <= kSmallTableDx ? 3 : 6;
-        }
-        for (int c = 0; c < kP2Lists; ++c)
-            append_row(lists + p2_list_start(c, n_mid, n_large), cnt + c, cls == c, v);
-    }
-}
-
-// ======================================================================================
 // finalize: R(u) = acc(u) / (w_max d (d - 1))
 // ======================================================================================
 __global__ void graph_scale_kernel(const unsigned long long *__restrict__ wmax_bits, int32_t ng, double *winv) {
@@ -2228,10 +2293,31 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(
         double r = 0.0;
         if (d >= 2) {
             double W = gid ? winv[gid[u]] : sh_w;
-            u128 s = ((u128)acc[2 * u + 1] << 64) | acc[2 * u];
-            if (s && W > 0.0) r = u128_to_double(s, -kAccFrac) * W * RD[d];
+            const u192 s{acc[3 * u], acc[3 * u + 1], acc[3 * u + 2]};
+            if ((s.w0 | s.w1 | s.w2) && W > 0.0) r = u192_to_double(s) * W * RD[d];
         }
         scores[perm ? (int64_t)perm[u] : u] = r;
+    }
+}
+
+// everything a scoring pass starts from, set by one launch (a memset each took about 2 us
+// of the chain: 13 us of a 97 us step on 2,000 nodes)
+struct InitRange {
+    unsigned long long *p;
+    int64_t words;
+    unsigned long long fill;
+};
+struct InitArgs {
+    InitRange r[10];
+    int n;
+};
+__global__ void __launch_bounds__(kThreads) init_kernel(InitArgs A) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int j = 0; j < A.n; ++j) {
+        const InitRange &r = A.r[j];
+        ulonglong2 *p2 = reinterpret_cast<ulonglong2 *>(r.p);
+        for (int64_t i = t0; i < r.words / 2; i += step) p2[i] = make_ulonglong2(r.fill, r.fill);
+        if (t0 == 0 && (r.words & 1)) r.p[r.words - 1] = r.fill;
     }
 }
 
@@ -2244,14 +2330,13 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(
 int rs::prepare_score_kernels() {
     static int done = 0;
     if (done) return 0;
-    const int p2_mid_smem = kMidWarps * kWarpCap * kMidSlotBytes;
     RS_CUDA_TRY(cudaFuncSetAttribute(p1_large_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kMidCap));
     RS_CUDA_TRY(cudaFuncSetAttribute(p1_large_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kMidCap));
     RS_CUDA_TRY(cudaFuncSetAttribute(p1_large_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kMidCap));
     RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
     RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
     RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
-    RS_CUDA_TRY(cudaFuncSetAttribute(p2_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, p2_mid_smem));
+    RS_CUDA_TRY(cudaFuncSetAttribute(p2_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2MidSmem));
     RS_CUDA_TRY(cudaFuncSetAttribute(p3_heavy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sizeof(P3Heavy)));
     RS_CUDA_TRY(cudaFuncSetAttribute(p1_small_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2267,12 +2352,14 @@ static void launch_p1_large(rs_graph *g, const Batch &B, int *err, size_t smem, 
         g->off, g->col, g->lab, g->rows_large, g->n_large, B, g->LG, g->rec, g->Lall, err,
         g->rsum, g->cl_col, g->cl_lab, g->wq + 1);
 }
+// p2_large over P2 list `list`, at most per_sm CTAs per SM
 template <int NT>
-static void launch_p2_large(rs_graph *g, const Batch &B, int *err, size_t smem, cudaStream_t st) {
-    int32_t *L4 = g->p2rows + p2_list_start(4, g->n_mid, g->n_large);
-    p2_large_kernel<NT><<<grid_for(g->n_large, 1, 2), NT, smem, st>>>(
-        g->off, L4, g->p2cnt + 4, B, g->tune.p2_cta_dx + 1, g->LG, g->rec, g->rsum, g->cl_col,
-        g->cl_lab, g->acc, g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, err, Strict{g->col, g->sx}, g->wq + 6);
+static void launch_p2_large(rs_graph *g, const Batch &B, int *err, size_t smem, int list, int per_sm,
+                            unsigned long long *wq, cudaStream_t st) {
+    p2_large_kernel<NT><<<grid_for(list == 3 ? g->n_large : g->n_mid + g->n_large, 1, per_sm), NT, smem, st>>>(
+        g->off, g->p2rows + p2_list_start(list, g->n_mid, g->n_large), g->p2cnt + list, B, g->LG, g->rec, g->rsum,
+        g->cl_col, g->cl_lab, g->acc, g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, err,
+        Strict{g->col, g->sx}, wq);
 }
 
 // a stride near n / golden ratio, coprime to n (a bijection of [0, n) by multiplication)
@@ -2293,19 +2380,28 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     const int cps = g->tune.ctas_per_sm;
     if (int rc = prepare_score_kernels()) return rc;
     prof_begin(g, s);
-    RS_CUDA_TRY(cudaMemsetAsync(g->wmax_bits, 0, g->n_graphs * sizeof(unsigned long long), s));
     Batch B{g->gid, g->gk, g->k, g->wmax_bits};
-    RS_CUDA_TRY(cudaMemsetAsync(g->acc, 0, 2 * n * sizeof(unsigned long long), s));
-    RS_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
-    // row counters and the G_x scan's ticket and tile words
-    RS_CUDA_TRY(cudaMemsetAsync(g->wq, 0, wq_hv_word(n) * sizeof(unsigned long long), s));
+    InitArgs I{};
+    int64_t init_words = 0;
+    auto init = [&](void *p, int64_t words, unsigned long long fill) {
+        I.r[I.n++] = InitRange{(unsigned long long *)p, words, fill};
+        init_words += words;
+    };
+    init(g->wmax_bits, g->n_graphs, 0);
+    init(g->acc, 3 * n, 0);
+    init(err, 1, 0);                                 // (and the unused flag word after it)
+    init(g->wq, wq_hv_word(n), 0);                   // row counters and the G_x scan's ticket and tile words
+    init(g->p2cnt, 8, 0);                            // P2 list counts; word 8: the last node with slots
     if (g->n_hubs) {
-        RS_CUDA_TRY(cudaMemsetAsync(g->hkey, 0xFF, g->hub_slots * sizeof(int32_t), s));
-        RS_CUDA_TRY(cudaMemsetAsync(g->hcnt, 0, g->hub_slots * sizeof(uint32_t), s));
-        RS_CUDA_TRY(cudaMemsetAsync(g->hq, 0, 2 * g->hub_slots * sizeof(unsigned long long), s));
-        RS_CUDA_TRY(cudaMemsetAsync(g->hagg, 0, g->n_hubs * sizeof(HubAgg), s));
+        init(g->hkey, g->hub_slots / 2, ~0ull);      // tables are powers of two of at least 2 slots
+        init(g->hcnt, g->hub_slots / 2, 0);
+        init(g->hq, 2 * g->hub_slots, 0);
+        init(g->hagg, g->n_hubs * (int64_t)(sizeof(HubAgg) / sizeof(unsigned long long)), 0);
     }
-    prof_mark(g, s, "memset", false);
+    if (g->strict) init(g->sx, 2 * g->nnz, 0);
+    static_assert(sizeof(HubAgg) % sizeof(unsigned long long) == 0, "HubAgg is cleared by words");
+    init_kernel<<<grid_for(init_words / 2 + 1, NT, 8), NT, 0, s>>>(I);
+    RS_LAUNCHED(g, s, "init");
     size_t p1_smem = 8 * (size_t)g->large_cap, p2_smem = 32 * (size_t)g->large_cap;
     // streams of the row kernels (rows_streams): every class on its own stream (0); the hub
     // chain on stream 3 and every other class in turn on stream 0 (1); every kernel in turn
@@ -2319,16 +2415,27 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     constexpr int64_t kRowsTwoStreamNnz = 32000000;
     const int rmode = g->tune.rows_streams >= 0 ? g->tune.rows_streams
                                                 : (g->n_hubs && g->nnz >= kRowsTwoStreamNnz ? 1 : 0);
-    auto AX = [&](int i) -> cudaStream_t {
-        if (rmode == 2) return s;
-        if (rmode == 1) return i == 3 ? g->aux[3] : g->aux[0];
-        return g->aux[i];
+    // (a phase with one class of rows takes the step's stream, and only the streams in use are
+    // forked and joined)
+    const bool mid_large = g->n_mid + g->n_large > 0;
+    unsigned used = 0;
+    auto plan = [&](std::initializer_list<std::pair<int, bool>> classes) {
+        used = 0;
+        int k = 0;
+        if (rmode != 2)
+            for (auto &c : classes)
+                if (c.second) { used |= 1u << (rmode == 1 ? (c.first == 3 ? 3 : 0) : c.first); ++k; }
+        if (k < 2) used = 0;
     };
+    auto AX = [&](int i) -> cudaStream_t {
+        const int j = rmode == 1 ? (i == 3 ? 3 : 0) : i;
+        return used >> j & 1 ? g->aux[j] : s;
+    };
+    plan({{3, g->n_hubs > 0}, {2, g->n_large > 0}, {4, g->n_mid > 0}, {0, g->n_small > 0}});
     // ---- P1: the larger classes are launched first (with per-class streams, on
     //      high-priority ones), so their maxima seed w_max early and most small rows skip
     //      theirs (the small rows fill in at the lowest priority)
-    if (rmode != 2)
-        if (int rc = fork_aux(g, s)) return rc;
+    if (int rc = fork_aux(g, s, used)) return rc;
     if (g->n_hubs) {
         hub_p1_insert_kernel<NT><<<grid_for(g->n_hub_items, 1, 8), NT, 0, AX(3)>>>(
             g->off, g->col, g->lab, g->hubs, g->hub_items, g->hub_item_chunk, g->n_hub_items,
@@ -2371,25 +2478,22 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
                 g->rsum, g->cl_col, g->cl_lab);
         RS_LAUNCHED(g, AX(0), "p1_small");
     }
-    if (rmode != 2)
-        if (int rc = join_aux(g, s, rs_graph::kAux)) return rc;
-    // ---- P2 row lists (on stream 5) beside the G_x offsets (on the step's stream)
+    if (int rc = join_aux(g, s, used)) return rc;
+    // ---- the G_x offsets (and the mirror's tiles) and the P2 row lists, in one launch
     const int64_t nm = g->n_mid, nl = g->n_large;
     auto Lst = [&](int c) { return g->p2rows + p2_list_start(c, nm, nl); };
-    if (nm + nl) {
-        RS_CUDA_TRY(cudaMemsetAsync(g->p2cnt, 0, kP2Lists * sizeof(int32_t), s));
-        p2_split_kernel<<<grid_for(nm + nl, 256, 8), 256, 0, s>>>(g->rows_mid, nm, g->rows_large, nl, g->rec,
-                                                                   g->tune.p2_cta_dx, g->p2rows, g->p2cnt);
-        RS_LAUNCHED(g, s, "p2_split");
-    }
+    int32_t *last_node = g->p2cnt + 8;
+    if (g->tune.p3_mirror && !g->xtile)
+        return fail(RS_EINVAL, "rs_score: p3_mirror is set but its tile table is missing");
     const int64_t gx_tiles = (n + kGxTile - 1) / kGxTile;
-    gx_offsets_kernel<<<(unsigned)gx_tiles, kGxThreads, 0, s>>>(g->rec, n, g->xoff, g->wq + kWqGxStatus,
-                                                              g->wq + kWqGxTicket, err, g->gx_spin,
-                                                              g->gx_withhold);
+    const int split_blocks = mid_large ? grid_for(nm + nl, kGxThreads, 8) : 0;
+    gx_offsets_kernel<<<(unsigned)(split_blocks + gx_tiles), kGxThreads, 0, s>>>(
+        g->rec, n, g->xoff, g->wq + kWqGxStatus, g->wq + kWqGxTicket, err, g->gx_spin, g->gx_withhold,
+        g->tune.p3_mirror ? g->xtile : nullptr, last_node,
+        P2Split{g->rows_mid, g->rows_large, nm, nl, g->tune.p2_cta_dx, g->p2rows, g->p2cnt}, split_blocks);
     RS_LAUNCHED(g, s, "gx_offsets");
     const Strict SX{g->col, g->strict ? g->sx : nullptr};
     if (g->strict) {
-        RS_CUDA_TRY(cudaMemsetAsync(g->sx, 0, 2 * g->nnz * sizeof(unsigned long long), s));
         strict_pairs_kernel<<<grid_for(g->nnz, NT, cps), NT, 0, s>>>(n, g->off, g->col, g->lab, g->rec, g->cl_col, B,
                                                                      g->tune.small_max, g->tune.cta_cap, g->sx);
         RS_LAUNCHED(g, s, "strict_pairs");
@@ -2398,8 +2502,8 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     //      streams 0 and 1, the rows with long chains on the others.  The hub
     //      chain (three dependent kernels, the longest of the phase on hub-skewed graphs)
     //      is issued first, so that its blocks are dispatched ahead of the other classes'
-    if (rmode != 2)
-        if (int rc = fork_aux(g, s)) return rc;
+    plan({{3, g->n_hubs > 0}, {0, g->n_small > 0}, {1, mid_large}, {5, mid_large}, {2, mid_large}, {4, g->n_large > 0}});
+    if (int rc = fork_aux(g, s, used)) return rc;
     if (g->n_hubs) {
         hub_p2_insert_kernel<NT><<<grid_for(g->n_hub_items, 1, 8), NT, 0, AX(3)>>>(
             g->off, g->col, g->hubs, g->hub_items, g->hub_item_chunk, g->n_hub_items, g->tune.hub_chunk, g->rec,
@@ -2407,7 +2511,7 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
             g->hitem_out, g->hitem_in, g->hslot, err);
         RS_LAUNCHED(g, AX(3), "hub_p2_insert");
         hub_p2_counts_kernel<NT><<<(unsigned)((g->n_hubs + NT - 1) / NT), NT, 0, AX(3)>>>(
-            g->hubs, g->n_hubs, g->hitem_out, g->hitem_in, g->xout, g->xin);
+            g->hubs, g->n_hubs, g->hitem_out, g->hitem_in, g->xoff, g->rec, g->xout, g->xin, g->xnode);
         RS_LAUNCHED(g, AX(3), "hub_p2_counts");
         hub_p2_emit_kernel<NT><<<grid_for(g->n_hub_items, 1, 8), NT, 0, AX(3)>>>(
             g->off, g->col, g->hubs, g->hub_items, g->hub_item_chunk, g->n_hub_items, g->tune.hub_chunk, g->rec,
@@ -2418,77 +2522,58 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     if (g->n_small) {
         p2_small_kernel<32><<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
             g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
-            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, SX);
+            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX);
         RS_LAUNCHED(g, AX(0), "p2_small");
     }
-    if (g->tune.p3_mirror) {                         // the mirror's tile table, beside P2
-        if (!g->xR || !g->xtile) return fail(RS_EINVAL, "rs_score: p3_mirror is set but its buffers are missing");
-        mirror_tiles_kernel<<<grid_for(n, NT, cps), NT, 0, AX(0)>>>(n, g->xoff, g->xtile);
-        RS_LAUNCHED(g, AX(0), "mirror_tiles");
-    }
-    const size_t smem256 = (size_t)kMidWarps * 256 * kMidSlotBytes, smem512 = (size_t)kMidWarps * 512 * kMidSlotBytes;
-    if (nm + nl) {
+    if (mid_large) {
         // the mid and large rows with at most 32 cross neighbours, in the tile kernel
         p2_small_kernel<kNarrowRows><<<grid_for((nm + nl) * (32 / kNarrowRows), NT, cps), NT, 0, AX(1)>>>(
             g->off, Lst(0), 0, g->p2cnt + 0, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc, g->xoff,
-            g->xcol, g->xS, g->xsk, g->xout, g->xin, SX);
+            g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX);
         RS_LAUNCHED(g, AX(1), "p2_narrow");
-    }
-    if (g->n_mid) {
-        p2_mid_kernel<<<grid_for(g->n_mid * 32, NT, 4), NT, smem256, AX(5)>>>(
-            g->off, Lst(1), g->p2cnt + 1, B, 1 << 30, 256, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
-            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, err, SX, g->wq + 2);
+        p2_mid_kernel<<<grid_for((nm + nl) * 32, NT, 4), NT, kP2MidSmem, AX(5)>>>(
+            g->off, Lst(1), g->p2cnt + 1, B, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc, g->xoff, g->xcol,
+            g->xS, g->xsk, g->xout, g->xin, g->xnode, err, SX, g->wq + 2);
         RS_LAUNCHED(g, AX(5), "p2_mid");
-        // few rows, each a long single-warp chain: on the lightly loaded stream
-        p2_mid_kernel<<<grid_for(g->n_mid * 32, NT, 2), NT, smem512, AX(2)>>>(
-            g->off, Lst(5), g->p2cnt + 5, B, 1 << 30, 512, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
-            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, err, SX, g->wq + 3);
-        RS_LAUNCHED(g, AX(2), "p2_mid_wide");
+        launch_p2_large<kP2SmallCta>(g, B, err, 32 * (size_t)kWarpCap, 2, 8, g->wq + 3, AX(2));
+        RS_LAUNCHED(g, AX(2), "p2_cta");
     }
     if (g->n_large) {
-        // large rows whose cross list fits a per-warp table go warp-per-row too
-        p2_mid_kernel<<<grid_for(g->n_large * 32, NT, 4), NT, smem256, AX(2)>>>(
-            g->off, Lst(3), g->p2cnt + 3, B, g->tune.p2_cta_dx, 256, g->LG, g->rec, g->rsum, g->cl_col,
-            g->cl_lab, g->acc, g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, err, SX, g->wq + 4);
-        RS_LAUNCHED(g, AX(2), "p2_large_warp");
-        // (with hubs, stream 3 carries the hub chain: these rows go beside p2_mid instead)
-        cudaStream_t sw = g->n_hubs || rmode == 1 ? AX(5) : AX(3);
-        p2_mid_kernel<<<grid_for(g->n_large * 32, NT, 2), NT, smem512, sw>>>(
-            g->off, Lst(6), g->p2cnt + 6, B, g->tune.p2_cta_dx, 512, g->LG, g->rec, g->rsum, g->cl_col,
-            g->cl_lab, g->acc, g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, err, SX, g->wq + 5);
-        RS_LAUNCHED(g, sw, "p2_large_warp_wide");
         switch (g->tune.p2_cta_threads) {
-        case 256: launch_p2_large<256>(g, B, err, p2_smem, AX(4)); break;
-        case 512: launch_p2_large<512>(g, B, err, p2_smem, AX(4)); break;
-        default: launch_p2_large<1024>(g, B, err, p2_smem, AX(4)); break;
+        case 256: launch_p2_large<256>(g, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
+        case 512: launch_p2_large<512>(g, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
+        default: launch_p2_large<1024>(g, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
         }
         RS_LAUNCHED(g, AX(4), "p2_large");
     }
-    if (rmode != 2)
-        if (int rc = join_aux(g, s, rs_graph::kAux)) return rc;
+    if (int rc = join_aux(g, s, used)) return rc;
     // ---- P3: reverse values (mirror mode), then triangles
     if (g->tune.p3_mirror) {
-        gx_mirror_kernel<<<grid_for(g->nnz, kMirTile, cps), NT, 0, s>>>(n, g->xoff, g->xcol, g->xS, g->xout,
-                                                                       g->xin, g->xtile, g->xR, g->xsk, err);
+        gx_mirror_kernel<<<grid_for(g->nnz, kMirTile, cps), NT, 0, s>>>(n, g->xoff, g->xcol, g->xS, g->xnode,
+                                                                       g->xin, g->xtile, last_node, g->xsk, err);
         RS_LAUNCHED(g, s, "gx_mirror");
     }
-    const Rev R{g->tune.p3_mirror ? g->xR : nullptr, g->xoff, g->xcol, g->xS, g->xin, err};
+    const Rev R{g->xS, g->xoff, g->xcol, g->xin, err, g->tune.p3_mirror != 0};
     unsigned long long *next_group = g->wq + 7;
     unsigned long long *hvl = g->wq + wq_hv_word(n);
     const int64_t hvcap = hv_cap(g->nnz);
+    // nodes per group: 32, or fewer on graphs with too few groups of 32 to go around
+    int32_t group = 32;
+    while (group > 4 && n / group < 16 * (int64_t)grid_for(INT64_MAX / 2, 1, 1)) group >>= 1;
+    const int list_grid = grid_for(n, group, kP3CtasPerSm);
     if (g->perm)                                     // a graph numbered by community: scrambled groups
-        p3_list_kernel<true><<<grid_for(n, NT, cps), NT, 0, s>>>(n, g->xoff, g->xcol, g->xsk, g->xS, R, g->xout,
-                                                                  g->rec, g->acc, next_group, p3_stride(n), hvl,
-                                                                  hvcap, g->wq + kWqHvCount);
+        p3_list_kernel<true><<<list_grid, kP3Threads, 0, s>>>(n, g->xoff, g->xcol, g->xsk, R, g->xout, g->xnode, g->acc,
+                                                              next_group, group, p3_stride(n), hvl, hvcap,
+                                                              g->wq + kWqHvCount);
     else
-        p3_list_kernel<false><<<grid_for(n, NT, cps), NT, 0, s>>>(n, g->xoff, g->xcol, g->xsk, g->xS, R, g->xout,
-                                                                   g->rec, g->acc, next_group, 1, hvl, hvcap,
-                                                                   g->wq + kWqHvCount);
+        p3_list_kernel<false><<<list_grid, kP3Threads, 0, s>>>(n, g->xoff, g->xcol, g->xsk, R, g->xout, g->xnode, g->acc,
+                                                               next_group, group, 1, hvl, hvcap, g->wq + kWqHvCount);
     RS_LAUNCHED(g, s, "p3_list");
-    p3_heavy_kernel<<<grid_for(hvcap, 1, 3), NT, sizeof(P3Heavy), s>>>(n, g->xoff, g->xcol, g->xS, R, g->xout,
-                                                                       g->acc, hvl, hvcap, g->wq + kWqHvCount,
-                                                                       g->wq + kWqHvNext);
-    RS_LAUNCHED(g, s, "p3_heavy");
+    if (g->dmax > kWinCap) {                         // else no node has that many out-neighbours
+        p3_heavy_kernel<<<grid_for(hvcap, 1, 3), NT, sizeof(P3Heavy), s>>>(
+            n, g->xoff, g->xcol, R, g->xout, g->xnode, g->acc, hvl, hvcap, g->wq + kWqHvCount, g->wq + kWqHvNext);
+        RS_LAUNCHED(g, s, "p3_heavy");
+    }
     // ---- finalize
     if (g->gid) {
         graph_scale_kernel<<<(g->n_graphs + 255) / 256, 256, 0, s>>>(g->wmax_bits, g->n_graphs, g->winv);

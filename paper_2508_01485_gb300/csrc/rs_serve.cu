@@ -72,7 +72,7 @@ struct BaseView {
     const int32_t *cl_col, *cl_lab;
     const int64_t *xoff;
     const int32_t *xcol;
-    const df *xS;
+    const SigPair *xS;
     const int32_t *xout, *xin;
     const uint64_t *LG;
     const double *RD;
@@ -501,22 +501,22 @@ __device__ __forceinline__ int64_t gx_slot(const BaseView &B, int32_t p, int32_t
     return (l < B.xin[p] && B.xcol[end - l] == q) ? end - l : -1;
 }
 
-__device__ __forceinline__ df s_base(const BaseView &B, const SlotView &S, int32_t p, int32_t q) {
+__device__ __forceinline__ uint64_t s_base(const BaseView &B, const SlotView &S, int32_t p, int32_t q) {
     int64_t sl = gx_slot(B, p, q);
-    if (sl < 0) { atomicOr(S.err, 32); return df{0.0f, 0.0f}; }
-    return B.xS[sl];
+    if (sl < 0) { atomicOr(S.err, 32); return 0; }
+    return B.xS[sl].f;
 }
 
 // S'(p -> q) after the removals
-__device__ __forceinline__ df s_after(const BaseView &B, const SlotView &S, int32_t p, int32_t q) {
+__device__ __forceinline__ uint64_t s_after(const BaseView &B, const SlotView &S, int32_t p, int32_t q) {
     if (!(S.flag[p] & kInT)) return s_base(B, S, p, q);
     TRow r = S.trow[S.tidx[p]];
-    if (r.cap == 0) return df{0.0f, 0.0f};
+    if (r.cap == 0) return 0;
     Tab t{S.tkey + r.tab, S.tcnt + r.tab, nullptr, nullptr, r.cap - 1};
     int sl = tab_find(t, B.lab[q]);
     uint32_t f = sl >= 0 ? t.cnt[sl] : 0u;
     RowAgg a{r.T, r.L, ((u128)r.xhi << 64) | r.xlo};
-    return df_cbrt(column_weight(a, f, B.LG));
+    return sig_fixed(df_cbrt(column_weight(a, f, B.LG)));
 }
 
 __device__ __forceinline__ int32_t dx_after(const BaseView &B, const SlotView &S, int32_t p) {
@@ -649,8 +649,8 @@ __global__ void __launch_bounds__(kSvThreads) sv_finalize(BaseView B, SlotView S
         int64_t d = (S.flag[u] & kInT) ? (int64_t)S.trow[S.tidx[u]].T : B.off[u + 1] - B.off[u];
         double r = 0.0;
         if (d >= 2) {
-            u128 s = ((u128)S.acc[2 * u + 1] << 64) | S.acc[2 * u];
-            if (s && W > 0.0) r = u128_to_double(s, -kAccFrac) * W * B.RD[d];
+            const u192 s{S.acc[3 * u], S.acc[3 * u + 1], S.acc[3 * u + 2]};
+            if ((s.w0 | s.w1 | s.w2) && W > 0.0) r = u192_to_double(s) * W * B.RD[d];
         }
         S.scores[u] = r;
     }
@@ -829,7 +829,7 @@ int prepare_base(Base &b) {
     if (g->perm) return fail(RS_EINVAL, "rs_server_create: graphs built with RS_REORDER are not served");
     b.n = g->n; b.nnz = g->nnz; b.k = g->k; b.dmax = g->dmax;
     int64_t unused = 0;
-    RS_CUDA_TRY(dalloc(&b.acc, 2 * (size_t)b.n, unused));
+    RS_CUDA_TRY(dalloc(&b.acc, 3 * (size_t)b.n, unused));
     RS_CUDA_TRY(dalloc(&b.scores, (size_t)b.n, unused));
     RS_CUDA_TRY(dalloc(&b.rowmax, (size_t)b.n, unused));
     cudaStream_t s = nullptr;
@@ -841,7 +841,7 @@ int prepare_base(Base &b) {
     uint32_t *ctab = nullptr;
     int *err = nullptr;
     if (!rc && b.n > 0) {
-        cudaError_t e = cudaMemcpyAsync(b.acc, g->acc, 2 * b.n * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s);
+        cudaError_t e = cudaMemcpyAsync(b.acc, g->acc, 3 * b.n * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s);
         int grid = 2 * sm_count();
         int64_t per = 1;
         { int64_t m = std::min<int64_t>(b.dmax, b.k); while (per < 2 * m) per <<= 1; }
@@ -912,7 +912,7 @@ int alloc_slot(rs_server *srv, Slot &sl) {
     RS_CUDA_TRY(dalloc(&v.xnew_col, (size_t)v.xpool_cap, b));
     RS_CUDA_TRY(dalloc(&v.xnew_lab, (size_t)v.xpool_cap, b));
     RS_CUDA_TRY(dalloc(&v.ctr, (size_t)C_NCTR, b));
-    RS_CUDA_TRY(dalloc(&v.acc, 2 * (size_t)n, b));
+    RS_CUDA_TRY(dalloc(&v.acc, 3 * (size_t)n, b));
     RS_CUDA_TRY(dalloc(&v.scores, (size_t)n, b));
     int64_t hub_slots = v.hub_cap > kCtaTab ? v.hub_cap * 4 * sm_count() : 1;
     RS_CUDA_TRY(dalloc(&v.hkey, (size_t)hub_slots, b));
@@ -996,7 +996,7 @@ int launch_incremental(rs_server *srv, Slot &sl, const Request &r) {
     RS_CUDA_TRY(cudaMemsetAsync(S.flag, 0, b.n * sizeof(int32_t), s));
     RS_CUDA_TRY(cudaMemsetAsync(S.ctr, 0, C_NCTR * sizeof(unsigned long long), s));
     RS_CUDA_TRY(cudaMemsetAsync(S.err, 0, sizeof(int32_t), s));
-    RS_CUDA_TRY(cudaMemcpyAsync(S.acc, b.acc, 2 * b.n * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
+    RS_CUDA_TRY(cudaMemcpyAsync(S.acc, b.acc, 3 * b.n * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
     Bounds x = request_bounds(b, r);
     int sms = sm_count();
     int64_t nn = (int64_t)r.nodes.size(), ne = (int64_t)r.src.size();
@@ -1022,7 +1022,7 @@ int launch_incremental(rs_server *srv, Slot &sl, const Request &r) {
 
 // device bytes of a full copy of a base graph (CSR twice, cross lists, G_x slots
 // with both values, per-node records and workspaces)
-int64_t full_bytes_estimate(const Base &b) { return 38 * b.nnz + 170 * b.n + (16 << 20); }
+int64_t full_bytes_estimate(const Base &b) { return 38 * b.nnz + 190 * b.n + (16 << 20); }
 
 // full path: restore a copy of the base graph, apply the removals, rescore
 int launch_full(rs_server *srv, Slot &sl, const Request &r) {
