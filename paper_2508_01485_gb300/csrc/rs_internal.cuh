@@ -16,9 +16,9 @@ namespace rs {
 // are launch parameters (rs_tuning in rs.h); these are their upper limits,
 // which size the shared-memory tables:
 //   small: d <= small_max (<= kSmallMax), tiles of 32 rows per warp;
-//   mid:   cap <= warp_cap (<= kWarpCap), one warp per row, a per-warp
+//   mid:   cap <= warp_cap (<= kWarpCap), d <= kMidDeg: one warp per row, a per-warp
 //          shared-memory table;
-//   large: cap <= cta_cap (<= kMidCap), one CTA per row, a per-CTA
+//   large: cap <= cta_cap (<= kMidCap), d <= kLargeDeg: one CTA per row, a per-CTA
 //          shared-memory table;
 //   hub:   larger rows; a hash table in global memory, rows split into chunks
 //          of hub_chunk neighbours processed by separate CTAs and merged by
@@ -27,6 +27,11 @@ constexpr int kSmallMax = 32;
 constexpr int kWarpCap = 512;
 constexpr int kMidCap = 2048;
 constexpr int32_t kEmpty = -1;
+// With few communities a long row's table is small all the same; a row's class therefore
+// also bounds its degree: a warp takes rows of at most kMidDeg entries, a CTA of at most
+// kLargeDeg.  (A 1.2M-entry graph of ten communities had rows of 5,000 entries in one
+// warp each: p2_mid 216 us.)
+constexpr int32_t kMidDeg = 512, kLargeDeg = 16384;
 
 // per-node record written by the first pass and gathered by the second
 struct __align__(16) NodeRec {
@@ -138,7 +143,6 @@ struct rs_graph {
     uint8_t *dead = nullptr;          // nnz edge marks used by removals
     // row classes
     int32_t *rows_small = nullptr, *rows_mid = nullptr, *rows_large = nullptr;
-    int32_t *rows_sort = nullptr;        // scratch of the degree ordering of the mid and large rows
     int64_t n_small = 0, n_mid = 0, n_large = 0;
     int32_t large_cap = 0;            // largest table among large rows
     rs::HubInfo *hubs = nullptr;      // device copy
@@ -148,6 +152,8 @@ struct rs_graph {
     int32_t *hub_sitem = nullptr;     // per slot-range item: hub index (a hub's table in ranges of
     int32_t *hub_srange = nullptr;    //   kHubSlotRange slots) and the range's number in the hub
     int64_t n_hub_sitems = 0;
+    // lengths the hub lists and tables are allocated for
+    int64_t cap_hubs = 0, cap_hub_items = 0, cap_hub_sitems = 0, cap_hub_entries = 0, cap_hub_slots = 0;
     int32_t *hslot = nullptr;         // per hub entry: its community's table slot (-1: own community)
     int32_t *hkey = nullptr;          // hub hash tables
     uint32_t *hcnt = nullptr;
@@ -158,6 +164,7 @@ struct rs_graph {
     // constant tables, sized dmax + 1
     uint64_t *LG = nullptr;           // round(log2(f) 2^58)
     double *RD = nullptr;             // 1 / (d (d - 1))
+    int32_t tab_dmax = -1;            // the largest degree they hold
     // scoring workspace
     rs::NodeRec *rec = nullptr;
     unsigned long long *acc = nullptr;        // 3 words per node

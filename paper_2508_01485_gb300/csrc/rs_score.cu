@@ -2211,7 +2211,7 @@ __global__ void __launch_bounds__(kThreads) strict_pairs_kernel(
                     const int64_t bu = off[u], bv = off[v];
                     const int32_t du = (int32_t)(off[u + 1] - bu), dv = (int32_t)(off[v + 1] - bv);
                     auto hub = [&](int32_t d) {        // a row of the hub class
-                        return d > small_max && dev_pow2_at_least(2u * (uint32_t)min(d, k)) > (uint32_t)cta_cap;
+                        return d > small_max && (d > kLargeDeg || dev_pow2_at_least(2u * (uint32_t)min(d, k)) > (uint32_t)cta_cap);
                     };
                     const bool hu = hub(du), hv = hub(dv);
                     const int32_t lu = hu ? du : ru.dx, lv = hv ? dv : rv.dx;
