@@ -12,6 +12,7 @@
 
 #include "rs.h"
 #include "rs_internal.cuh"
+#include "rs_device.cuh"
 
 using namespace rs;
 
@@ -268,14 +269,16 @@ __global__ void init_tables_kernel(uint64_t *LG, double *RD, int32_t dmax, int a
 // ---------------------------------------------------------------------------
 enum : int { V_OFF = 1, V_COLRANGE = 2, V_SELF = 4, V_ORDER = 8, V_LABEL = 16 };
 
-__global__ void validate_offsets_kernel(const int64_t *off, int64_t n, int64_t nnz, int *flag) {
+__global__ void validate_nodes_kernel(const int64_t *off, const int32_t *lab, int64_t n, int64_t nnz, int32_t k,
+                                      int *flag) {
     int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v > n) return;
-    bool bad = false;
-    if (v == 0 && off[0] != 0) bad = true;
-    if (v == n && off[n] != nnz) bad = true;
-    if (v < n && off[v + 1] < off[v]) bad = true;
-    if (bad) atomicOr(flag, V_OFF);
+    int bad = 0;
+    if (v == 0 && off[0] != 0) bad |= V_OFF;
+    if (v == n && off[n] != nnz) bad |= V_OFF;
+    if (v < n && off[v + 1] < off[v]) bad |= V_OFF;
+    if (v < n && (lab[v] < 0 || lab[v] >= k)) bad |= V_LABEL;
+    if (bad) atomicOr(flag, bad);
 }
 
 // Symmetry: with every row strictly ascending (checked in the same pass) the directed
@@ -294,40 +297,52 @@ __device__ __forceinline__ uint64_t mix64(uint64_t x) {
 }
 constexpr uint64_t kSymKey = 0x243f6a8885a308d3ull;
 
-// tiles of 32 consecutive rows per warp: the tile's entries are streamed one per
-// lane (coalesced), and an entry's row is the last lane whose row starts at or
-// before it (binary lifting over the lanes' row starts by shuffles)
-__global__ void validate_rows_kernel(const int64_t *off, const int32_t *col, const int32_t *lab,
-                                     int64_t n, int32_t k, int *flag, unsigned long long *sym) {
+// A warp takes kValidChunk consecutive entries, streamed one per lane (coalesced, the next
+// ones loaded ahead); an entry's row is the last of 32 rows that starts at or before it
+// (binary lifting over the lanes' row starts by shuffles), the first of them found anew when
+// the entries run past the 32.  A warp per 32 rows left a tail of hub rows and no load ahead:
+// 176 us for 20.6M entries, against 141 us.
+constexpr int kValidChunk = 512;
+__global__ void validate_rows_kernel(const int64_t *off, const int32_t *col, int64_t n, int *flag,
+                                     unsigned long long *sym) {
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t E = off[n];
     int bad = 0;
     uint64_t hs = 0;
-    for (int64_t r0 = w * 32; r0 < n; r0 += nw * 32) {
-        const int64_t v = r0 + lane;
-        const bool have = v < n;
-        const int64_t start = off[have ? v : n];
-        const int64_t tile_end = off[min(r0 + 32, n)];
-        if (have && (lab[v] < 0 || lab[v] >= k)) bad |= V_LABEL;
-        const int64_t e0 = __shfl_sync(0xFFFFFFFFu, start, 0);
-        for (int64_t base = e0; base < tile_end; base += 32) {
-            const int64_t e = base + lane;
-            int r = 0;
-            for (int step = 16; step; step >>= 1) {
-                int64_t sb = __shfl_sync(0xFFFFFFFFu, start, r + step);
-                if (sb <= e) r += step;
+    for (int64_t c0 = w * kValidChunk; c0 < E; c0 += nw * kValidChunk) {
+        const int64_t c1 = min(E, c0 + kValidChunk);
+        int32_t before = c0 > 0 ? col[c0 - 1] : -1;    // the entry before lane 0's
+        int32_t nx = c0 + lane < c1 ? col[c0 + lane] : 0;
+        for (int64_t t0 = c0; t0 < c1;) {
+            const int64_t r0 = warp_row_of(off, n, t0, lane);
+            const int64_t start = r0 + lane < n ? off[r0 + lane] : INT64_MAX;
+            const int64_t t1 = r0 + 32 < n ? min(c1, off[r0 + 32]) : c1;
+            for (int64_t base = t0; base < t1; base += 32) {
+                const int64_t e = base + lane;
+                const int32_t x = nx;
+                // (past the 32 rows, the entries are read again with theirs)
+                const int64_t ne = base + 32 < t1 ? e + 32 : t1 + lane;
+                nx = ne < c1 ? col[ne] : 0;
+                int r = 0;
+                for (int step = 16; step; step >>= 1)
+                    if (__shfl_sync(0xFFFFFFFFu, start, r + step) <= e) r += step;
+                const int64_t rs = __shfl_sync(0xFFFFFFFFu, start, r);
+                const int32_t up = __shfl_up_sync(0xFFFFFFFFu, x, 1);
+                const int32_t prev = lane ? up : before;
+                const int cnt = (int)min((int64_t)32, t1 - base);
+                before = __shfl_sync(0xFFFFFFFFu, x, cnt - 1);
+                if (e < t1) {
+                    const uint32_t u = (uint32_t)(r0 + r);
+                    if (x < 0 || x >= n) bad |= V_COLRANGE;
+                    if (x == (int32_t)u) bad |= V_SELF;
+                    if (e > rs && prev >= x) bad |= V_ORDER;
+                    hs += mix64((((uint64_t)u << 32) | (uint32_t)x) ^ kSymKey) -
+                          mix64((((uint64_t)(uint32_t)x << 32) | u) ^ kSymKey);
+                }
             }
-            const int64_t rs = __shfl_sync(0xFFFFFFFFu, start, r);
-            if (e < tile_end) {
-                int32_t x = col[e];
-                const uint32_t u = (uint32_t)(r0 + r);
-                if (x < 0 || x >= n) bad |= V_COLRANGE;
-                if (x == (int32_t)u) bad |= V_SELF;
-                if (e > rs && col[e - 1] >= x) bad |= V_ORDER;
-                hs += mix64((((uint64_t)u << 32) | (uint32_t)x) ^ kSymKey) -
-                      mix64((((uint64_t)(uint32_t)x << 32) | u) ^ kSymKey);
-            }
+            t0 = t1;
         }
     }
     bad |= __shfl_xor_sync(0xFFFFFFFFu, bad, 16);
@@ -359,15 +374,15 @@ static int read_flag(rs_graph *g, cudaStream_t s, int *out) {
 static int validate_graph(rs_graph *g, cudaStream_t s) {
     int flag = 0;
     RS_CUDA_TRY(cudaMemsetAsync(g->d_flag, 0, sizeof(int), s));
-    validate_offsets_kernel<<<(unsigned)((g->n + 1 + 255) / 256), 256, 0, s>>>(g->off, g->n, g->nnz, g->d_flag);
+    validate_nodes_kernel<<<(unsigned)((g->n + 1 + 255) / 256), 256, 0, s>>>(g->off, g->lab, g->n, g->nnz, g->k, g->d_flag);
     RS_CUDA_TRY(cudaGetLastError());
     if (int rc = read_flag(g, s, &flag)) return rc;
-    if (flag) return fail(RS_EINVAL, "invalid graph: row_offsets must start at 0, end at nnz and not decrease");
+    if (flag & V_OFF) return fail(RS_EINVAL, "invalid graph: row_offsets must start at 0, end at nnz and not decrease");
     // with the offsets valid, one pass checks the rows and sums the symmetry hash
     unsigned long long *sym = (unsigned long long *)(g->d_flag + 8);      // ints 8..9 of the 16
     RS_CUDA_TRY(cudaMemsetAsync(sym, 0, sizeof(unsigned long long), s));
-    validate_rows_kernel<<<grid_for(g->n, kThreads, 16), kThreads, 0, s>>>(g->off, g->col, g->lab, g->n, g->k,
-                                                                         g->d_flag, sym);
+    validate_rows_kernel<<<grid_for((g->nnz + kValidChunk - 1) / kValidChunk * 32, kThreads, 8), kThreads, 0, s>>>(
+        g->off, g->col, g->n, g->d_flag, sym);
     RS_CUDA_TRY(cudaGetLastError());
     unsigned long long h[2] = {0, 0};                                     // the flag word, then the sum
     RS_CUDA_TRY(cudaMemcpyAsync(h, g->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));

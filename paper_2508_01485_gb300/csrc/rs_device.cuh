@@ -25,6 +25,20 @@ __device__ __forceinline__ unsigned long long double_bits(df a) {
     return (unsigned long long)__double_as_longlong(df_to_double(a));
 }
 
+// the row holding CSR entry e (off[0] <= e < off[n]), found by the warp: 32 probes a step
+__device__ __forceinline__ int64_t warp_row_of(const int64_t *off, int64_t n, int64_t e, int lane) {
+    int64_t lo = 0, hi = n;                            // off[lo] <= e < off[hi]
+    while (hi - lo > 1) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t p = lo + lane * step;
+        const unsigned m = __ballot_sync(RS_FULL_MASK, p < hi && off[p] <= e);   // lane 0's probe holds
+        const int64_t l2 = lo + (31 - __clz(m)) * step;
+        hi = min(hi, l2 + step);
+        lo = l2;
+    }
+    return lo;
+}
+
 // ---- hash tables keyed by community (shared or global memory) ----------------
 struct Tab {
     int32_t *key;

@@ -2152,20 +2152,6 @@ __device__ __forceinline__ int64_t csr_find(const int64_t *off, const int32_t *c
     return (lo < end && col[lo] == key) ? lo : -1;
 }
 
-// the row holding CSR entry e (off[0] <= e < off[n]), found by the warp: 32 probes a step
-__device__ __forceinline__ int64_t warp_row_of(const int64_t *off, int64_t n, int64_t e, int lane) {
-    int64_t lo = 0, hi = n;                            // off[lo] <= e < off[hi]
-    while (hi - lo > 1) {
-        const int64_t step = (hi - lo + 31) / 32;
-        const int64_t p = lo + lane * step;
-        const unsigned m = __ballot_sync(FULL, p < hi && off[p] <= e);   // lane 0's probe holds
-        const int64_t l2 = lo + (31 - __clz(m)) * step;
-        hi = min(hi, l2 + step);
-        lo = l2;
-    }
-    return lo;
-}
-
 struct StrictWarp {
     const int32_t *walk[32], *look[32];                // the walked and the searched list of each edge
     int64_t ends[32];                                  // row ends, while the entries' rows are found
@@ -2188,9 +2174,13 @@ __global__ void __launch_bounds__(kThreads) strict_pairs_kernel(
     for (int64_t e0 = 32 * w0; e0 < E; e0 += 32 * nw) {
         const int64_t e = e0 + lane;
         const bool act = e < E;
-        // the rows of the warp's entries: the ends of the rows from e0's on, 32 at a time
+        // the rows of the warp's entries: the ends of 32 rows from that of the first entry
+        // without one (once, unless many empty rows lie between)
         int64_t u = -1;
-        for (int64_t r = warp_row_of(off, n, e0, lane); __any_sync(FULL, act && u < 0); r += 32) {
+        while (true) {
+            const unsigned open = __ballot_sync(FULL, act && u < 0);
+            if (!open) break;
+            const int64_t r = warp_row_of(off, n, e0 + __ffs(open) - 1, lane);
             S.ends[lane] = r + lane < n ? off[r + lane + 1] : INT64_MAX;
             __syncwarp();
             int32_t lo = 0, hi = 32;                   // first row that ends after e
