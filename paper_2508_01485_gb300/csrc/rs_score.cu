@@ -132,6 +132,8 @@ __device__ __forceinline__ int64_t cta_next(unsigned long long *ctr, long long *
 
 constexpr int kSlots = kSmallMax;
 
+constexpr int kFewRows = 8;             // rows per tile of the small-row kernels on small graphs
+
 __device__ __forceinline__ void store_rowsum(RowSum *rsum, int32_t v, const RowAgg &a) {
     RowSum r;
     r.xlo = (uint64_t)a.X;
@@ -235,14 +237,15 @@ __device__ __forceinline__ void p1_small_finish(SmallTile &T, int32_t v, int32_t
     Lall[v] = (int32_t)a.L;
 }
 
-// the tile's rows: lane l takes row rows[t0 + l]; prefix sums of the degrees, row starts
+// the tile's R rows: lane l takes row rows[t0 + l]; prefix sums of the degrees, row starts
 // and labels into T; returns the tile's entry count D
+template <int R>
 __device__ __forceinline__ int32_t p1_small_setup(SmallTile &T, const int64_t *__restrict__ off,
                                                   const int32_t *__restrict__ lab, const int32_t *__restrict__ rows,
                                                   int64_t nrows, int64_t t0, int lane, bool &have, int32_t &v,
                                                   int32_t &d, int32_t &cv) {
     int64_t i = t0 + lane;
-    have = i < nrows;
+    have = lane < R && i < nrows;
     v = have ? rows[i] : 0;
     int64_t b = have ? off[v] : 0;
     d = have ? (int32_t)(off[v + 1] - b) : 0;
@@ -263,6 +266,9 @@ __device__ __forceinline__ int32_t p1_small_setup(SmallTile &T, const int64_t *_
     return __shfl_sync(FULL, incl, 31);
 }
 
+// R rows per tile: 32, or kFewRows where that leaves too few warps to fill the GPU, whose time
+// is then one tile's chain of chunks (2,000 rows: 17 -> 12 us)
+template <int R>
 __global__ void __launch_bounds__(kThreads) p1_small_kernel(
     const int64_t *__restrict__ off, const int32_t *__restrict__ col, const int32_t *__restrict__ lab,
     const int32_t *__restrict__ rows, int64_t nrows, Batch B, const uint64_t *__restrict__ LG,
@@ -273,10 +279,10 @@ __global__ void __launch_bounds__(kThreads) p1_small_kernel(
     SmallTile &T = tiles[wid];
     int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t t0 = warp * 32; t0 < nrows; t0 += nwarps * 32) {
+    for (int64_t t0 = warp * R; t0 < nrows; t0 += nwarps * R) {
         bool have;
         int32_t v, d, cv;
-        const int32_t D = p1_small_setup(T, off, lab, rows, nrows, t0, lane, have, v, d, cv);
+        const int32_t D = p1_small_setup<R>(T, off, lab, rows, nrows, t0, lane, have, v, d, cv);
         // entry e of the tile: its row (last r with pre[r] <= e) and its CSR column
         auto locate = [&](int32_t e, int32_t &r, int32_t &x) {
             int32_t lo = 0, hi = 32;
@@ -343,7 +349,7 @@ __global__ void __launch_bounds__(kStageWarps * 32) p1_small_staged_kernel(
     for (int64_t t0 = warp * 32; t0 < nrows; t0 += nwarps * 32) {
         bool have;
         int32_t v, d, cv;
-        const int32_t D = p1_small_setup(T, off, lab, rows, nrows, t0, lane, have, v, d, cv);
+        const int32_t D = p1_small_setup<32>(T, off, lab, rows, nrows, t0, lane, have, v, d, cv);
         {
             const int32_t p0 = T.pre[lane];
             const int32_t *src = col + T.rb[lane];
@@ -2408,6 +2414,8 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     // (a phase with one class of rows takes the step's stream, and only the streams in use are
     // forked and joined)
     const bool mid_large = g->n_mid + g->n_large > 0;
+    // at most two 32-row tiles per SM: smaller ones
+    const bool few_rows = g->n_small <= 32 * 2 * (int64_t)grid_for(INT64_MAX / 2, 1, 1);
     unsigned used = 0;
     auto plan = [&](std::initializer_list<std::pair<int, bool>> classes) {
         used = 0;
@@ -2462,8 +2470,12 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
                                      kStageWarps * (sizeof(SmallTile) + sizeof(SmallStage)), AX(0)>>>(
                 g->off, g->col, g->lab, g->rows_small, g->n_small, B, g->LG, g->rec, g->Lall,
                 g->rsum, g->cl_col, g->cl_lab);
+        else if (few_rows)
+            p1_small_kernel<kFewRows><<<grid_for(g->n_small * (32 / kFewRows), NT, cps), NT, 0, AX(0)>>>(
+                g->off, g->col, g->lab, g->rows_small, g->n_small, B, g->LG, g->rec, g->Lall,
+                g->rsum, g->cl_col, g->cl_lab);
         else
-            p1_small_kernel<<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
+            p1_small_kernel<32><<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
                 g->off, g->col, g->lab, g->rows_small, g->n_small, B, g->LG, g->rec, g->Lall,
                 g->rsum, g->cl_col, g->cl_lab);
         RS_LAUNCHED(g, AX(0), "p1_small");
@@ -2510,7 +2522,12 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
         RS_LAUNCHED(g, AX(3), "hub_p2_emit");
     }
     if (g->n_small) {
-        p2_small_kernel<32><<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
+        if (few_rows)
+            p2_small_kernel<kNarrowRows><<<grid_for(g->n_small * (32 / kNarrowRows), NT, cps), NT, 0, AX(0)>>>(
+            g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
+            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX);
+        else
+            p2_small_kernel<32><<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
             g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
             g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX);
         RS_LAUNCHED(g, AX(0), "p2_small");
