@@ -278,6 +278,31 @@ int join_aux(rs_graph *g, cudaStream_t s, unsigned used);
         ::rs::prof_mark((g), (s), (name), true);       \
     } while (0)
 
+// Chained launches: a kernel that directly follows another of this library in its stream is
+// launched as its programmatic dependent, so that its launch and its blocks' start overlap
+// the other's end (a chain of ten kernels on 2,000 nodes: 71.5 -> 51.4 us).  Every kernel of
+// a chain begins with chain_wait(), before it touches memory: it lets its own dependent start
+// and waits until the kernels before it have finished and their writes are visible (no wait
+// for a kernel launched in the ordinary way).
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch(bool chained, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                   A &&...args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &attr;
+    c.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // grid size for grid-stride kernels: at most `cap_per_sm` CTAs per SM
 int grid_for(int64_t items, int per_block, int cap_per_sm);
 

@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(kThreads) p1_small_kernel(
     const int32_t *__restrict__ rows, int64_t nrows, Batch B, const uint64_t *__restrict__ LG,
     NodeRec *__restrict__ rec, int32_t *__restrict__ Lall,
     RowSum *__restrict__ rsum, int32_t *__restrict__ cl_col, int32_t *__restrict__ cl_lab) {
+    chain_wait();
     __shared__ SmallTile tiles[kThreads / 32];
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     SmallTile &T = tiles[wid];
@@ -752,6 +753,7 @@ __global__ void __launch_bounds__(kGxThreads) gx_offsets_kernel(
     const NodeRec *__restrict__ rec, int64_t n, int64_t *__restrict__ xoff, unsigned long long *status,
     unsigned long long *ticket, int *err, long spin_limit, int64_t withhold_tile, int32_t *__restrict__ cover,
     int32_t *last, P2Split split, int split_blocks) {
+    chain_wait();
     if ((int)blockIdx.x < split_blocks) {              // the P2 row lists, by blocks of their own
         p2_split(split, rec, blockIdx.x, split_blocks);
         return;
@@ -908,6 +910,7 @@ __global__ void __launch_bounds__(kThreads) p2_small_kernel(
     const int32_t *__restrict__ cl_col, const int32_t *__restrict__ cl_lab, unsigned long long *acc,
     const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, SigPair *__restrict__ xS, int32_t *__restrict__ xsk,
     int32_t *__restrict__ xout, int32_t *__restrict__ xin, GxNode *__restrict__ xnode, Strict SX) {
+    chain_wait();
     __shared__ P2Tile tiles[kThreads / 32];
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     P2Tile &T = tiles[wid];
@@ -1491,6 +1494,7 @@ __global__ void __launch_bounds__(kThreads) gx_mirror_kernel(
     int64_t n, const int64_t *__restrict__ xoff, const int32_t *__restrict__ xcol, SigPair *__restrict__ xS,
     const GxNode *__restrict__ xnode, const int32_t *__restrict__ xin, const int32_t *__restrict__ cover,
     const int32_t *__restrict__ last, const int32_t *__restrict__ xsk, int *err) {
+    chain_wait();
     __shared__ int64_t s_lo[kMirNodes];          // first in-slot of each staged node inside the tile
     __shared__ int32_t s_pre[kMirNodes + 1];     // prefix sums of the staged nodes' in-slots in the tile
     __shared__ int32_t s_wsum[kThreads / 32];
@@ -1659,6 +1663,7 @@ __global__ void __launch_bounds__(kP3Threads, kP3CtasPerSm) p3_list_kernel(
     Rev R, const int32_t *__restrict__ xout, const GxNode *__restrict__ xnode, unsigned long long *acc,
     unsigned long long *next_group, int32_t group, int64_t stride, unsigned long long *hvl, int64_t hvcap,
     unsigned long long *hv_count) {
+    chain_wait();
     __shared__ P3Stage S;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 #pragma unroll
@@ -2034,6 +2039,7 @@ __global__ void __launch_bounds__(kThreads, 3) p3_heavy_kernel(
     const int32_t *__restrict__ xout, const GxNode *__restrict__ xnode, unsigned long long *acc,
     const unsigned long long *__restrict__ hvl, int64_t hvcap, const unsigned long long *hv_count,
     unsigned long long *hv_next) {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char hv_smem[];
     P3Heavy &H = *reinterpret_cast<P3Heavy *>(hv_smem);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tid = threadIdx.x;
@@ -2276,6 +2282,7 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(
     int64_t n, const int64_t *__restrict__ off, const unsigned long long *__restrict__ acc,
     const int32_t *__restrict__ gid, const double *__restrict__ winv, const unsigned long long *__restrict__ wmax_bits,
     const double *__restrict__ RD, const int32_t *__restrict__ perm, double *scores) {
+    chain_wait();
     __shared__ double sh_w;
     if (!gid) {
         if (threadIdx.x == 0) {
@@ -2308,6 +2315,7 @@ struct InitArgs {
     int n;
 };
 __global__ void __launch_bounds__(kThreads) init_kernel(InitArgs A) {
+    chain_wait();
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int j = 0; j < A.n; ++j) {
         const InitRange &r = A.r[j];
@@ -2396,7 +2404,7 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     }
     if (g->strict) init(g->sx, 2 * g->nnz, 0);
     static_assert(sizeof(HubAgg) % sizeof(unsigned long long) == 0, "HubAgg is cleared by words");
-    init_kernel<<<grid_for(init_words / 2 + 1, NT, 8), NT, 0, s>>>(I);
+    RS_CUDA_TRY(launch(false, init_kernel, grid_for(init_words / 2 + 1, NT, 8), NT, 0, s, I));
     RS_LAUNCHED(g, s, "init");
     size_t p1_smem = 8 * (size_t)g->large_cap, p2_smem = 32 * (size_t)g->large_cap;
     // streams of the row kernels (rows_streams): every class on its own stream (0); the hub
@@ -2415,6 +2423,7 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     // forked and joined)
     const bool mid_large = g->n_mid + g->n_large > 0;
     // at most two 32-row tiles per SM: smaller ones
+    // (and where launches are most of the time, chained ones)
     const bool few_rows = g->n_small <= 32 * 2 * (int64_t)grid_for(INT64_MAX / 2, 1, 1);
     unsigned used = 0;
     auto plan = [&](std::initializer_list<std::pair<int, bool>> classes) {
@@ -2429,6 +2438,7 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
         const int j = rmode == 1 ? (i == 3 ? 3 : 0) : i;
         return used >> j & 1 ? g->aux[j] : s;
     };
+    const bool chain = few_rows && !mid_large && !g->n_hubs && !g->strict;
     plan({{3, g->n_hubs > 0}, {2, g->n_large > 0}, {4, g->n_mid > 0}, {0, g->n_small > 0}});
     // ---- P1: the larger classes are launched first (with per-class streams, on
     //      high-priority ones), so their maxima seed w_max early and most small rows skip
@@ -2471,9 +2481,9 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
                 g->off, g->col, g->lab, g->rows_small, g->n_small, B, g->LG, g->rec, g->Lall,
                 g->rsum, g->cl_col, g->cl_lab);
         else if (few_rows)
-            p1_small_kernel<kFewRows><<<grid_for(g->n_small * (32 / kFewRows), NT, cps), NT, 0, AX(0)>>>(
+            RS_CUDA_TRY(launch(chain, p1_small_kernel<kFewRows>, grid_for(g->n_small * (32 / kFewRows), NT, cps), NT, 0, AX(0),
                 g->off, g->col, g->lab, g->rows_small, g->n_small, B, g->LG, g->rec, g->Lall,
-                g->rsum, g->cl_col, g->cl_lab);
+                g->rsum, g->cl_col, g->cl_lab));
         else
             p1_small_kernel<32><<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
                 g->off, g->col, g->lab, g->rows_small, g->n_small, B, g->LG, g->rec, g->Lall,
@@ -2489,10 +2499,10 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
         return fail(RS_EINVAL, "rs_score: p3_mirror is set but its tile table is missing");
     const int64_t gx_tiles = (n + kGxTile - 1) / kGxTile;
     const int split_blocks = mid_large ? grid_for(nm + nl, kGxThreads, 8) : 0;
-    gx_offsets_kernel<<<(unsigned)(split_blocks + gx_tiles), kGxThreads, 0, s>>>(
+    RS_CUDA_TRY(launch(chain, gx_offsets_kernel, (unsigned)(split_blocks + gx_tiles), kGxThreads, 0, s,
         g->rec, n, g->xoff, g->wq + kWqGxStatus, g->wq + kWqGxTicket, err, g->gx_spin, g->gx_withhold,
         g->tune.p3_mirror ? g->xtile : nullptr, last_node,
-        P2Split{g->rows_mid, g->rows_large, nm, nl, g->tune.p2_cta_dx, g->p2rows, g->p2cnt}, split_blocks);
+        P2Split{g->rows_mid, g->rows_large, nm, nl, g->tune.p2_cta_dx, g->p2rows, g->p2cnt}, split_blocks));
     RS_LAUNCHED(g, s, "gx_offsets");
     const Strict SX{g->col, g->strict ? g->sx : nullptr};
     if (g->strict) {
@@ -2523,9 +2533,9 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     }
     if (g->n_small) {
         if (few_rows)
-            p2_small_kernel<kNarrowRows><<<grid_for(g->n_small * (32 / kNarrowRows), NT, cps), NT, 0, AX(0)>>>(
+            RS_CUDA_TRY(launch(chain, p2_small_kernel<kNarrowRows>, grid_for(g->n_small * (32 / kNarrowRows), NT, cps), NT, 0, AX(0),
             g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
-            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX);
+            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX));
         else
             p2_small_kernel<32><<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
             g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
@@ -2556,8 +2566,8 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     if (int rc = join_aux(g, s, used)) return rc;
     // ---- P3: reverse values (mirror mode), then triangles
     if (g->tune.p3_mirror) {
-        gx_mirror_kernel<<<grid_for(g->nnz, kMirTile, cps), NT, 0, s>>>(n, g->xoff, g->xcol, g->xS, g->xnode,
-                                                                       g->xin, g->xtile, last_node, g->xsk, err);
+        RS_CUDA_TRY(launch(chain, gx_mirror_kernel, grid_for(g->nnz, kMirTile, cps), NT, 0, s, n, g->xoff, g->xcol, g->xS, g->xnode,
+                                                                       g->xin, g->xtile, last_node, g->xsk, err));
         RS_LAUNCHED(g, s, "gx_mirror");
     }
     const Rev R{g->xS, g->xoff, g->xcol, g->xin, err, g->tune.p3_mirror != 0};
@@ -2569,16 +2579,16 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     while (group > 4 && n / group < 16 * (int64_t)grid_for(INT64_MAX / 2, 1, 1)) group >>= 1;
     const int list_grid = grid_for(n, group, kP3CtasPerSm);
     if (g->perm)                                     // a graph numbered by community: scrambled groups
-        p3_list_kernel<true><<<list_grid, kP3Threads, 0, s>>>(n, g->xoff, g->xcol, g->xsk, R, g->xout, g->xnode, g->acc,
+        RS_CUDA_TRY(launch(chain, p3_list_kernel<true>, list_grid, kP3Threads, 0, s, n, g->xoff, g->xcol, g->xsk, R, g->xout, g->xnode, g->acc,
                                                               next_group, group, p3_stride(n), hvl, hvcap,
-                                                              g->wq + kWqHvCount);
+                                                              g->wq + kWqHvCount));
     else
-        p3_list_kernel<false><<<list_grid, kP3Threads, 0, s>>>(n, g->xoff, g->xcol, g->xsk, R, g->xout, g->xnode, g->acc,
-                                                               next_group, group, 1, hvl, hvcap, g->wq + kWqHvCount);
+        RS_CUDA_TRY(launch(chain, p3_list_kernel<false>, list_grid, kP3Threads, 0, s, n, g->xoff, g->xcol, g->xsk, R, g->xout, g->xnode, g->acc,
+                                                               next_group, group, 1, hvl, hvcap, g->wq + kWqHvCount));
     RS_LAUNCHED(g, s, "p3_list");
     if (g->dmax > kWinCap) {                         // else no node has that many out-neighbours
-        p3_heavy_kernel<<<grid_for(hvcap, 1, 3), NT, sizeof(P3Heavy), s>>>(
-            n, g->xoff, g->xcol, R, g->xout, g->xnode, g->acc, hvl, hvcap, g->wq + kWqHvCount, g->wq + kWqHvNext);
+        RS_CUDA_TRY(launch(chain, p3_heavy_kernel, grid_for(hvcap, 1, 3), NT, sizeof(P3Heavy), s,
+            n, g->xoff, g->xcol, R, g->xout, g->xnode, g->acc, hvl, hvcap, g->wq + kWqHvCount, g->wq + kWqHvNext));
         RS_LAUNCHED(g, s, "p3_heavy");
     }
     // ---- finalize
@@ -2586,8 +2596,8 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
         graph_scale_kernel<<<(g->n_graphs + 255) / 256, 256, 0, s>>>(g->wmax_bits, g->n_graphs, g->winv);
         RS_LAUNCHED(g, s, "graph_scale");
     }
-    finalize_kernel<<<grid_for(n, NT, cps), NT, 0, s>>>(n, g->off, g->acc, g->gid, g->winv, g->wmax_bits, g->RD,
-                                                         g->perm, scores);
+    RS_CUDA_TRY(launch(chain && !g->gid, finalize_kernel, grid_for(n, NT, cps), NT, 0, s, n, g->off, g->acc, g->gid, g->winv, g->wmax_bits, g->RD,
+                                                         g->perm, scores));
     RS_LAUNCHED(g, s, "finalize");
     return 0;
 }

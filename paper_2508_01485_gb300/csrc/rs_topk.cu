@@ -302,9 +302,13 @@ __global__ void __launch_bounds__(kTkThreads) tk_select_kernel(TkArgs A) {
 // barrier between them costs less than a cooperative launch does)
 __global__ void __launch_bounds__(kTkThreads) tk_runs_kernel(TkArgs A) {
     __shared__ __align__(16) uint32_t sh[4 * kRun];
+    chain_wait();
     sort_runs(A, 0, 0, 0, (int)A.n, sh);
 }
-__global__ void __launch_bounds__(kTkThreads) tk_rank_kernel(TkArgs A) { rank_runs(A, 0, (int)A.n); }
+__global__ void __launch_bounds__(kTkThreads) tk_rank_kernel(TkArgs A) {
+    chain_wait();
+    rank_runs(A, 0, (int)A.n);
+}
 
 }  // namespace
 
@@ -355,10 +359,11 @@ int rs::topk_scores(rs_graph *g, const double *scores, int64_t n, int32_t k, int
     prof_begin(g, s);
     if (n <= rank_target(k)) {
         const int runs = (int)((n + kRun - 1) / kRun);
-        tk_runs_kernel<<<runs, kTkThreads, 0, s>>>(A);
+        RS_CUDA_TRY(launch(true, tk_runs_kernel, runs, kTkThreads, 0, s, A));
         RS_LAUNCHED(g, s, "tk_runs");
-        tk_rank_kernel<<<std::min(tk_grid, (int)((n * std::min(runs, 32) + kTkThreads - 1) / kTkThreads) + 1),
-                         kTkThreads, 0, s>>>(A);
+        RS_CUDA_TRY(launch(true, tk_rank_kernel,
+                           std::min(tk_grid, (int)((n * std::min(runs, 32) + kTkThreads - 1) / kTkThreads) + 1),
+                           kTkThreads, 0, s, A));
         RS_LAUNCHED(g, s, "tk_rank");
         return 0;
     }
