@@ -44,7 +44,7 @@ using namespace rs;
 
 namespace {
 
-constexpr int32_t kInT = 1, kRemoved = 2, kInW = 4;
+constexpr int32_t kInT = 1, kInW = 2;
 constexpr int kSvThreads = 256;
 constexpr int kWarpTab = 256;           // per-warp table slots of the Type-II warp kernel
 constexpr int kCtaTab = 1024;           // per-CTA shared table slots of the Type-II CTA kernel
@@ -85,7 +85,7 @@ enum { C_T = 0, C_WS, C_WB, C_TAB, C_X, C_WMAX, C_PAIR, C_TRI, C_NCTR = 8 };
 // per-request device state of a slot
 struct SlotView {
     uint32_t *dead;                  // removed CSR entries (bits)
-    int32_t *flag;                   // kInT | kRemoved | kInW per node
+    int32_t *flag;                   // kInT | kInW per node
     int32_t *tidx;                   // index in tlist (valid with kInT)
     int32_t *tlist, *wsmall, *wbig;
     int64_t tcap, wcap;
@@ -140,20 +140,21 @@ __device__ __forceinline__ void add_T(const SlotView &S, int32_t x) {
 }
 
 // ---- 1. removals: dead entries and the touched rows ------------------------------
+// kMarkStripes warps per node, each over every kMarkStripes-th run of 32 entries (the removed
+// nodes are mostly large ones, and a warp each left a tail: 194 us per request of the serving
+// burst, against 20 us); a node listed twice is marked again to no effect
+constexpr int kMarkStripes = 16;
 __global__ void sv_mark_nodes(BaseView B, SlotView S, const int32_t *nodes, int64_t m) {
     int lane = threadIdx.x & 31;
     int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = w; i < m; i += nw) {
-        int32_t v = nodes[i];
-        int first = 0;
-        if (lane == 0) first = !(atomicOr(&S.flag[v], kRemoved) & kRemoved);
-        first = __shfl_sync(FULL, first, 0);
-        if (!first) continue;
-        if (lane == 0) add_T(S, v);
-        for (int64_t e = B.off[v] + lane; e < B.off[v + 1]; e += 32) {
-            set_dead(S.dead, e);
-            int32_t u = B.col[e];
+    for (int64_t i = w; i < m * kMarkStripes; i += nw) {
+        const int32_t v = nodes[i / kMarkStripes];
+        const int64_t b = B.off[v], d = B.off[v + 1] - b;
+        if (i % kMarkStripes == 0 && lane == 0) add_T(S, v);
+        for (int64_t e = 32 * (i % kMarkStripes) + lane; e < d; e += 32 * kMarkStripes) {
+            set_dead(S.dead, b + e);
+            int32_t u = B.col[b + e];
             int64_t r = row_find(B.off, B.col, u, v);
             if (r >= 0) set_dead(S.dead, r);
             add_T(S, u);
@@ -297,12 +298,15 @@ __global__ void __launch_bounds__(kSvThreads) sv_trows(BaseView B, SlotView S) {
     }
 }
 
-// ---- 3. W = T and its neighbours, split by table size --------------------------------
+// ---- 3. W = T and its cross neighbours, split by table size ---------------------------
+// (an untouched row pushes terms that depend on its cross neighbours alone, so a touched
+// neighbour of its own community changes nothing there; with every neighbour of T in W, most
+// rows of W had nothing to do)
 __device__ __forceinline__ void add_W(const BaseView &B, const SlotView &S, int32_t u) {
     int32_t old = atomicOr(&S.flag[u], kInW);
     if (old & kInW) return;
     int64_t d = B.off[u + 1] - B.off[u];
-    bool small = table_cap(d, B.k) <= (uint32_t)kWarpTab;
+    bool small = table_cap(d, B.k) <= (uint32_t)kWarpTab && d <= kMidDeg;   // (few communities: small tables, long rows)
     unsigned long long i = atomicAdd(&S.ctr[small ? C_WS : C_WB], 1ull);
     if ((int64_t)i < S.wcap) (small ? S.wsmall : S.wbig)[i] = u;
     else atomicOr(S.err, 4);
@@ -313,7 +317,11 @@ __global__ void __launch_bounds__(kSvThreads) sv_mark_w(BaseView B, SlotView S) 
     for (int64_t i = blockIdx.x; i < nT; i += gridDim.x) {          // a CTA per touched row
         int32_t x = S.tlist[i];
         if (threadIdx.x == 0) add_W(B, S, x);
-        for (int64_t e = B.off[x] + threadIdx.x; e < B.off[x + 1]; e += blockDim.x) add_W(B, S, B.col[e]);
+        const int32_t cx = B.lab[x];
+        for (int64_t e = B.off[x] + threadIdx.x; e < B.off[x + 1]; e += blockDim.x) {
+            const int32_t u = B.col[e];
+            if (B.lab[u] != cx) add_W(B, S, u);
+        }
     }
 }
 
@@ -1003,7 +1011,7 @@ int launch_incremental(rs_server *srv, Slot &sl, const Request &r) {
     auto warps_grid = [&](int64_t items, int per_sm) {
         return (int)std::max<int64_t>(1, std::min<int64_t>((items * 32 + kSvThreads - 1) / kSvThreads, (int64_t)sms * per_sm));
     };
-    if (nn) sv_mark_nodes<<<warps_grid(nn, 8), kSvThreads, 0, s>>>(B, S, dn, nn);
+    if (nn) sv_mark_nodes<<<warps_grid(nn * kMarkStripes, 8), kSvThreads, 0, s>>>(B, S, dn, nn);
     if (ne) sv_mark_edges<<<(int)std::min<int64_t>((ne + 255) / 256, sms * 8), 256, 0, s>>>(B, S, ds, dd, ne);
     int64_t tb = std::max<int64_t>(x.t, 1);
     int64_t wb = std::min<int64_t>(b.n, x.t + x.dt + 1);
