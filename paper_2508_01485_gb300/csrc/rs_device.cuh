@@ -17,6 +17,22 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
+__device__ __forceinline__ unsigned lanemask_le() {
+    unsigned m;
+    asm("mov.u32 %0, %%lanemask_le;" : "=r"(m));
+    return m;
+}
+
+// Entries of consecutive rows, one per lane: `starts` has the bit of every lane whose entry is
+// its row's first (a row that began before has none).  The lanes of this lane's row, without
+// a warp match; and how many of the rows that start here start at or before this lane
+__device__ __forceinline__ unsigned row_lanes(unsigned starts) {
+    const unsigned below = starts & lanemask_le(), above = starts & ~lanemask_le();
+    const unsigned from = below ? RS_FULL_MASK << (31 - __clz(below)) : RS_FULL_MASK;
+    return from & (above ? (above & (0u - above)) - 1u : RS_FULL_MASK);
+}
+__device__ __forceinline__ int rows_started(unsigned starts) { return __popc(starts & lanemask_le()); }
+
 __device__ __forceinline__ uint32_t dev_pow2_at_least(uint32_t x) {
     return x <= 1 ? 1u : 1u << (32 - __clz(x - 1));
 }
