@@ -707,16 +707,18 @@ static void free_hub_tables(rs_graph *g) {
     pool_free_many(ptrs, sizeof(ptrs) / sizeof(ptrs[0]));
 }
 
-// builds rows_small / rows_mid / rows_large / hub tables from the current offsets; syncs
-static int classify_rows(rs_graph *g, cudaStream_t s) {
+static_assert(8 - 2 + H_WORDS <= rs::kCountWords, "the class header and the flag words before it");
+
+// builds rows_small / rows_mid / rows_large from the current offsets and copies d_flag's words
+// from 2 on (the applied count, the class header) to counts
+static int classify_begin(rs_graph *g, int *counts, cudaStream_t s) {
     int64_t n = g->n;
     g->version++;                  // row lists and hub tables are rebuilt: captured steps are stale
     const ClassSplit cs{g->tune.small_max, g->tune.warp_cap, g->tune.cta_cap};
-    int hdr[H_WORDS] = {};
     int *d_hdr = g->d_flag + 8, *hist = g->d_flag + 64;   // d_flag's words 0..7 are the scoring flags
     int32_t *hub_list = g->xout;  // n int32 scratch (workspace is allocated by now)
+    RS_CUDA_TRY(cudaMemsetAsync(d_hdr, 0, (64 - 8 + 2 * kDegBuckets) * sizeof(int), s));
     if (n > 0) {
-        RS_CUDA_TRY(cudaMemsetAsync(d_hdr, 0, (64 - 8 + 2 * kDegBuckets) * sizeof(int), s));
         const ClsArgs A{g->off, n, g->k, g->gid, g->gk, cs};
         const int64_t tiles = (n + kClsTile - 1) / kClsTile;
         int64_t *tile_small = g->xoff;
@@ -728,9 +730,17 @@ static int classify_rows(rs_graph *g, cudaStream_t s) {
         classify_scatter_kernel<<<(unsigned)tiles, kClsThreads, 0, s>>>(A, tile_small, hist, g->rows_small, g->rows_mid,
                                                                         g->rows_large);
         RS_CUDA_TRY(cudaGetLastError());
-        RS_CUDA_TRY(cudaMemcpyAsync(hdr, d_hdr, sizeof(hdr), cudaMemcpyDeviceToHost, s));
     }
-    RS_CUDA_TRY(cudaStreamSynchronize(s));
+    RS_CUDA_TRY(cudaMemcpyAsync(counts, g->d_flag + 2, rs::kCountWords * sizeof(int), cudaMemcpyDeviceToHost, s));
+    return 0;
+}
+
+// the class counts and, with hub rows, their work lists and tables; after s has reached the copy
+// of classify_begin, whose counts these are.  Waits for s only when there are hub rows
+static int classify_finish(rs_graph *g, const int *counts, cudaStream_t s) {
+    const int *hdr = counts + 6;
+    int *d_hdr = g->d_flag + 8;
+    int32_t *hub_list = g->xout;
     g->n_small = hdr[H_SMALL]; g->n_mid = hdr[H_MID]; g->n_large = hdr[H_LARGE];
     g->dmax = hdr[H_DMAX];
     g->large_cap = std::max(hdr[H_LARGECAP], 64);
@@ -839,6 +849,13 @@ static int classify_rows(rs_graph *g, cudaStream_t s) {
     }
     g->hub_slots = slots;
     return 0;
+}
+
+static int classify_rows(rs_graph *g, cudaStream_t s) {
+    int counts[rs::kCountWords] = {};
+    if (int rc = classify_begin(g, counts, s)) return rc;
+    RS_CUDA_TRY(cudaStreamSynchronize(s));
+    return classify_finish(g, counts, s);
 }
 
 int rs::reclassify(rs_graph *g, cudaStream_t s) {
@@ -1306,6 +1323,47 @@ static int compact_graph(rs_graph *g, cudaStream_t s) {
     return 0;
 }
 
+int rs::removal_begin(rs_graph *g, const int32_t *nodes, int64_t n_nodes, const int32_t *edge_src,
+                      const int32_t *edge_dst, int64_t n_edges, Removal &r, cudaStream_t s) {
+    // the lists in the P2 row lists' space (4 n words) when they fit, the counter in a flag word
+    int64_t words = n_nodes + 2 * n_edges;
+    int32_t *buf = g->p2rows;
+    unsigned long long *d_applied = (unsigned long long *)(g->d_flag + 2);
+    if (words > 4 * g->n) {
+        if (cudaError_t e = dmalloc(&r.own, words)) return cuda_fail(e, "alloc removal lists");
+        buf = r.own;
+    }
+    cudaError_t e = cudaMemsetAsync(d_applied, 0, sizeof(unsigned long long), s);
+    if (!e && n_nodes) e = cudaMemcpyAsync(buf, nodes, n_nodes * 4, cudaMemcpyHostToDevice, s);
+    if (!e && n_edges) e = cudaMemcpyAsync(buf + n_nodes, edge_src, n_edges * 4, cudaMemcpyHostToDevice, s);
+    if (!e && n_edges) e = cudaMemcpyAsync(buf + n_nodes + n_edges, edge_dst, n_edges * 4, cudaMemcpyHostToDevice, s);
+    if (!e && g->nnz) e = cudaMemsetAsync(g->dead, 0, 4 * ((g->nnz + 31) / 32), s);
+    if (e) return cuda_fail(e, "stage removals");
+    if (n_nodes) {
+        remove_nodes_kernel<<<grid_for(n_nodes * 32 * kStripes, kThreads, 8), kThreads, 0, s>>>(
+            g->off, g->col, (int32_t *)g->removed, (uint32_t *)g->dead, buf, n_nodes, d_applied);
+        if ((e = cudaGetLastError())) return cuda_fail(e, "remove nodes");
+    }
+    if (n_edges) {
+        remove_edges_kernel<<<(unsigned)((n_edges + 255) / 256), 256, 0, s>>>(
+            g->off, g->col, (uint32_t *)g->dead, buf + n_nodes, buf + n_nodes + n_edges, n_edges, d_applied);
+        if ((e = cudaGetLastError())) return cuda_fail(e, "remove edges");
+    }
+    if (g->n > 0)
+        if (int rc = compact_graph(g, s)) return rc;
+    return classify_begin(g, r.counts, s);
+}
+
+int rs::removal_finish(rs_graph *g, Removal &r, int64_t *applied, cudaStream_t s) {
+    unsigned long long a;
+    std::memcpy(&a, r.counts, sizeof(a));
+    if (applied) *applied = (int64_t)a;
+    pool_free(r.own);
+    r.own = nullptr;
+    if (int rc = classify_finish(g, r.counts, s)) return rc;
+    return build_tables(g, s);
+}
+
 extern "C" rs_status rs_apply_removals(rs_graph *g, const int32_t *nodes, int64_t n_nodes,
                                        const int32_t *edge_src, const int32_t *edge_dst, int64_t n_edges,
                                        int64_t *applied_out, void *stream) {
@@ -1332,41 +1390,16 @@ extern "C" rs_status rs_apply_removals(rs_graph *g, const int32_t *nodes, int64_
         edge_src = mapped.data() + n_nodes;
         edge_dst = mapped.data() + n_nodes + n_edges;
     }
-    // the lists in the P2 row lists' space (4 n words) when they fit, the counter in a flag word
-    int64_t words = n_nodes + 2 * n_edges;
-    int32_t *own = nullptr, *buf = g->p2rows;
-    unsigned long long *d_applied = (unsigned long long *)(g->d_flag + 2);
-    auto done = [&](int rc) { pool_free(own); return (rs_status)rc; };
-    if (words > 4 * g->n) {
-        if (cudaError_t e = dmalloc(&own, words)) return done(cuda_fail(e, "alloc removal lists"));
-        buf = own;
-    }
-    cudaError_t e = cudaMemsetAsync(d_applied, 0, sizeof(unsigned long long), s);
-    if (!e && n_nodes) e = cudaMemcpyAsync(buf, nodes, n_nodes * 4, cudaMemcpyHostToDevice, s);
-    if (!e && n_edges) e = cudaMemcpyAsync(buf + n_nodes, edge_src, n_edges * 4, cudaMemcpyHostToDevice, s);
-    if (!e && n_edges) e = cudaMemcpyAsync(buf + n_nodes + n_edges, edge_dst, n_edges * 4, cudaMemcpyHostToDevice, s);
-    if (!e && g->nnz) e = cudaMemsetAsync(g->dead, 0, 4 * ((g->nnz + 31) / 32), s);
-    if (e) return done(cuda_fail(e, "stage removals"));
-    if (n_nodes) {
-        remove_nodes_kernel<<<grid_for(n_nodes * 32 * kStripes, kThreads, 8), kThreads, 0, s>>>(
-            g->off, g->col, (int32_t *)g->removed, (uint32_t *)g->dead, buf, n_nodes, d_applied);
-        if ((e = cudaGetLastError())) return done(cuda_fail(e, "remove nodes"));
-    }
-    if (n_edges) {
-        remove_edges_kernel<<<(unsigned)((n_edges + 255) / 256), 256, 0, s>>>(
-            g->off, g->col, (uint32_t *)g->dead, buf + n_nodes, buf + n_nodes + n_edges, n_edges, d_applied);
-        if ((e = cudaGetLastError())) return done(cuda_fail(e, "remove edges"));
-    }
-    if (g->n > 0)
-        if (int rc = compact_graph(g, s)) return done(rc);
-    if (int rc = classify_rows(g, s)) return done(rc);
-    if (int rc = build_tables(g, s)) return done(rc);
-    unsigned long long applied = 0;
-    if ((e = cudaMemcpyAsync(&applied, d_applied, sizeof(applied), cudaMemcpyDeviceToHost, s)))
-        return done(cuda_fail(e, "read applied"));
-    if ((e = cudaStreamSynchronize(s))) return done(cuda_fail(e, "removals"));
-    if (applied_out) *applied_out = (int64_t)applied;
-    return done(RS_OK);
+    int counts[rs::kCountWords] = {};
+    rs::Removal r;
+    r.counts = counts;
+    int rc = rs::removal_begin(g, nodes, n_nodes, edge_src, edge_dst, n_edges, r, s);
+    cudaError_t e = cudaStreamSynchronize(s);
+    if (!rc && e) rc = cuda_fail(e, "removals");
+    if (!rc) rc = rs::removal_finish(g, r, applied_out, s);
+    pool_free(r.own);
+    if (!rc && (e = cudaStreamSynchronize(s))) rc = cuda_fail(e, "removals");
+    return (rs_status)rc;
 }
 
 // ---------------------------------------------------------------------------

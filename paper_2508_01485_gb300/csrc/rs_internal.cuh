@@ -319,4 +319,17 @@ int topk_prepare(rs_graph *g, int64_t n);
 // re-split g's rows by g->tune (rs_api.cu); synchronises s
 int reclassify(rs_graph *g, cudaStream_t s);
 
+// rs_apply_removals in two halves: the first enqueues everything up to the copy of the class
+// counts (with the applied count) into `counts`, without waiting for the device when `counts` is
+// pinned; the second, called after s has reached that copy, builds what is sized by them.
+// Ids are the graph's own and in range.
+constexpr int kCountWords = 16;
+struct Removal {
+    int *counts = nullptr;      // kCountWords words of host memory
+    int32_t *own = nullptr;     // the lists, when they don't fit the graph's scratch
+};
+int removal_begin(rs_graph *g, const int32_t *nodes, int64_t n_nodes, const int32_t *edge_src,
+                  const int32_t *edge_dst, int64_t n_edges, Removal &r, cudaStream_t s);
+int removal_finish(rs_graph *g, Removal &r, int64_t *applied, cudaStream_t s);
+
 }  // namespace rs
