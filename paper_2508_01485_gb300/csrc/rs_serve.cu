@@ -1108,6 +1108,14 @@ int launch_full(rs_server *srv, Slot &sl, const Request &r) {
 // the second half, after the slot's stream has run the first
 int finish_full(rs_server *srv, Slot &sl) {
     rs_graph *g = srv->copies[sl.copy].g;
+    // beside other requests the row kernels take turns on the slot's stream: the requests fill the
+    // GPU, and a stream per row class for each of them exceeds the device's hardware queues, whose
+    // streams then wait for one another (burst of 24 requests on 8 slots: 7.1 -> 6.8 ms); alone,
+    // or with streams chosen for the base graph, as for any graph
+    int busy = 0;
+    for (auto &o : srv->slots) busy += o.busy;
+    const int32_t streams = srv->bases[srv->copies[sl.copy].graph].g->tune.rows_streams;
+    g->tune.rows_streams = streams < 0 && busy > 1 ? 2 : streams;
     if (int rc = removal_finish(g, sl.removal, nullptr, sl.s)) return rc;
     if (int rc = score_graph(g, sl.v.scores, sl.s)) return rc;
     RS_CUDA_TRY(cudaMemsetAsync(sl.v.err, 0, sizeof(int32_t), sl.s));
