@@ -216,7 +216,7 @@ def peaks():
 
 def graph_stats(g, k_class=None):
     """Per row class (the library's default classes: small d <= 32, mid/large by
-    hash-table size 2 min(d, k) <= 512 / 2048, hub above) the rows R, CSR entries
+    hash-table size 2 min(d, k) <= 512 / 2048 with d <= 512 / 16,384, hub above) the rows R, CSR entries
     E, cross entries X (neighbours of another community) and G_x slots G; and the
     oriented G_x out-slots O.  k_class replaces g.k in the class rule (a packed
     batch sizes tables by its total number of communities)."""
@@ -232,7 +232,7 @@ def graph_stats(g, k_class=None):
     out = (dx[b] > dx[a]) | ((dx[b] == dx[a]) & (b > a))
     m = np.minimum(deg, k_class or g.k)
     cap = np.where(m > 0, 2 ** np.ceil(np.log2(np.maximum(2 * m, 1))), 1)
-    cls = np.where(deg <= 32, 0, np.where(cap <= 512, 1, np.where(cap <= 2048, 2, 3)))
+    cls = np.where(deg <= 32, 0, np.where((cap <= 512) & (deg <= 512), 1, np.where((cap <= 2048) & (deg <= 16384), 2, 3)))
     st = {"n": n, "E": E, "m": E // 2, "k": g.k, "dmax": int(deg.max()) if n else 0,
           "gx_slots": int(keep.sum()), "out_slots": int(out.sum()), "cross": int(cross.sum())}
     # P3's heavy nodes (more than 128 G_x out-neighbours): their out-slots and the
@@ -250,15 +250,13 @@ def graph_stats(g, k_class=None):
         st["G_" + name] = int((keep & sel[rows]).sum())
     for c, name in enumerate(["small", "mid", "large", "hub"]):
         put(name, cls == c)
-    # P2 splits mid and large rows by cross degree: <= 32 (no table), <= 128 (256-slot warp table),
-    # <= 256 (512-slot warp table), more (CTA)
-    put("mid_w", (cls == 1) & (dx <= 32))
-    put("mid_t", (cls == 1) & (dx > 32) & (dx <= 128))
-    put("mid_tw", (cls == 1) & (dx > 128))
-    put("large_w", (cls == 2) & (dx <= 32))
-    put("large_t", (cls == 2) & (dx > 32) & (dx <= 128))
-    put("large_tw", (cls == 2) & (dx > 128) & (dx <= 256))
-    put("large_c", (cls == 2) & (dx > 256))
+    # P2 splits mid and large rows by cross degree: <= 32 (tiles of rows), <= 128 (a warp), more
+    # (256 threads; rows of the large class with more than 256 the large CTA)
+    rest = (cls == 1) | (cls == 2)
+    put("p2_narrow", rest & (dx <= 32))
+    put("p2_mid", rest & (dx > 32) & (dx <= 128))
+    put("p2_large", (cls == 2) & (dx > 256))
+    put("p2_cta", rest & (dx > 128) & ~((cls == 2) & (dx > 256)))
     # compatibility names used by the JSON line
     st["n_small"], st["E_small"] = st["R_small"], st["E_small"]
     st["gx_slots_small"] = st["G_small"]
@@ -268,8 +266,7 @@ def graph_stats(g, k_class=None):
 # kernels launched on the forked streams of P1 and P2 (they overlap one another)
 CONCURRENT = {"p1_small", "p1_mid", "p1_large", "hub_p1_insert", "hub_p1_sums", "hub_p1_finish", "hub_p1_colmax",
               "p2_small", "p2_narrow",
-              "p2_mid", "p2_mid_wide", "p2_large_warp", "p2_large_warp_wide", "p2_large",
-              "hub_p2_insert", "hub_p2_counts", "hub_p2_emit", "mirror_tiles", "p2_split"}
+              "p2_mid", "p2_cta", "p2_large", "hub_p2_insert", "hub_p2_counts", "hub_p2_emit"}
 
 
 def kernel_bytes(name, st):
@@ -287,10 +284,8 @@ def kernel_bytes(name, st):
         return (4 + 8 + 16 + 24 + 8 + 8) * R + 8 * Xc + 16 * n * Xc / X + 12 * Gc
     table = {
         "p1_small": lambda: p1("small"), "p1_mid": lambda: p1("mid"), "p1_large": lambda: p1("large"),
-        "p2_small": lambda: p2("small"), "p2_narrow": lambda: p2("mid_w") + p2("large_w"),
-        "p2_mid": lambda: p2("mid_t"), "p2_mid_wide": lambda: p2("mid_tw"),
-        "p2_large_warp": lambda: p2("large_t"), "p2_large_warp_wide": lambda: p2("large_tw"),
-        "p2_large": lambda: p2("large_c"),
+        "p2_small": lambda: p2("small"), "p2_narrow": lambda: p2("p2_narrow"),
+        "p2_mid": lambda: p2("p2_mid"), "p2_cta": lambda: p2("p2_cta"), "p2_large": lambda: p2("p2_large"),
         # out-lists (ids, forward and reverse values are read only for triangles), out counts,
         # offsets and ranks of every node
         "p3_list": lambda: 4 * st["out_slots"] + (4 + 8 + 4) * n,
@@ -302,7 +297,8 @@ def kernel_bytes(name, st):
         "gx_mirror": lambda: (4 + 8 + 8) * st["out_slots"] + (4 + 8 + 4) * n,
         # the first id of every 8-slot sector of the G_x slots, read and written once
         "gx_skip": lambda: (4 + 4) * st["gx_slots"] / 8,
-        "finalize": lambda: (8 + 16 + 8) * n,
+        # offsets, three-word sums, scores
+        "finalize": lambda: (8 + 24 + 8) * n,
         "tk_select": lambda: 8 * n,
         # every node record (its dx) read, every G_x row offset written
         "gx_offsets": lambda: 16 * n + 8 * n,

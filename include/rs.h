@@ -240,9 +240,11 @@ rs_status rs_launch_count(const rs_graph *g, int64_t *launches);
  * fixed launch shapes, Sec. V).  Rows are split by degree d and by the hash
  * capacity cap = smallest power of two >= 2 min(d, k):
  *   small_max    rows with d <= small_max take the 32-row tile kernels    [1, 32]
- *   warp_cap     other rows with cap <= warp_cap take one warp each       {64,...,512}
- *   cta_cap      then rows with cap <= cta_cap take one CTA each;         {warp_cap,...,2048}
- *                larger rows are hubs (global table, split into chunks)
+ *   warp_cap     other rows with cap <= warp_cap (and d <= 512) take      {64,...,512}
+ *                one warp each
+ *   cta_cap      then rows with cap <= cta_cap (and d <= 16,384) take     {warp_cap,...,2048}
+ *                one CTA each; larger rows are hubs (global table, split
+ *                into chunks)
  *   hub_chunk    neighbours per hub work item                             {512,...,65536}
  *   p2_cta_dx    CTA rows with more cross neighbours than this take a     [32, 256]
  *                large CTA (p2_cta_threads) in the second pass (else a
