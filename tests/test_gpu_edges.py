@@ -4,6 +4,7 @@ a warp and of a CTA, removals and validation at the edges of 32-entry words and 
 import numpy as np
 import pytest
 
+import graphgen
 import oracle
 from tests.conftest import csr_from_edges
 
@@ -107,3 +108,30 @@ def test_validation_at_chunk_edges(rs, gap, at):
     labels[n - 1] = 2
     with pytest.raises(rs.RSError):
         rs.Graph.build(off, cols, labels, 2)
+
+
+@pytest.mark.parametrize("removed", [1, 40, 400])
+def test_whatif_with_few_and_many_pairs_per_warp(rs, removed):
+    """The triangle search takes one pair of a touched node and a neighbour per warp, or many:
+    the same bits as a full rescoring."""
+    g = graphgen.dcsbm_small(50000, seed=8, dmax=3000, mu=0.4)
+    nodes = np.random.default_rng(removed).choice(g.n, removed, replace=False)
+    srv = rs.Server([rs.Graph.from_generated(g)], max_slots=1, max_top_k=10)
+    a, path = srv.whatif(0, nodes=nodes, full="incremental")
+    b, _ = srv.whatif(0, nodes=nodes, full=True)
+    assert path == 1
+    np.testing.assert_array_equal(a.cpu().numpy().view(np.uint64), b.cpu().numpy().view(np.uint64))
+    srv.close()
+
+
+def test_full_request_needs_no_second_poll_to_run(rs):
+    """A poll that admits full requests leaves all of their work in the device's queues."""
+    g = graphgen.sbm_2000()
+    srv = rs.Server([rs.Graph.from_generated(g)], max_slots=3, max_top_k=10, mode="full")
+    for i in range(3):
+        srv.submit(0, nodes=[i], edges=[], top_k=10)
+    done = list(srv.poll(block=False))
+    torch.cuda.synchronize()
+    done += list(srv.poll(block=False))
+    assert len(done) == 3 and all(status == 0 and path == 0 for _, status, path, _, _ in done)
+    srv.close()
