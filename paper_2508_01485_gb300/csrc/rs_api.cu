@@ -771,8 +771,19 @@ static int classify_finish(rs_graph *g, const int *counts, cudaStream_t s) {
         hl.swap(hl2);
         offs.swap(offs2);
     }
-    std::vector<HubInfo> info(nh);
-    std::vector<int32_t> items, chunks;
+    // the uploads below are ordered on s, before the kernels there that read them; their sources
+    // are kept with the graph, because such a copy may still be reading them when it returns
+    std::vector<HubInfo> &info = g->h_hubs;
+    std::vector<int32_t> &items = g->h_hub_items, &chunks = g->h_hub_item_chunk;
+    std::vector<int32_t> &sitem = g->h_hub_sitem, &srange = g->h_hub_srange;
+    auto upload = [s](auto *dst, const auto &v) {
+        return cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, s);
+    };
+    info.assign(nh, HubInfo{});
+    items.clear();
+    chunks.clear();
+    sitem.clear();
+    srange.clear();
     int64_t slots = 0, hub_entries = 0;
     for (int i = 0; i < nh; ++i) {
         int64_t d = offs[3 * i + 1] - offs[3 * i];
@@ -797,9 +808,9 @@ static int classify_finish(rs_graph *g, const int *counts, cudaStream_t s) {
                           {{(void **)&g->hub_items, 4}, {(void **)&g->hub_item_chunk, 4},
                            {(void **)&g->hitem_out, 4}, {(void **)&g->hitem_in, 4}}))
             return rc;
-        RS_CUDA_TRY(cudaMemcpy(g->hubs, info.data(), nh * sizeof(HubInfo), cudaMemcpyHostToDevice));
-        RS_CUDA_TRY(cudaMemcpy(g->hub_items, items.data(), items.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-        RS_CUDA_TRY(cudaMemcpy(g->hub_item_chunk, chunks.data(), chunks.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        RS_CUDA_TRY(upload(g->hubs, info));
+        RS_CUDA_TRY(upload(g->hub_items, items));
+        RS_CUDA_TRY(upload(g->hub_item_chunk, chunks));
         // each hub's distinct foreign communities L_f, in scratch tables sized by degree;
         // the scoring tables then take 2 L_f slots (rounded up to a power of two), which
         // is far less on hub-skewed graphs (degree 54,097 with 4,671 communities)
@@ -828,8 +839,7 @@ static int classify_finish(rs_graph *g, const int *counts, cudaStream_t s) {
             info[i].tab = slots;
             slots += info[i].cap;
         }
-        RS_CUDA_TRY(cudaMemcpy(g->hubs, info.data(), nh * sizeof(HubInfo), cudaMemcpyHostToDevice));
-        std::vector<int32_t> sitem, srange;
+        RS_CUDA_TRY(upload(g->hubs, info));            // (s has run the first copy of info: it was waited for)
         for (int i = 0; i < nh; ++i)
             for (int32_t r = 0; (int64_t)r * kHubSlotRange < info[i].cap; ++r) {
                 sitem.push_back(i);
@@ -839,8 +849,8 @@ static int classify_finish(rs_graph *g, const int *counts, cudaStream_t s) {
         if (int rc = grow((int64_t)sitem.size(), g->cap_hub_sitems,
                           {{(void **)&g->hub_sitem, 4}, {(void **)&g->hub_srange, 4}}))
             return rc;
-        RS_CUDA_TRY(cudaMemcpy(g->hub_sitem, sitem.data(), sitem.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-        RS_CUDA_TRY(cudaMemcpy(g->hub_srange, srange.data(), srange.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        RS_CUDA_TRY(upload(g->hub_sitem, sitem));
+        RS_CUDA_TRY(upload(g->hub_srange, srange));
         if (int rc = grow(hub_entries, g->cap_hub_entries, {{(void **)&g->hslot, 4}})) return rc;
         if (int rc = grow(slots, g->cap_hub_slots,
                           {{(void **)&g->hkey, 4}, {(void **)&g->hcnt, 4}, {(void **)&g->hq, 16},

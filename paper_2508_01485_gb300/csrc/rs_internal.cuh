@@ -152,6 +152,10 @@ struct rs_graph {
     int32_t *hub_sitem = nullptr;     // per slot-range item: hub index (a hub's table in ranges of
     int32_t *hub_srange = nullptr;    //   kHubSlotRange slots) and the range's number in the hub
     int64_t n_hub_sitems = 0;
+    // what the hub lists were copied from: kept until the next classification, whose counts are
+    // read only after the stream has run these copies
+    std::vector<rs::HubInfo> h_hubs;
+    std::vector<int32_t> h_hub_items, h_hub_item_chunk, h_hub_sitem, h_hub_srange;
     // lengths the hub lists and tables are allocated for
     int64_t cap_hubs = 0, cap_hub_items = 0, cap_hub_sitems = 0, cap_hub_entries = 0, cap_hub_slots = 0;
     int32_t *hslot = nullptr;         // per hub entry: its community's table slot (-1: own community)

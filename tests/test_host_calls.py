@@ -1,0 +1,117 @@
+"""The library's host code on a stand-in for the CUDA runtime (tests/cuda_fake.cpp), without a GPU:
+what it copies, allocates and launches, and in which order.
+
+* the hub lists reach the device before the kernels that read them, on any stream."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+SRC = os.path.join(HERE, "cuda_fake.cpp")
+N, DEGREE = 64, 40                                        # nodes of the test graph and their degree
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2508_01485_gb300 import build
+    cxx = shutil.which("g++")
+    try:
+        if not cxx:
+            raise RuntimeError("no host C++ compiler")
+        build.build()
+        objs = [os.path.join(build.OUT_DIR, os.path.basename(s).replace(".cu", ".o")) for s in build.sources()]
+        if not all(os.path.exists(o) for o in objs):
+            build.build(force=True)
+    except RuntimeError as e:                             # no compiler on this machine
+        pytest.skip(str(e))
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+    out = os.path.join(HERE, "_build", "librs_fake.so")
+    os.makedirs(os.path.dirname(out), exist_ok=True)
+    tmp = out + ".%d.tmp" % os.getpid()
+    subprocess.check_call([cxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", inc, "-o", tmp, SRC, *objs])
+    os.replace(tmp, out)
+    L = ctypes.CDLL(out)
+    L.fake_stream.restype = ctypes.c_void_p
+    L.fake_unordered.restype = ctypes.c_char_p
+    L.fake_live_bytes.restype = ctypes.c_int64
+    L.fake_fail_allocation.argtypes = [ctypes.c_int64]
+    L.rs_last_error.restype = ctypes.c_char_p
+    return L
+
+
+def _ptr(a):
+    return ctypes.c_void_p(a.ctypes.data)
+
+
+class Calls:
+    """The C calls on one stream of the stand-in, which is non-blocking like a server's or a
+    torch side stream."""
+
+    def __init__(self, lib):
+        self.lib, self.s = lib, ctypes.c_void_p(lib.fake_stream())
+        self.scores = np.zeros(N)
+
+    def build(self, flags=0, nnz=N * DEGREE):
+        off = np.minimum(np.arange(N + 1) * DEGREE, nnz).astype(np.int64)
+        cols, labels = np.zeros(nnz, np.int32), np.zeros(N, np.int32)
+        g = ctypes.c_void_p()
+        assert self.lib.rs_build_graph(ctypes.c_int64(N), ctypes.c_int64(nnz), _ptr(off), 1, _ptr(cols), _ptr(labels), 8, 0,
+                                       flags, self.s, ctypes.byref(g)) == 0
+        return g
+
+    def score(self, g):
+        return self.lib.rs_score(g, _ptr(self.scores), None, self.s)
+
+    def remove(self, g, nodes=(0,), applied=None):
+        v = np.asarray(nodes, np.int32)
+        return self.lib.rs_apply_removals(g, _ptr(v), ctypes.c_int64(v.size), None, None, ctypes.c_int64(0),
+                                          ctypes.byref(applied) if applied is not None else None, self.s)
+
+    def server(self, graphs, slots=1, budget=1 << 40, mode=0):
+        arr, srv = (ctypes.c_void_p * len(graphs))(*[g.value for g in graphs]), ctypes.c_void_p()
+        assert self.lib.rs_server_create(arr, len(graphs), slots, ctypes.c_int64(budget), 4, mode, ctypes.byref(srv)) == 0
+        return srv
+
+    def submit(self, srv, nodes=(0,)):
+        v, ticket = np.asarray(nodes, np.int32), ctypes.c_int64()
+        assert self.lib.rs_server_submit(srv, 0, _ptr(v), ctypes.c_int64(v.size), None, None, ctypes.c_int64(0), 4,
+                                         ctypes.byref(ticket)) == 0
+
+    def poll(self, srv, block=1):
+        tickets, status, path = np.zeros(8, np.int64), np.zeros(8, np.int32), np.zeros(8, np.int32)
+        n = ctypes.c_int32()
+        assert self.lib.rs_server_poll(srv, 8, 0, _ptr(tickets), _ptr(status), _ptr(path), None, None, ctypes.byref(n), block) == 0
+        return list(zip(status[: n.value].tolist(), path[: n.value].tolist()))
+
+
+@pytest.fixture
+def calls(lib):
+    lib.fake_fail_allocation(-1)
+    return Calls(lib)
+
+
+@pytest.mark.parametrize("hubs", [1, 3])
+def test_hub_lists_are_ordered_before_their_readers(lib, calls, hubs):
+    """A build, removals that find the lists long enough and keep them, a re-split of the rows and
+    requests rescored on a server's copies: no kernel runs beside a copy that nothing orders
+    before it."""
+    lib.fake_classes(N - hubs, 0, 0, hubs, DEGREE, DEGREE, 3)
+    before = lib.fake_launches(b"hub_p1_insert"), lib.fake_launches(b"hub_distinct")
+    g = calls.build()
+    assert calls.score(g) == 0
+    for left in (hubs, max(1, hubs - 1)):
+        lib.fake_classes(N - left, 0, 0, left, DEGREE, DEGREE, 3)
+        assert calls.remove(g) == 0 and calls.score(g) == 0
+    lib.fake_classes(N - hubs, 0, 0, hubs, DEGREE, DEGREE, 3)
+    srv = calls.server([g], mode=1)
+    for _ in range(2):
+        calls.submit(srv)
+        assert calls.poll(srv) == [(0, 0)]
+    lib.rs_server_free(srv)
+    after = lib.fake_launches(b"hub_p1_insert"), lib.fake_launches(b"hub_distinct")
+    assert all(b - a >= 5 for a, b in zip(before, after))         # the paths with hub rows ran
+    assert lib.fake_unordered() == b""
