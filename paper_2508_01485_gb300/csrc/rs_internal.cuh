@@ -40,7 +40,7 @@ struct __align__(16) NodeRec {
     int32_t dx;       // cross-community degree (neighbours with another label)
 };
 
-// a G_x slot's values, 2^-48 fixed point: f = S(row -> neighbour), written by P2; at out-slots
+// a G_x slot's values, 2^-53 fixed point: f = S(row -> neighbour), written by P2; at out-slots
 // r = S(neighbour -> row), written by the mirror pass.  One 16-byte load brings both
 struct __align__(16) SigPair {
     uint64_t f, r;

@@ -13,7 +13,7 @@
 //    "A floating-point technique for extending the available precision");
 //  * Type-I terms are exact products of fixed-point values (see the pair products
 //    below), so that sums of them may be taken in any grouping;
-//  * every sum of terms is accumulated in 192-bit fixed point (2^-112 lsb), so
+//  * every sum of terms is accumulated in 192-bit fixed point (2^-128 lsb), so
 //    atomics commute and results are bit-identical whatever the schedule.
 #pragma once
 #include <stdint.h>
@@ -25,8 +25,8 @@ typedef unsigned __int128 u128;
 constexpr int kLogFrac = 58;      // LG[f] = round(log2(f) * 2^58)
 constexpr int kSFrac = 52;        // node scalar s_v stored as round(s_v * 2^52)
 constexpr int kTermFrac = 64;     // Type-II terms and pair products: 2^-64 lsb
-constexpr int kSigFrac = 48;      // G_x values S(x->y) stored as round(S 2^48)
-constexpr int kAccFrac = kSigFrac + kTermFrac;   // accumulators (three words): 2^-112 lsb
+constexpr int kSigFrac = 53;      // G_x values S(x->y) stored as round(S 2^53)
+constexpr int kAccFrac = 128;     // accumulators (three words): 2^-128 lsb
 
 // ---- double-float ----------------------------------------------------------
 
@@ -220,7 +220,12 @@ __device__ __forceinline__ void atomic_add_u128(unsigned long long *acc, u128 v)
     if (hi) atomicAdd(acc + 1, hi);
 }
 
-// ---- accumulators: three 64-bit words, 2^-112 lsb, modulo 2^192 ---------------------
+// ---- accumulators: three 64-bit words, 2^-128 lsb, modulo 2^192 ---------------------
+//
+// The last word counts whole units and the second one Type-II terms' lsb, so that such a term
+// touches two words and takes one returning atomic.  A node's terms are ordered pairs of
+// neighbours (w, v), fewer than nnz (< 2^33 in a GPU's memory), each below 2^28.6, the largest
+// weight: a sum stays below 2^62.
 
 struct u192 { uint64_t w0, w1, w2; };
 
@@ -234,8 +239,8 @@ __device__ __forceinline__ u192 u192_neg(u192 a) {
 }
 // a Type-II term (2^-64 lsb) in accumulator units
 __device__ __forceinline__ u192 u192_from_term(u128 v) {
-    constexpr int sh = kAccFrac - kTermFrac;
-    return u192{(uint64_t)v << sh, (uint64_t)(v >> (64 - sh)), (uint64_t)(v >> (128 - sh))};
+    static_assert(kAccFrac - kTermFrac == 64, "a term's words are the upper two");
+    return u192{0, (uint64_t)v, (uint64_t)(v >> 64)};
 }
 // concurrent adds commute; a word is touched only where it changes
 __device__ __forceinline__ void atomic_add_u192(unsigned long long *acc, u192 v) {
@@ -252,7 +257,7 @@ __device__ __forceinline__ void atomic_add_u192(unsigned long long *acc, u192 v)
     }
     if (a2) atomicAdd(acc + 2, (unsigned long long)a2);
 }
-// the double nearest to v 2^-112 (v below 2^176)
+// the double nearest to v 2^-128 (with a third word, what the first holds only breaks ties)
 __device__ __forceinline__ double u192_to_double(u192 v) {
     if (v.w2) return u128_to_double(((u128)v.w2 << 64) | v.w1 | (v.w0 ? 1 : 0), 64 - kAccFrac);
     return u128_to_double(((u128)v.w1 << 64) | v.w0, -kAccFrac);
@@ -260,14 +265,22 @@ __device__ __forceinline__ double u192_to_double(u192 v) {
 
 // ---- exact Type-I terms -------------------------------------------------------------
 //
-// The term of apex x of a triangle is S S (S + S).  The values S(x->y) are 2^-48 fixed
+// The term of apex x of a triangle is S S (S + S).  The values S(x->y) are 2^-53 fixed
 // point (S < 2^9.6: a weight is at most L log2 L, and L <= d < 2^24), so they and the pair
 // sums P = S + S fit 64 bits, and a term is formed as
-//     scale(S, pair(S', P)),   pair(x, y) = floor(x y 2^-32)  (2^-64 lsb, below 2^85),
-// the product of S and the pair exactly, in accumulator units.  As scale is linear, the
-// terms that share an outer S may be summed as pairs first and scaled once, and the sum
-// of any grouping has the same bits.  The floor drops less than 2^-64 of a value that is
-// at least 2^-12 when it is not 0 (S >= 0.014).
+//     scale(S, pair(S', P)),   pair(x, y) = floor(x y 2^-42)  (2^-64 lsb, below 2^85),
+// the product of S and the pair exactly (2^-117 lsb, in accumulator units).  As scale is
+// linear, the terms that share an outer S may be summed as pairs first and scaled once, and the
+// sum of any grouping has the same bits.
+//
+// The smallest S other than 0 is 0.0144: two communities, one of them with one of 2^24 - 1
+// neighbours.  Rounded to 2^-53 it keeps 2^-47 of its size, larger values more.  One term against
+// 113-bit arithmetic, rms error with S near 0.6 / 0.14 / 0.03 / 0.015: 8e-18, 2e-16, 2.8e-15 and
+// 8e-15; products of double-floats 2.6e-15, 2.7e-15, 2.3e-15 and 3.9e-15 (largest 1.8e-14 both
+// ways); S rounded to 2^-48, as it was, 5e-15, 2.4e-14, 1.2e-13 and 2.7e-13.  (Below 0.03 a row has
+// millions of neighbours and its entropy E / Y the log table's rounding: 1e-13 and more.)  More
+// bits would let P reach 2^64.  The floor of a pair drops less than 2^-64 of a value that is at
+// least 2^-12.
 
 // S(x->y) from its double-float value
 __device__ __forceinline__ uint64_t sig_fixed(df s) {
@@ -277,12 +290,20 @@ __device__ __forceinline__ uint64_t sig_fixed(df s) {
 // sums of pairs: at most 2^11 of them stay below 2^96
 struct u96 { uint64_t lo; uint32_t hi; };
 
-__device__ __forceinline__ u96 pair_term(uint64_t x, uint64_t y) {
+// x y without its lowest 32 bits
+struct Product { uint64_t hi; uint32_t lo; };
+__device__ __forceinline__ Product product(uint64_t x, uint64_t y) {
     const uint32_t x0 = (uint32_t)x, x1 = (uint32_t)(x >> 32), y0 = (uint32_t)y, y1 = (uint32_t)(y >> 32);
     const uint64_t m1 = (uint64_t)x0 * y1 + (((uint64_t)x0 * y0) >> 32);
     const uint64_t m2 = (uint64_t)x1 * y0 + (uint32_t)m1;
-    const uint64_t top = (uint64_t)x1 * y1 + (m1 >> 32) + (m2 >> 32);
-    return u96{(top << 32) | (uint32_t)m2, (uint32_t)(top >> 32)};
+    return Product{(uint64_t)x1 * y1 + (m1 >> 32) + (m2 >> 32), (uint32_t)m2};
+}
+// a pair is the product from bit kPairBit on
+constexpr int kPairBit = 2 * kSigFrac - kTermFrac - 32;
+static_assert(kPairBit > 0 && kPairBit < 32, "a product's lowest word is below the pair");
+__device__ __forceinline__ u96 pair_term(uint64_t x, uint64_t y) {
+    const Product p = product(x, y);
+    return u96{(p.hi << (32 - kPairBit)) | (p.lo >> kPairBit), (uint32_t)(p.hi >> (32 + kPairBit))};
 }
 __device__ __forceinline__ void u96_add(u96 &a, u96 b) {
     const u128 s = (((u128)a.hi << 64) | a.lo) + (((u128)b.hi << 64) | b.lo);
@@ -290,15 +311,21 @@ __device__ __forceinline__ void u96_add(u96 &a, u96 b) {
 }
 __device__ __forceinline__ u192 scale(uint64_t s, u96 p) {
     const u128 lo = (u128)s * p.lo, hi = (u128)s * p.hi + (uint64_t)(lo >> 64);
-    return u192{(uint64_t)lo, (uint64_t)hi, (uint64_t)(hi >> 64)};
+    constexpr int sh = kAccFrac - kSigFrac - kTermFrac;
+    return u192{(uint64_t)lo << sh, (uint64_t)(((u128)(uint64_t)hi << 64 | (uint64_t)lo) >> (64 - sh)),
+                (uint64_t)(hi >> (64 - sh))};
 }
 
 // sums of pairs as carry-free 32-bit words: word j takes bits [25 j, 25 j + 25) of a pair,
 // so up to 128 pairs may be added to the words, each by an add whose old value is not needed
+// (the words come straight from the product: a pair's own shift is left out).  The last word is
+// empty for pairs below 2^11, the usual ones, and its add is then left out: with pairs to 2^-74,
+// which need no shift anywhere, it never is, and a batch of 256 graphs lost 0.6% instead of 0.2%
+// (the 8M-node hub-skewed graph 0.9% instead of 1.1%) against S in 2^-48
 constexpr int kLimbs = 4, kLimbBits = 25;
-__device__ __forceinline__ uint32_t pair_limb(u96 p, int j) {
-    const u128 v = ((u128)p.hi << 64) | p.lo;
-    return (uint32_t)(v >> (kLimbBits * j)) & ((1u << kLimbBits) - 1);
+__device__ __forceinline__ uint32_t pair_limb(Product p, int j) {
+    const u128 v = ((u128)p.hi << 32) | p.lo;
+    return (uint32_t)(v >> (kPairBit + kLimbBits * j)) & ((1u << kLimbBits) - 1);
 }
 __device__ __forceinline__ u96 from_limbs(uint32_t l0, uint32_t l1, uint32_t l2, uint32_t l3) {
     const u128 v = (u128)l0 + ((u128)l1 << kLimbBits) + ((u128)l2 << (2 * kLimbBits)) + ((u128)l3 << (3 * kLimbBits));

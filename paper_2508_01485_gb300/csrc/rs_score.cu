@@ -1630,7 +1630,7 @@ struct P3Stage {
     long long ticket;
 };
 
-__device__ __forceinline__ void limbs_add(uint32_t (*l)[kWinCap], int e, u96 p) {
+__device__ __forceinline__ void limbs_add(uint32_t (*l)[kWinCap], int e, Product p) {
 #pragma unroll
     for (int j = 0; j < kLimbs; ++j) {
         const uint32_t v = pair_limb(p, j);
@@ -1657,9 +1657,9 @@ __device__ __forceinline__ void p3_flush(P3Stage &S, int wid, int m, const Rev &
         const int32_t a = S.anode[S.owner[el]], b = S.nb[el], c = S.nb[eh];
         const SigPair bc = R.get(S.qpos[wid][lane], c, b), ab = R.get(p3_slot(S, el), b, a),
                       ac = R.get(p3_slot(S, eh), c, a);
-        limbs_add(S.from, el, pair_term(ac.r, bc.f + bc.r));      // a: scaled by S(b->a)
-        limbs_add(S.to, el, pair_term(bc.r, ac.f + ac.r));        // b: scaled by S(a->b)
-        limbs_add(S.to, eh, pair_term(bc.f, ab.f + ab.r));        // c: scaled by S(a->c)
+        limbs_add(S.from, el, product(ac.r, bc.f + bc.r));      // a: scaled by S(b->a)
+        limbs_add(S.to, el, product(bc.r, ac.f + ac.r));        // b: scaled by S(a->b)
+        limbs_add(S.to, eh, product(bc.f, ab.f + ab.r));        // c: scaled by S(a->c)
     }
 }
 
@@ -2021,7 +2021,7 @@ __device__ __forceinline__ void hv_walk_b(P3Heavy &H, uint32_t *Q, const HvB &B,
                 const SigPair bc = R.get(pc, R.mirrored ? 0 : xcol[pc], B.b), sp = H.sp[p];
                 u96_add(sum_a, pair_term(sp.f, bc.f + bc.r));
                 u96_add(sum_b, pair_term(bc.r, sp.r));
-                const u96 t = pair_term(bc.f, Pab);
+                const Product t = product(bc.f, Pab);
 #pragma unroll
                 for (int j = 0; j < kLimbs; ++j) {
                     const uint32_t v = pair_limb(t, j);
