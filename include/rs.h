@@ -179,8 +179,10 @@ rs_status rs_topk(rs_graph *g, const double *scores, int32_t k, int32_t *ids_out
  * is already removed, or an edge that is absent (or already removed), is a
  * no-op and is not counted.  Any id outside [0, n) makes the call fail with
  * RS_EINVAL before anything is changed.  Node ids keep their meaning; a
- * removed node has degree 0 and scores 0.  Synchronises `stream` when
- * applied_out is given.
+ * removed node has degree 0 and scores 0.  Synchronises `stream`.  When the
+ * call fails for want of memory, the removals may have been made all the same
+ * and the graph's work lists not: rs_score is then refused (RS_EINVAL) until a
+ * call that rebuilds them succeeds (this one, with empty lists too).
  */
 rs_status rs_apply_removals(rs_graph *g, const int32_t *nodes, int64_t n_nodes,
                             const int32_t *edge_src, const int32_t *edge_dst, int64_t n_edges,

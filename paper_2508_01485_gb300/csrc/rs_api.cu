@@ -714,6 +714,7 @@ static_assert(8 - 2 + H_WORDS <= rs::kCountWords, "the class header and the flag
 static int classify_begin(rs_graph *g, int *counts, cudaStream_t s) {
     int64_t n = g->n;
     g->version++;                  // row lists and hub tables are rebuilt: captured steps are stale
+    g->classified = false;
     const ClassSplit cs{g->tune.small_max, g->tune.warp_cap, g->tune.cta_cap};
     int *d_hdr = g->d_flag + 8, *hist = g->d_flag + 64;   // d_flag's words 0..7 are the scoring flags
     int32_t *hub_list = g->xout;  // n int32 scratch (workspace is allocated by now)
@@ -858,6 +859,7 @@ static int classify_finish(rs_graph *g, const int *counts, cudaStream_t s) {
             return rc;
     }
     g->hub_slots = slots;
+    g->classified = true;
     return 0;
 }
 
@@ -876,12 +878,18 @@ int rs::reclassify(rs_graph *g, cudaStream_t s) {
 
 static int build_tables(rs_graph *g, cudaStream_t s) {
     if (g->LG && g->dmax <= g->tab_dmax) return 0;     // entries do not depend on dmax
-    g->tab_dmax = g->dmax;
+    const int64_t m = (int64_t)g->dmax + 1;
+    uint64_t *LG = nullptr;
+    double *RD = nullptr;
+    cudaError_t e = dmalloc(&LG, m);
+    if (!e) e = dmalloc(&RD, m);
+    if (e) {
+        pool_free(LG);
+        return cuda_fail(e, "alloc tables");
+    }
     pool_free(g->LG); pool_free(g->RD);
-    g->LG = nullptr; g->RD = nullptr;
-    int64_t m = (int64_t)g->dmax + 1;
-    RS_CUDA_TRY(dmalloc(&g->LG, m));
-    RS_CUDA_TRY(dmalloc(&g->RD, m));
+    g->LG = LG; g->RD = RD;
+    g->tab_dmax = g->dmax;
     init_tables_kernel<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(g->LG, g->RD, g->dmax, g->alg2 ? 1 : 0);
     RS_CUDA_TRY(cudaGetLastError());
     return 0;

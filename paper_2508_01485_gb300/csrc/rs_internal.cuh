@@ -215,6 +215,8 @@ struct rs_graph {
     std::vector<int32_t> iperm;               // RS_REORDER: the caller's id -> internal id (host)
     rs_tuning tune = rs::default_tuning_value();
     uint64_t version = 0;
+    bool classified = false;                  // the row lists, hub lists and tables are those of the CSR
+                                              // (not after a change that failed: scoring is refused)
     bool alg2 = false;                        // RS_ALG2_COMPAT: |L| = L_all - 1 for every column
     bool strict = false;                      // RS_TRIAD_STRICT: no closed triad with C(v) = C(u)
     unsigned long long *sx = nullptr;         // strict: X(w, u) per CSR entry (2 words), else null

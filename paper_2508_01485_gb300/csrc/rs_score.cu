@@ -2393,6 +2393,8 @@ static int64_t p3_stride(int64_t n) {
 
 int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     int64_t n = g->n;
+    if (!g->classified || g->dmax > g->tab_dmax)     // row lists or constant tables that are not there
+        return fail(RS_EINVAL, "rs_score: the last change of the graph failed half way; repeat it (or rs_set_tuning) first");
     g->scored_version = g->version;
     if (n == 0) return 0;
     constexpr int NT = kThreads;

@@ -1,7 +1,8 @@
 """The library's host code on a stand-in for the CUDA runtime (tests/cuda_fake.cpp), without a GPU:
 what it copies, allocates and launches, and in which order.
 
-* the hub lists reach the device before the kernels that read them, on any stream."""
+* the hub lists reach the device before the kernels that read them, on any stream;
+* an allocation that fails is reported, leaks nothing, and leaves nothing that a kernel would read."""
 import ctypes
 import os
 import shutil
@@ -115,3 +116,45 @@ def test_hub_lists_are_ordered_before_their_readers(lib, calls, hubs):
     after = lib.fake_launches(b"hub_p1_insert"), lib.fake_launches(b"hub_distinct")
     assert all(b - a >= 5 for a, b in zip(before, after))         # the paths with hub rows ran
     assert lib.fake_unordered() == b""
+
+
+def test_every_failed_allocation_of_a_build(lib, calls):
+    lib.fake_classes(N - 2, 0, 0, 2, DEGREE, DEGREE, 3)
+    before = lib.fake_live_bytes()
+    for n in range(200):
+        lib.fake_fail_allocation(n)
+        off, g = np.arange(N + 1) * DEGREE, ctypes.c_void_p()
+        cols, labels = np.zeros(N * DEGREE, np.int32), np.zeros(N, np.int32)
+        rc = lib.rs_build_graph(ctypes.c_int64(N), ctypes.c_int64(N * DEGREE), _ptr(off), 1, _ptr(cols), _ptr(labels), 8, 0, 0,
+                                calls.s, ctypes.byref(g))
+        if rc == 0:
+            break
+        assert rc == 2 and not g.value and lib.fake_live_bytes() == before, n          # RS_ENOMEM
+    lib.fake_fail_allocation(-1)
+    assert n > 40 and calls.score(g) == 0
+    lib.rs_free_graph(g)
+    assert lib.fake_live_bytes() == before
+
+
+def test_a_graph_whose_change_failed_is_not_scored(lib, calls):
+    """Removals that need longer hub lists and tables than there are, with each of the allocations
+    failing: the scoring that follows is refused, not run on what is missing."""
+    before = lib.fake_live_bytes()
+    for n in range(40):
+        lib.fake_classes(N, 0, 0, 0, 0, 0, 0)
+        g = calls.build()
+        lib.fake_classes(N - 3, 0, 0, 3, DEGREE, DEGREE, 3)
+        lib.fake_fail_allocation(n)
+        rc = calls.remove(g)
+        lib.fake_fail_allocation(-1)
+        ran = lib.fake_launches(b"hub_p1_insert")
+        if rc == 0:
+            break
+        assert rc == 2 and calls.score(g) == 1 and lib.fake_launches(b"hub_p1_insert") == ran, n      # RS_ENOMEM, RS_EINVAL
+        step = ctypes.c_void_p()
+        assert lib.rs_step_capture(g, _ptr(calls.scores), 0, None, None, ctypes.byref(step)) == 1
+        assert calls.remove(g) == 0 and calls.score(g) == 0 and lib.fake_launches(b"hub_p1_insert") == ran + 1
+        lib.rs_free_graph(g)
+        assert lib.fake_live_bytes() == before
+    assert n > 8 and calls.score(g) == 0
+    lib.rs_free_graph(g)
