@@ -1373,13 +1373,14 @@ int rs::removal_begin(rs_graph *g, const int32_t *nodes, int64_t n_nodes, const 
 }
 
 int rs::removal_finish(rs_graph *g, Removal &r, int64_t *applied, cudaStream_t s) {
-    unsigned long long a;
-    std::memcpy(&a, r.counts, sizeof(a));
-    if (applied) *applied = (int64_t)a;
     pool_free(r.own);
     r.own = nullptr;
     if (int rc = classify_finish(g, r.counts, s)) return rc;
-    return build_tables(g, s);
+    if (int rc = build_tables(g, s)) return rc;
+    unsigned long long a;
+    std::memcpy(&a, r.counts, sizeof(a));
+    if (applied) *applied = (int64_t)a;
+    return 0;
 }
 
 extern "C" rs_status rs_apply_removals(rs_graph *g, const int32_t *nodes, int64_t n_nodes,
@@ -1414,9 +1415,11 @@ extern "C" rs_status rs_apply_removals(rs_graph *g, const int32_t *nodes, int64_
     int rc = rs::removal_begin(g, nodes, n_nodes, edge_src, edge_dst, n_edges, r, s);
     cudaError_t e = cudaStreamSynchronize(s);
     if (!rc && e) rc = cuda_fail(e, "removals");
-    if (!rc) rc = rs::removal_finish(g, r, applied_out, s);
+    int64_t applied = 0;
+    if (!rc) rc = rs::removal_finish(g, r, &applied, s);
     pool_free(r.own);
     if (!rc && (e = cudaStreamSynchronize(s))) rc = cuda_fail(e, "removals");
+    if (!rc && applied_out) *applied_out = applied;
     return (rs_status)rc;
 }
 

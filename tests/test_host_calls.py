@@ -2,7 +2,8 @@
 what it copies, allocates and launches, and in which order.
 
 * the hub lists reach the device before the kernels that read them, on any stream;
-* an allocation that fails is reported, leaks nothing, and leaves nothing that a kernel would read."""
+* an allocation that fails is reported, leaks nothing, and leaves nothing that a kernel would read;
+* a call that fails writes no out-parameter."""
 import ctypes
 import os
 import shutil
@@ -157,4 +158,15 @@ def test_a_graph_whose_change_failed_is_not_scored(lib, calls):
         lib.rs_free_graph(g)
         assert lib.fake_live_bytes() == before
     assert n > 8 and calls.score(g) == 0
+    lib.rs_free_graph(g)
+
+
+def test_a_failed_removal_writes_no_count(lib, calls):
+    lib.fake_classes(N, 0, 0, 0, DEGREE, 0, 0)
+    g, applied = calls.build(), ctypes.c_int64(-7)
+    lib.fake_classes(N - 3, 0, 0, 3, DEGREE, DEGREE, 3)
+    lib.fake_fail_allocation(0)
+    assert calls.remove(g, applied=applied) == 2 and applied.value == -7
+    lib.fake_fail_allocation(-1)
+    assert calls.remove(g, applied=applied) == 0 and applied.value == 0     # (the stand-in's kernels count nothing)
     lib.rs_free_graph(g)
