@@ -87,7 +87,8 @@ struct SlotView {
     uint32_t *dead;                  // removed CSR entries (bits)
     int32_t *flag;                   // kInT | kInW per node
     int32_t *tidx;                   // index in tlist (valid with kInT)
-    int32_t *tlist, *wsmall, *wbig;
+    int32_t *tlist;
+    int32_t *wsmall, *wbig;          // n each, in the space of scores (done with before it is written)
     int64_t tcap, wcap;
     TRow *trow;
     int32_t *tkey;                   // touched rows' tables
@@ -938,8 +939,8 @@ int prepare_base(Base &b) {
 }
 
 void free_slot(Slot &sl) {
-    cudaFree(sl.v.dead); cudaFree(sl.v.flag); cudaFree(sl.v.tidx); cudaFree(sl.v.tlist); cudaFree(sl.v.wsmall);
-    cudaFree(sl.v.wbig); cudaFree(sl.v.trow); cudaFree(sl.v.tkey); cudaFree(sl.v.tcnt); cudaFree(sl.v.xnew_col);
+    cudaFree(sl.v.dead); cudaFree(sl.v.flag); cudaFree(sl.v.tidx); cudaFree(sl.v.tlist);
+    cudaFree(sl.v.trow); cudaFree(sl.v.tkey); cudaFree(sl.v.tcnt); cudaFree(sl.v.xnew_col);
     cudaFree(sl.v.xnew_lab); cudaFree(sl.v.ctr); cudaFree(sl.v.acc); cudaFree(sl.v.scores); cudaFree(sl.v.hkey);
     cudaFree(sl.v.hcnt); cudaFree(sl.v.hq); cudaFree(sl.v.pairs); cudaFree(sl.v.tris); cudaFree(sl.v.err); cudaFree(sl.d_req); cudaFree(sl.ids); cudaFree(sl.vals);
     cudaFreeHost(sl.h_counts);
@@ -965,8 +966,6 @@ int alloc_slot(rs_server *srv, Slot &sl) {
     RS_CUDA_TRY(dalloc(&v.flag, (size_t)n, b));
     RS_CUDA_TRY(dalloc(&v.tidx, (size_t)n, b));
     RS_CUDA_TRY(dalloc(&v.tlist, (size_t)v.tcap, b));
-    RS_CUDA_TRY(dalloc(&v.wsmall, (size_t)v.wcap, b));
-    RS_CUDA_TRY(dalloc(&v.wbig, (size_t)v.wcap, b));
     RS_CUDA_TRY(dalloc(&v.trow, (size_t)v.tcap, b));
     RS_CUDA_TRY(dalloc(&v.tkey, (size_t)v.pool_cap, b));
     RS_CUDA_TRY(dalloc(&v.tcnt, (size_t)v.pool_cap, b));
@@ -975,6 +974,10 @@ int alloc_slot(rs_server *srv, Slot &sl) {
     RS_CUDA_TRY(dalloc(&v.ctr, (size_t)C_NCTR, b));
     RS_CUDA_TRY(dalloc(&v.acc, 3 * (size_t)n, b));
     RS_CUDA_TRY(dalloc(&v.scores, (size_t)n, b));
+    // the lists of W are read last by the Type-II kernels, the scores written by sv_finalize: a
+    // slot with three-word sums takes the memory that one with two-word sums took
+    v.wsmall = (int32_t *)v.scores;
+    v.wbig = v.wsmall + n;
     int64_t hub_slots = v.hub_cap > kCtaTab ? v.hub_cap * 4 * sm_count() : 1;
     RS_CUDA_TRY(dalloc(&v.hkey, (size_t)hub_slots, b));
     RS_CUDA_TRY(dalloc(&v.hcnt, (size_t)hub_slots, b));
@@ -1083,8 +1086,9 @@ int launch_incremental(rs_server *srv, Slot &sl, const Request &r) {
 }
 
 // device bytes of a full copy of a base graph (CSR twice, cross lists, G_x slots
-// with both values, per-node records and workspaces)
-int64_t full_bytes_estimate(const Base &b) { return 38 * b.nnz + 190 * b.n + (16 << 20); }
+// with both values, per-node records and workspaces: 37 bytes an entry and 153 a node, the rest
+// for hub lists and tables)
+int64_t full_bytes_estimate(const Base &b) { return 38 * b.nnz + 170 * b.n + (16 << 20); }
 
 // full path: restore a copy of the base graph, apply the removals, rescore; in two halves,
 // because the rescoring's launches are sized by the row classes after the removals.  The server

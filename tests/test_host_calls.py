@@ -3,7 +3,8 @@ what it copies, allocates and launches, and in which order.
 
 * the hub lists reach the device before the kernels that read them, on any stream;
 * an allocation that fails is reported, leaks nothing, and leaves nothing that a kernel would read;
-* a call that fails writes no out-parameter."""
+* a call that fails writes no out-parameter;
+* a server's slots and copies take the memory that its budget is charged for."""
 import ctypes
 import os
 import shutil
@@ -57,11 +58,11 @@ class Calls:
         self.lib, self.s = lib, ctypes.c_void_p(lib.fake_stream())
         self.scores = np.zeros(N)
 
-    def build(self, flags=0, nnz=N * DEGREE):
-        off = np.minimum(np.arange(N + 1) * DEGREE, nnz).astype(np.int64)
-        cols, labels = np.zeros(nnz, np.int32), np.zeros(N, np.int32)
+    def build(self, flags=0, n=N):
+        nnz, off = n * DEGREE, np.arange(n + 1) * DEGREE
+        cols, labels = np.zeros(nnz, np.int32), np.zeros(n, np.int32)
         g = ctypes.c_void_p()
-        assert self.lib.rs_build_graph(ctypes.c_int64(N), ctypes.c_int64(nnz), _ptr(off), 1, _ptr(cols), _ptr(labels), 8, 0,
+        assert self.lib.rs_build_graph(ctypes.c_int64(n), ctypes.c_int64(nnz), _ptr(off), 1, _ptr(cols), _ptr(labels), 8, 0,
                                        flags, self.s, ctypes.byref(g)) == 0
         return g
 
@@ -77,6 +78,11 @@ class Calls:
         arr, srv = (ctypes.c_void_p * len(graphs))(*[g.value for g in graphs]), ctypes.c_void_p()
         assert self.lib.rs_server_create(arr, len(graphs), slots, ctypes.c_int64(budget), 4, mode, ctypes.byref(srv)) == 0
         return srv
+
+    def used(self, srv):
+        used = ctypes.c_int64()
+        assert self.lib.rs_server_info(srv, None, ctypes.byref(used), None, None) == 0
+        return used.value
 
     def submit(self, srv, nodes=(0,)):
         v, ticket = np.asarray(nodes, np.int32), ctypes.c_int64()
@@ -170,3 +176,27 @@ def test_a_failed_removal_writes_no_count(lib, calls):
     lib.fake_fail_allocation(-1)
     assert calls.remove(g, applied=applied) == 0 and applied.value == 0     # (the stand-in's kernels count nothing)
     lib.rs_free_graph(g)
+
+
+@pytest.mark.parametrize("n", [64, 30_000, 300_000])
+def test_memory_of_slots_and_copies(lib, calls, n):
+    """A slot takes 64 bytes a node beside its pools and a copy of a graph is counted as 170 a node and
+    38 an entry: a budget that held so many slots and copies holds them, and the copy fits its share."""
+    lib.fake_classes(n, 0, 0, 0, DEGREE, 0, 0)
+    g, nnz = calls.build(n=n), n * DEGREE
+    tcap, xcap = min(n, max(1 << 16, n // 4)), min(nnz, max(1 << 20, nnz // 4))
+    # dead bits, flags, touched rows and their tables, W and scores, sums, pairs, triangles, lists, ranking
+    slot = (nnz + 31) // 32 * 4 + 8 * n + 4 * tcap + 80 * tcap + 8 * (4 * xcap + 2 * tcap) + 8 * xcap + 64
+    slot += 8 * n + 16 * n + 8 * n + 24 + 8 * xcap + 12 * xcap + 4 + 4 * (1 << 16) + 12 * 4 + (2 * n + 16384) * 12 + 64
+    srv = calls.server([g], slots=2, budget=2 * slot, mode=1)
+    slots = ctypes.c_int32()
+    assert lib.rs_server_info(srv, ctypes.byref(slots), None, None, None) == 0
+    assert slots.value == 2 and calls.used(srv) == 2 * slot
+    lib.rs_server_free(srv)
+    g, copy = calls.build(n=n), 38 * nnz + 170 * n + (16 << 20)
+    srv = calls.server([g], slots=1, budget=slot + copy, mode=1)
+    before = lib.fake_live_bytes()
+    calls.submit(srv)
+    assert calls.poll(srv) == [(0, 0)]
+    assert calls.used(srv) == slot + copy and lib.fake_live_bytes() - before <= copy - (16 << 20)
+    lib.rs_server_free(srv)
