@@ -255,9 +255,10 @@ rs_status rs_launch_count(const rs_graph *g, int64_t *launches);
  *   p2_cta_threads  threads per CTA row in the second pass                {256, 512, 1024}
  *   ctas_per_sm  grid size of the grid-stride kernels, in CTAs per SM     [1, 32]
  *   p3_mirror    1: a pass pairs every G_x edge's two directed values     {0, 1}
- *                before the triangle listing; 0: the listing looks the
- *                reverse values of each triangle up in in-lists (fewer
- *                searches when G_x has few triangles per edge)
+ *                before the triangle listing (8 bytes more per CSR entry);
+ *                0: the listing looks the reverse values of each
+ *                triangle up in in-lists (fewer searches when G_x has
+ *                few triangles per edge)
  *   p1_stage     1: the small-row tiles of the first pass copy their          {0, 1}
  *                columns, then the neighbours' labels, into shared memory
  *                with asynchronous copies (cp.async) before matching; 0:

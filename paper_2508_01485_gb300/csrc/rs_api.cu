@@ -815,9 +815,13 @@ static int classify_finish(rs_graph *g, const int *counts, cudaStream_t s) {
         // each hub's distinct foreign communities L_f, in scratch tables sized by degree;
         // the scoring tables then take 2 L_f slots (rounded up to a power of two), which
         // is far less on hub-skewed graphs (degree 54,097 with 4,671 communities)
-        // (the scratch tables have fewer than 4 d slots for a row of degree d, 16 bytes of its
-        // 16-byte G_x slots)
-        int32_t *tkey = (int32_t *)g->xS, *lf = g->p2rows;
+        // (the scratch tables have fewer than 4 d slots for a row of degree d: 16 bytes a G_x slot
+        // hold them)
+        int32_t *tkey = (int32_t *)g->xS, *own = nullptr, *lf = g->p2rows;
+        if (slots * (int64_t)sizeof(int32_t) > (g->xS ? g->nnz * (int64_t)g->xS_bytes : 0)) {
+            RS_CUDA_TRY(dmalloc(&own, slots));
+            tkey = own;
+        }
         cudaError_t e = cudaMemsetAsync(tkey, 0xFF, (size_t)slots * sizeof(int32_t), s);
         if (!e) e = cudaMemsetAsync(lf, 0, (size_t)nh * sizeof(int32_t), s);
         if (!e) e = cudaMemsetAsync(d_hdr + H_ERR, 0, sizeof(int), s);
@@ -832,6 +836,7 @@ static int classify_finish(rs_graph *g, const int *counts, cudaStream_t s) {
         if (!e) e = cudaMemcpyAsync(L.data(), lf, nh * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
         if (!e) e = cudaMemcpyAsync(&overflow, d_hdr + H_ERR, sizeof(int), cudaMemcpyDeviceToHost, s);
         if (!e) e = cudaStreamSynchronize(s);
+        pool_free(own);
         if (e) return cuda_fail(e, "hub community counts");
         if (overflow) return fail(RS_ECUDA, "hub community count: scratch table full (library bug)");
         slots = 0;
@@ -895,14 +900,18 @@ static int build_tables(rs_graph *g, cudaStream_t s) {
     return 0;
 }
 
-// the mirror pass's tile table exists while that pass is selected
+// the G_x slots hold both values and the mirror pass has its tile table while that pass is
+// selected; without it a slot holds one, 8 bytes less
 int rs::set_mirror_buffer(rs_graph *g) {
-    if (g->tune.p3_mirror && !g->xtile) {
-        RS_CUDA_TRY(dmalloc(&g->xtile, g->nnz / kMirTile + 2));
-    } else if (!g->tune.p3_mirror && g->xtile) {
-        RS_CUDA_TRY(pool_free(g->xtile));
-        g->xtile = nullptr;
-    }
+    const uint32_t bytes = g->tune.p3_mirror ? sizeof(SigPair) : sizeof(uint64_t);
+    if (g->xS && g->xS_bytes == bytes) return 0;
+    void *old[] = {g->xS, g->xtile};
+    g->xS = nullptr;
+    g->xtile = nullptr;
+    RS_CUDA_TRY(pool_free_many(old, 2));
+    if (g->tune.p3_mirror) RS_CUDA_TRY(dmalloc(&g->xtile, g->nnz / kMirTile + 2));
+    RS_CUDA_TRY(pool_malloc(&g->xS, (size_t)std::max<int64_t>(g->nnz, 1) * bytes));
+    g->xS_bytes = bytes;
     return 0;
 }
 
@@ -929,7 +938,6 @@ static int alloc_workspace(rs_graph *g) {
     RS_CUDA_TRY(dmalloc(&g->xoff, n + 1));
     RS_CUDA_TRY(dmalloc(&g->xcol, nnz + 8));
     RS_CUDA_TRY(dmalloc(&g->xsk, nnz / 8 + 1));
-    RS_CUDA_TRY(dmalloc(&g->xS, nnz));
     RS_CUDA_TRY(dmalloc(&g->xnode, n));
     RS_CUDA_TRY(dmalloc(&g->xout, n));
     RS_CUDA_TRY(dmalloc(&g->xin, n));

@@ -45,6 +45,14 @@ struct __align__(16) NodeRec {
 struct __align__(16) SigPair {
     uint64_t f, r;
 };
+// the values of all slots: pairs while the mirror pass is selected (p3_mirror), else f alone
+struct SigSlots {
+    unsigned char *base;
+    uint32_t bytes;                           // per slot
+    __device__ __forceinline__ uint64_t &f(int64_t slot) const {
+        return *reinterpret_cast<uint64_t *>(base + slot * bytes);
+    }
+};
 
 // what P3 gathers of a G_x node: the start of its slots, its out-neighbours and its cross
 // degree (rank); written by P2 for every row with cross neighbours
@@ -180,7 +188,9 @@ struct rs_graph {
     int64_t *xoff = nullptr;                  // G_x row offsets (n + 1)
     int32_t *xcol = nullptr;                  // G_x neighbours (capacity nnz + 8: whole 8-slot sectors)
     int32_t *xsk = nullptr;                   // first id of every 8-slot sector of xcol (nnz / 8 + 1)
-    rs::SigPair *xS = nullptr;                // S(w -> u) = w_w(C(u))^(1/3) and, at out-slots, S(u -> w)
+    void *xS = nullptr;                       // S(w -> u) = w_w(C(u))^(1/3) and, with p3_mirror at
+    uint32_t xS_bytes = 0;                    //   out-slots, S(u -> w); bytes per slot (16, or 8 without)
+    rs::SigSlots sig() const { return rs::SigSlots{(unsigned char *)xS, xS_bytes}; }
     int32_t *xout = nullptr, *xin = nullptr;  // out / in counts per node
     rs::GxNode *xnode = nullptr;
     int32_t *p2rows = nullptr;                // P2 row lists by cross degree (4 n), counted in p2cnt

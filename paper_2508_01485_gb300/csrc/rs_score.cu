@@ -33,6 +33,7 @@
 // exact products, so the scores depend neither on the order in which threads run
 // nor on how terms are grouped before they are added.
 #include <initializer_list>
+#include <type_traits>
 #include <utility>
 
 #include "rs.h"
@@ -897,9 +898,14 @@ constexpr int kNarrowRows = 8;                 // rows per tile of the narrow mi
 // the slot space also the packed index entry xsk[p / 8] (searches of long out-lists read it;
 // every slot inside a row is written once here, so the entries of sectors starting inside
 // rows are complete when P2 ends)
-__device__ __forceinline__ void gx_put(int32_t *xcol, SigPair *xS, int32_t *xsk, int64_t p, int32_t u, uint64_t sig) {
+// (the P2 kernels are compiled for both kinds of slots: a stride in bytes, known to the launch only,
+// took 0.6% of a batch of 256 graphs)
+__device__ __forceinline__ void put_sig(SigPair *xS, int64_t p, uint64_t sig) { xS[p].f = sig; }
+__device__ __forceinline__ void put_sig(uint64_t *xS, int64_t p, uint64_t sig) { xS[p] = sig; }
+template <class Slot>
+__device__ __forceinline__ void gx_put(int32_t *xcol, Slot *xS, int32_t *xsk, int64_t p, int32_t u, uint64_t sig) {
     xcol[p] = u;
-    xS[p].f = sig;
+    put_sig(xS, p, sig);
     if ((p & 7) == 0) xsk[p >> 3] = u;
 }
 
@@ -921,12 +927,12 @@ struct P2Tile {
     uint64_t st[32];
 };
 
-template <int R>
+template <int R, class Slot>
 __global__ void __launch_bounds__(kThreads) p2_small_kernel(
     const int64_t *__restrict__ off, const int32_t *__restrict__ rows, int64_t nrows_host,
     const int32_t *__restrict__ nrows_dev, const uint64_t *__restrict__ LG, const NodeRec *__restrict__ rec, const RowSum *__restrict__ rsum,
     const int32_t *__restrict__ cl_col, const int32_t *__restrict__ cl_lab, unsigned long long *acc,
-    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, SigPair *__restrict__ xS, int32_t *__restrict__ xsk,
+    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, Slot *__restrict__ xS, int32_t *__restrict__ xsk,
     int32_t *__restrict__ xout, int32_t *__restrict__ xin, GxNode *__restrict__ xnode, Strict SX) {
     chain_wait();
     __shared__ P2Tile tiles[kThreads / 32];
@@ -1048,11 +1054,12 @@ constexpr int kP2Per = kP2WarpDx / 32;
 constexpr int kP2MidSlots = 2 * kP2WarpDx, kMidSlotBytes = 4 + 4 + 16;   // key, count, 2-word sum
 constexpr size_t kP2MidSmem = (size_t)kMidWarps * kP2MidSlots * kMidSlotBytes;
 
+template <class Slot>
 __global__ void __launch_bounds__(kThreads) p2_mid_kernel(
     const int64_t *__restrict__ off, const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, Batch B,
     const uint64_t *__restrict__ LG, const NodeRec *__restrict__ rec, const RowSum *__restrict__ rsum,
     const int32_t *__restrict__ cl_col, const int32_t *__restrict__ cl_lab, unsigned long long *acc,
-    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, SigPair *__restrict__ xS, int32_t *__restrict__ xsk,
+    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, Slot *__restrict__ xS, int32_t *__restrict__ xsk,
     int32_t *__restrict__ xout, int32_t *__restrict__ xin, GxNode *__restrict__ xnode, int *err, Strict SX, unsigned long long *wq) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t stage[kThreads];
@@ -1155,9 +1162,9 @@ __device__ __forceinline__ Tab p2_table(unsigned char *base, uint32_t cap) {
 }
 
 // CTA-ordered compaction of the G_x entries of one round; returns this thread's position
-template <int NT>
+template <int NT, class Slot>
 __device__ __forceinline__ void gx_round(bool out, bool in, int64_t xb, int32_t dxw, int32_t u, uint64_t sig,
-                                         int32_t &base_out, int32_t &base_in, int32_t *xcol, SigPair *xS,
+                                         int32_t &base_out, int32_t &base_in, int32_t *xcol, Slot *xS,
                                          int32_t *xsk, int32_t *sh_cnt /* 2 * NT/32 */) {
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned mo = __ballot_sync(FULL, out), mi = __ballot_sync(FULL, in);
@@ -1174,12 +1181,12 @@ __device__ __forceinline__ void gx_round(bool out, bool in, int64_t xb, int32_t 
     __syncthreads();
 }
 
-template <int NT>
+template <int NT, class Slot>
 __global__ void __launch_bounds__(NT) p2_large_kernel(
     const int64_t *__restrict__ off, const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, Batch B,
     const uint64_t *__restrict__ LG, const NodeRec *__restrict__ rec, const RowSum *__restrict__ rsum,
     const int32_t *__restrict__ cl_col, const int32_t *__restrict__ cl_lab, unsigned long long *acc,
-    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, SigPair *__restrict__ xS, int32_t *__restrict__ xsk,
+    const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol, Slot *__restrict__ xS, int32_t *__restrict__ xsk,
     int32_t *__restrict__ xout, int32_t *__restrict__ xin, GxNode *__restrict__ xnode, int *err, Strict SX, unsigned long long *wq) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int32_t sh_cnt[2 * NT / 32];
@@ -1329,14 +1336,14 @@ __global__ void __launch_bounds__(NT) hub_p2_counts_kernel(
 }
 
 // hub rows, P2 step 3: Type-II terms and the G_x entries of each chunk
-template <int NT>
+template <int NT, class Slot>
 __global__ void __launch_bounds__(NT) hub_p2_emit_kernel(
     const int64_t *__restrict__ off, const int32_t *__restrict__ col, const HubInfo *__restrict__ hubs,
     const int32_t *__restrict__ items, const int32_t *__restrict__ chunks, int64_t nitems, int32_t chunk_len,
     const NodeRec *__restrict__ rec, const int32_t *__restrict__ hslot,
     const unsigned long long *hq, const df *hsig, const int32_t *hitem_out, const int32_t *hitem_in,
     unsigned long long *acc, const int64_t *__restrict__ xoff, int32_t *__restrict__ xcol,
-    SigPair *__restrict__ xS, int32_t *__restrict__ xsk, int *err, Strict SX) {
+    Slot *__restrict__ xS, int32_t *__restrict__ xsk, int *err, Strict SX) {
     __shared__ int32_t sh_cnt[2 * NT / 32];
     int tid = threadIdx.x;
     for (int64_t it = blockIdx.x; it < nitems; it += gridDim.x) {
@@ -1393,7 +1400,7 @@ __global__ void __launch_bounds__(NT) hub_p2_emit_kernel(
 // (0.11 on the 1M-node DC-SBM graph), the second when they are many; the
 // choice is a launch parameter (p3_mirror).
 __device__ __forceinline__ uint64_t in_value(int32_t x, int32_t y, const int64_t *xoff, const int32_t *xcol,
-                                             const SigPair *xS, const int32_t *xin, int *err) {
+                                             const uint64_t *xf, const int32_t *xin, int *err) {
     const int64_t last = xoff[x + 1] - 1;
     const int32_t len = xin[x];
     int32_t l = 0, h = len;
@@ -1401,7 +1408,7 @@ __device__ __forceinline__ uint64_t in_value(int32_t x, int32_t y, const int64_t
         int32_t mid = (l + h) >> 1;
         if (xcol[last - mid] < y) l = mid + 1; else h = mid;
     }
-    if (l < len && xcol[last - l] == y) return xS[last - l].f;
+    if (l < len && xcol[last - l] == y) return xf[last - l];
     atomicOr(err, 16);
     return 0;
 }
@@ -1409,7 +1416,7 @@ __device__ __forceinline__ uint64_t in_value(int32_t x, int32_t y, const int64_t
 // where P3 takes an edge's values: both at the out-slot (mirror pass), or the reverse one
 // in the in-list of the higher-ranked end
 struct Rev {
-    const SigPair *xS;
+    const void *xS;                  // SigPair per slot, or (not mirrored) f alone
     const int64_t *xoff;
     const int32_t *xcol;
     const int32_t *xin;
@@ -1418,10 +1425,11 @@ struct Rev {
     // S(lo -> hi) and S(hi -> lo) for the G_x edge whose out-slot (lo -> hi) is `slot`
     __device__ __forceinline__ SigPair get(int64_t slot, int32_t hi, int32_t lo) const {
         if (mirrored) {
-            const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(xS + slot));
+            const ulonglong2 v = __ldg(static_cast<const ulonglong2 *>(xS) + slot);
             return SigPair{v.x, v.y};
         }
-        return SigPair{xS[slot].f, in_value(hi, lo, xoff, xcol, xS, xin, err)};
+        const uint64_t *xf = static_cast<const uint64_t *>(xS);
+        return SigPair{xf[slot], in_value(hi, lo, xoff, xcol, xf, xin, err)};
     }
 };
 
@@ -2347,16 +2355,22 @@ __global__ void __launch_bounds__(kThreads) init_kernel(InitArgs A) {
 // host orchestration
 // ======================================================================================
 // dynamic shared memory limits of the table kernels, set once per process
+template <class Slot>
+static int prepare_p2_kernels() {
+    RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<256, Slot>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
+    RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<512, Slot>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
+    RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<1024, Slot>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
+    RS_CUDA_TRY(cudaFuncSetAttribute(p2_mid_kernel<Slot>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2MidSmem));
+    return 0;
+}
 int rs::prepare_score_kernels() {
     static int done = 0;
     if (done) return 0;
     RS_CUDA_TRY(cudaFuncSetAttribute(p1_large_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kMidCap));
     RS_CUDA_TRY(cudaFuncSetAttribute(p1_large_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kMidCap));
     RS_CUDA_TRY(cudaFuncSetAttribute(p1_large_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kMidCap));
-    RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
-    RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
-    RS_CUDA_TRY(cudaFuncSetAttribute(p2_large_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * kMidCap));
-    RS_CUDA_TRY(cudaFuncSetAttribute(p2_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2MidSmem));
+    if (int rc = prepare_p2_kernels<SigPair>()) return rc;
+    if (int rc = prepare_p2_kernels<uint64_t>()) return rc;
     RS_CUDA_TRY(cudaFuncSetAttribute(p3_heavy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sizeof(P3Heavy)));
     RS_CUDA_TRY(cudaFuncSetAttribute(p1_small_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2373,12 +2387,12 @@ static void launch_p1_large(rs_graph *g, const Batch &B, int *err, size_t smem, 
         g->rsum, g->cl_col, g->cl_lab, g->wq + 1);
 }
 // p2_large over P2 list `list`, at most per_sm CTAs per SM
-template <int NT>
-static void launch_p2_large(rs_graph *g, const Batch &B, int *err, size_t smem, int list, int per_sm,
+template <int NT, class Slot>
+static void launch_p2_large(rs_graph *g, Slot *xS, const Batch &B, int *err, size_t smem, int list, int per_sm,
                             unsigned long long *wq, cudaStream_t st) {
-    p2_large_kernel<NT><<<grid_for(list == 3 ? g->n_large : g->n_mid + g->n_large, 1, per_sm), NT, smem, st>>>(
+    p2_large_kernel<NT, Slot><<<grid_for(list == 3 ? g->n_large : g->n_mid + g->n_large, 1, per_sm), NT, smem, st>>>(
         g->off, g->p2rows + p2_list_start(list, g->n_mid, g->n_large), g->p2cnt + list, B, g->LG, g->rec, g->rsum,
-        g->cl_col, g->cl_lab, g->acc, g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, err,
+        g->cl_col, g->cl_lab, g->acc, g->xoff, g->xcol, xS, g->xsk, g->xout, g->xin, g->xnode, err,
         Strict{g->col, g->sx}, wq);
 }
 
@@ -2395,6 +2409,8 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     int64_t n = g->n;
     if (!g->classified || g->dmax > g->tab_dmax)     // row lists or constant tables that are not there
         return fail(RS_EINVAL, "rs_score: the last change of the graph failed half way; repeat it (or rs_set_tuning) first");
+    if (!g->xS || g->xS_bytes != (g->tune.p3_mirror ? sizeof(SigPair) : sizeof(uint64_t)))
+        return fail(RS_EINVAL, "rs_score: the buffers of p3_mirror are missing (rs_set_tuning failed); set it again");
     g->scored_version = g->version;
     if (n == 0) return 0;
     constexpr int NT = kThreads;
@@ -2513,8 +2529,6 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     const int64_t nm = g->n_mid, nl = g->n_large;
     auto Lst = [&](int c) { return g->p2rows + p2_list_start(c, nm, nl); };
     int32_t *last_node = g->p2cnt + 8;
-    if (g->tune.p3_mirror && !g->xtile)
-        return fail(RS_EINVAL, "rs_score: p3_mirror is set but its tile table is missing");
     const int64_t gx_tiles = (n + kGxTile - 1) / kGxTile;
     const int split_blocks = mid_large ? grid_for(nm + nl, kGxThreads, 8) : 0;
     RS_CUDA_TRY(launch(chain, gx_offsets_kernel, (unsigned)(split_blocks + gx_tiles), kGxThreads, 0, s,
@@ -2534,57 +2548,62 @@ int rs::score_graph(rs_graph *g, double *scores, cudaStream_t s) {
     //      is issued first, so that its blocks are dispatched ahead of the other classes'
     plan({{3, g->n_hubs > 0}, {0, g->n_small > 0}, {1, mid_large}, {5, mid_large}, {2, mid_large}, {4, g->n_large > 0}});
     if (int rc = fork_aux(g, s, used)) return rc;
-    if (g->n_hubs) {
-        hub_p2_insert_kernel<NT><<<grid_for(g->n_hub_items, 1, 8), NT, 0, AX(3)>>>(
-            g->off, g->col, g->hubs, g->hub_items, g->hub_item_chunk, g->n_hub_items, g->tune.hub_chunk, g->rec,
-            g->hkey, g->hq,
-            g->hitem_out, g->hitem_in, g->hslot, err);
-        RS_LAUNCHED(g, AX(3), "hub_p2_insert");
-        hub_p2_counts_kernel<NT><<<(unsigned)((g->n_hubs + NT - 1) / NT), NT, 0, AX(3)>>>(
-            g->hubs, g->n_hubs, g->hitem_out, g->hitem_in, g->xoff, g->rec, g->xout, g->xin, g->xnode);
-        RS_LAUNCHED(g, AX(3), "hub_p2_counts");
-        hub_p2_emit_kernel<NT><<<grid_for(g->n_hub_items, 1, 8), NT, 0, AX(3)>>>(
-            g->off, g->col, g->hubs, g->hub_items, g->hub_item_chunk, g->n_hub_items, g->tune.hub_chunk, g->rec,
-            g->hslot,
-            g->hq, g->hsig, g->hitem_out, g->hitem_in, g->acc, g->xoff, g->xcol, g->xS, g->xsk, err, SX);
-        RS_LAUNCHED(g, AX(3), "hub_p2_emit");
-    }
-    if (g->n_small) {
-        if (few_rows)
-            RS_CUDA_TRY(launch(chain, p2_small_kernel<kNarrowRows>, grid_for(g->n_small * (32 / kNarrowRows), NT, cps), NT, 0, AX(0),
-            g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
-            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX));
-        else
-            p2_small_kernel<32><<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
-            g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
-            g->xoff, g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX);
-        RS_LAUNCHED(g, AX(0), "p2_small");
-    }
-    if (mid_large) {
-        // the mid and large rows with at most 32 cross neighbours, in the tile kernel
-        p2_small_kernel<kNarrowRows><<<grid_for((nm + nl) * (32 / kNarrowRows), NT, cps), NT, 0, AX(1)>>>(
-            g->off, Lst(0), 0, g->p2cnt + 0, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc, g->xoff,
-            g->xcol, g->xS, g->xsk, g->xout, g->xin, g->xnode, SX);
-        RS_LAUNCHED(g, AX(1), "p2_narrow");
-        p2_mid_kernel<<<grid_for((nm + nl) * 32, NT, 4), NT, kP2MidSmem, AX(5)>>>(
-            g->off, Lst(1), g->p2cnt + 1, B, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc, g->xoff, g->xcol,
-            g->xS, g->xsk, g->xout, g->xin, g->xnode, err, SX, g->wq + 2);
-        RS_LAUNCHED(g, AX(5), "p2_mid");
-        launch_p2_large<kP2SmallCta>(g, B, err, 32 * (size_t)kWarpCap, 2, 8, g->wq + 3, AX(2));
-        RS_LAUNCHED(g, AX(2), "p2_cta");
-    }
-    if (g->n_large) {
-        switch (g->tune.p2_cta_threads) {
-        case 256: launch_p2_large<256>(g, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
-        case 512: launch_p2_large<512>(g, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
-        default: launch_p2_large<1024>(g, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
+    auto p2 = [&](auto *xS) -> int {
+        using Slot = std::remove_pointer_t<decltype(xS)>;
+        if (g->n_hubs) {
+            hub_p2_insert_kernel<NT><<<grid_for(g->n_hub_items, 1, 8), NT, 0, AX(3)>>>(
+                g->off, g->col, g->hubs, g->hub_items, g->hub_item_chunk, g->n_hub_items, g->tune.hub_chunk, g->rec,
+                g->hkey, g->hq,
+                g->hitem_out, g->hitem_in, g->hslot, err);
+            RS_LAUNCHED(g, AX(3), "hub_p2_insert");
+            hub_p2_counts_kernel<NT><<<(unsigned)((g->n_hubs + NT - 1) / NT), NT, 0, AX(3)>>>(
+                g->hubs, g->n_hubs, g->hitem_out, g->hitem_in, g->xoff, g->rec, g->xout, g->xin, g->xnode);
+            RS_LAUNCHED(g, AX(3), "hub_p2_counts");
+            hub_p2_emit_kernel<NT, Slot><<<grid_for(g->n_hub_items, 1, 8), NT, 0, AX(3)>>>(
+                g->off, g->col, g->hubs, g->hub_items, g->hub_item_chunk, g->n_hub_items, g->tune.hub_chunk, g->rec,
+                g->hslot,
+                g->hq, g->hsig, g->hitem_out, g->hitem_in, g->acc, g->xoff, g->xcol, xS, g->xsk, err, SX);
+            RS_LAUNCHED(g, AX(3), "hub_p2_emit");
         }
-        RS_LAUNCHED(g, AX(4), "p2_large");
-    }
+        if (g->n_small) {
+            if (few_rows)
+                RS_CUDA_TRY(launch(chain, p2_small_kernel<kNarrowRows, Slot>, grid_for(g->n_small * (32 / kNarrowRows), NT, cps), NT, 0, AX(0),
+                g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
+                g->xoff, g->xcol, xS, g->xsk, g->xout, g->xin, g->xnode, SX));
+            else
+                p2_small_kernel<32, Slot><<<grid_for(g->n_small, NT, cps), NT, 0, AX(0)>>>(
+                g->off, g->rows_small, g->n_small, nullptr, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc,
+                g->xoff, g->xcol, xS, g->xsk, g->xout, g->xin, g->xnode, SX);
+            RS_LAUNCHED(g, AX(0), "p2_small");
+        }
+        if (mid_large) {
+            // the mid and large rows with at most 32 cross neighbours, in the tile kernel
+            p2_small_kernel<kNarrowRows, Slot><<<grid_for((nm + nl) * (32 / kNarrowRows), NT, cps), NT, 0, AX(1)>>>(
+                g->off, Lst(0), 0, g->p2cnt + 0, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc, g->xoff,
+                g->xcol, xS, g->xsk, g->xout, g->xin, g->xnode, SX);
+            RS_LAUNCHED(g, AX(1), "p2_narrow");
+            p2_mid_kernel<Slot><<<grid_for((nm + nl) * 32, NT, 4), NT, kP2MidSmem, AX(5)>>>(
+                g->off, Lst(1), g->p2cnt + 1, B, g->LG, g->rec, g->rsum, g->cl_col, g->cl_lab, g->acc, g->xoff, g->xcol,
+                xS, g->xsk, g->xout, g->xin, g->xnode, err, SX, g->wq + 2);
+            RS_LAUNCHED(g, AX(5), "p2_mid");
+            launch_p2_large<kP2SmallCta>(g, xS, B, err, 32 * (size_t)kWarpCap, 2, 8, g->wq + 3, AX(2));
+            RS_LAUNCHED(g, AX(2), "p2_cta");
+        }
+        if (g->n_large) {
+            switch (g->tune.p2_cta_threads) {
+            case 256: launch_p2_large<256>(g, xS, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
+            case 512: launch_p2_large<512>(g, xS, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
+            default: launch_p2_large<1024>(g, xS, B, err, p2_smem, 3, 2, g->wq + 6, AX(4)); break;
+            }
+            RS_LAUNCHED(g, AX(4), "p2_large");
+        }
+        return 0;
+    };
+    if (int rc = g->tune.p3_mirror ? p2(static_cast<SigPair *>(g->xS)) : p2(static_cast<uint64_t *>(g->xS))) return rc;
     if (int rc = join_aux(g, s, used)) return rc;
     // ---- P3: reverse values (mirror mode), then triangles
     if (g->tune.p3_mirror) {
-        RS_CUDA_TRY(launch(chain, gx_mirror_kernel, grid_for(g->nnz, kMirTile, cps), NT, 0, s, n, g->xoff, g->xcol, g->xS, g->xnode,
+        RS_CUDA_TRY(launch(chain, gx_mirror_kernel, grid_for(g->nnz, kMirTile, cps), NT, 0, s, n, g->xoff, g->xcol, static_cast<SigPair *>(g->xS), g->xnode,
                                                                        g->xin, g->xtile, last_node, g->xsk, err));
         RS_LAUNCHED(g, s, "gx_mirror");
     }

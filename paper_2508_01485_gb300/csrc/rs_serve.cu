@@ -72,7 +72,7 @@ struct BaseView {
     const int32_t *cl_col, *cl_lab;
     const int64_t *xoff;
     const int32_t *xcol;
-    const SigPair *xS;
+    SigSlots xS;
     const int32_t *xout, *xin;
     const uint64_t *LG;
     const double *RD;
@@ -513,7 +513,7 @@ __device__ __forceinline__ int64_t gx_slot(const BaseView &B, int32_t p, int32_t
 __device__ __forceinline__ uint64_t s_base(const BaseView &B, const SlotView &S, int32_t p, int32_t q) {
     int64_t sl = gx_slot(B, p, q);
     if (sl < 0) { atomicOr(S.err, 32); return 0; }
-    return B.xS[sl].f;
+    return B.xS.f(sl);
 }
 
 // S'(p -> q) after the removals
@@ -818,7 +818,7 @@ struct Base {
     BaseView view() const {
         BaseView v;
         v.n = n; v.k = k; v.off = g->off; v.col = g->col; v.lab = g->lab; v.rec = g->rec; v.rsum = g->rsum;
-        v.cl_col = g->cl_col; v.cl_lab = g->cl_lab; v.xoff = g->xoff; v.xcol = g->xcol; v.xS = g->xS;
+        v.cl_col = g->cl_col; v.cl_lab = g->cl_lab; v.xoff = g->xoff; v.xcol = g->xcol; v.xS = g->sig();
         v.xout = g->xout; v.xin = g->xin; v.LG = g->LG; v.RD = g->RD; v.rowmax = rowmax;
         return v;
     }

@@ -77,9 +77,11 @@ extern "C" rs_status rs_set_tuning(rs_graph *g, const rs_tuning *t, void *stream
     cudaStream_t s = as_stream(stream);
     rs_tuning old = g->tune;
     if (int rc = apply_tuning(g, *t, s)) {
-        g->tune = old;               // best effort: restore the previous split
+        g->tune = old;               // best effort: restore the previous buffers and split
+        const std::string why = rs_last_error();
+        set_mirror_buffer(g);
         reclassify(g, s);
-        return (rs_status)rc;
+        return (rs_status)fail(rc, why);
     }
     return RS_OK;
 }

@@ -4,7 +4,8 @@ what it copies, allocates and launches, and in which order.
 * the hub lists reach the device before the kernels that read them, on any stream;
 * an allocation that fails is reported, leaks nothing, and leaves nothing that a kernel would read;
 * a call that fails writes no out-parameter;
-* a server's slots and copies take the memory that its budget is charged for."""
+* a server's slots and copies take the memory that its budget is charged for;
+* a graph without the mirror pass holds 8 bytes less per entry."""
 import ctypes
 import os
 import shutil
@@ -78,6 +79,14 @@ class Calls:
         arr, srv = (ctypes.c_void_p * len(graphs))(*[g.value for g in graphs]), ctypes.c_void_p()
         assert self.lib.rs_server_create(arr, len(graphs), slots, ctypes.c_int64(budget), 4, mode, ctypes.byref(srv)) == 0
         return srv
+
+    def tune(self, g, **fields):
+        from paper_2508_01485_gb300 import _lib
+        t = _lib.Tuning()
+        assert self.lib.rs_get_tuning(g, ctypes.byref(t)) == 0
+        for k, v in fields.items():
+            setattr(t, k, v)
+        return self.lib.rs_set_tuning(g, ctypes.byref(t), self.s)
 
     def used(self, srv):
         used = ctypes.c_int64()
@@ -200,3 +209,41 @@ def test_memory_of_slots_and_copies(lib, calls, n):
     assert calls.poll(srv) == [(0, 0)]
     assert calls.used(srv) == slot + copy and lib.fake_live_bytes() - before <= copy - (16 << 20)
     lib.rs_server_free(srv)
+
+
+@pytest.mark.parametrize("n", [64, 10_000])
+def test_memory_without_the_mirror_pass(lib, calls, n):
+    lib.fake_classes(n, 0, 0, 0, DEGREE, 0, 0)
+    g, nnz = calls.build(n=n), n * DEGREE
+    calls.scores = np.zeros(n)
+    tiles = 4 * (nnz // 2048 + 2)
+    with_pass = lib.fake_live_bytes()
+    for _ in range(2):
+        assert calls.tune(g, p3_mirror=0) == 0 and lib.fake_live_bytes() == with_pass - 8 * nnz - tiles
+        assert calls.score(g) == 0
+        c = ctypes.c_void_p()
+        before = lib.fake_live_bytes()
+        lib.fake_classes(n - 2, 0, 0, 2, DEGREE, DEGREE, 3)      # (the hubs' scratch tables need more than 8 bytes a slot)
+        assert lib.rs_clone_graph(g, ctypes.byref(c), calls.s) == 0 and calls.score(c) == 0
+        lib.rs_free_graph(c)
+        assert lib.fake_live_bytes() == before
+        lib.fake_classes(n, 0, 0, 0, DEGREE, 0, 0)
+        assert calls.tune(g, p3_mirror=1) == 0 and lib.fake_live_bytes() == with_pass
+        assert calls.score(g) == 0
+    lib.rs_free_graph(g)
+
+
+@pytest.mark.parametrize("to", [0, 1])
+def test_a_failed_change_of_the_mirror_pass(lib, calls, to):
+    """Each allocation of the change failing: the setting before it stays, with its buffers."""
+    lib.fake_classes(N, 0, 0, 0, DEGREE, 0, 0)
+    g = calls.build()
+    assert calls.tune(g, p3_mirror=1 - to) == 0
+    held = lib.fake_live_bytes()
+    for n in range(1 + to):
+        lib.fake_fail_allocation(n)
+        assert calls.tune(g, p3_mirror=to) == 2                     # RS_ENOMEM
+        lib.fake_fail_allocation(-1)
+        assert lib.fake_live_bytes() == held and calls.score(g) == 0
+    assert calls.tune(g, p3_mirror=to) == 0 and calls.score(g) == 0
+    lib.rs_free_graph(g)
