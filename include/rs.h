@@ -382,7 +382,9 @@ rs_status rs_awcc(rs_graph *g, const int32_t *nodes, int64_t m, const int64_t *d
  *   returns its ticket.  No device work starts before rs_server_poll.
  * rs_server_poll -- start queued requests, in order, on free slots when the
  *   memory budget allows, and collect finished ones without waiting (block = 0)
- *   or until at least one finished or nothing is left (block != 0).  For each
+ *   or until at least one finished or nothing is left (block != 0).  Either way
+ *   a poll waits, before it returns, for the removals of the requests that it
+ *   has sent down the full path: their rescoring is launched by then.  For each
  *   of at most `max` finished requests: tickets[i], status[i] (RS_OK, or
  *   RS_EBUDGET when it could not fit), path[i] (1 incremental, 0 full; may be
  *   NULL), and its min(kmax, top_k) best (id, score) pairs at ids[i*kmax] and

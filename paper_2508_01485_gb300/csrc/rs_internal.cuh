@@ -336,9 +336,11 @@ int topk_prepare(rs_graph *g, int64_t n);
 int reclassify(rs_graph *g, cudaStream_t s);
 
 // rs_apply_removals in two halves: the first enqueues everything up to the copy of the class
-// counts (with the applied count) into `counts`, without waiting for the device when `counts` is
-// pinned; the second, called after s has reached that copy, builds what is sized by them.
-// Ids are the graph's own and in range.
+// counts (with the applied count) into `counts`; the second, called after s has reached that copy,
+// builds what is sized by them.  The first does not wait for the device when `counts` and the lists
+// are pinned and the lists have at most 4 n words: copies of pageable lists may wait for the work
+// before them on s, and longer lists take an allocation that is waited for (and, in the second half,
+// a free that waits for the device).  Ids are the graph's own and in range.
 constexpr int kCountWords = 16;
 struct Removal {
     int *counts = nullptr;      // kCountWords words of host memory

@@ -1873,7 +1873,7 @@ __global__ void __launch_bounds__(kP3Threads, kP3CtasPerSm) p3_list_kernel(
 // Issue slots and the latency of the loads bound it.  Before this form
 // (4-slot buckets read 16 bytes at a time, three double-float products and three fixed-point
 // conversions per triangle, c's sums by 64-bit shared atomics, which take five times as long
-// as 32-bit ones) it ran the shared-memory pipe at 74% and issue at 66%: 43.8 -> 36.5 ms on the
+// as 32-bit ones) it ran the shared-memory pipe at 74% and issue at 66%: 43.8 -> 36.2 ms on the
 // 8M-node graph (6.4e9 wedges, 2.1e9 triangles), 5.87 -> 4.52 ms on 2M nodes, where the pipe is
 // now at 41% and issue at 58%.
 //

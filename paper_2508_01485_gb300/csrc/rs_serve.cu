@@ -142,8 +142,8 @@ __device__ __forceinline__ void add_T(const SlotView &S, int32_t x) {
 
 // ---- 1. removals: dead entries and the touched rows ------------------------------
 // kMarkStripes warps per node, each over every kMarkStripes-th run of 32 entries (the removed
-// nodes are mostly large ones, and a warp each left a tail: 194 us per request of the serving
-// burst, against 20 us); a node listed twice is marked again to no effect
+// nodes are mostly large ones, and a warp each left a tail: 194 us per request of a burst of 24
+// requests on four graphs, against 20 us); a node listed twice is marked again to no effect
 constexpr int kMarkStripes = 16;
 __global__ void sv_mark_nodes(BaseView B, SlotView S, const int32_t *nodes, int64_t m) {
     int lane = threadIdx.x & 31;
@@ -606,8 +606,8 @@ __global__ void __launch_bounds__(kSvThreads) sv_tri_pairs(BaseView B, SlotView 
 //     as leave no warp without) and spreads the entries of their shorter lists, mostly a few each,
 //     over its lanes.  Its pairs lie
 //     far apart: those of one touched hub, which are neighbours, have the long lists
-//     (a burst of 24 requests: 7.26 ms with a warp per pair, 7.09 this way, 8.9 with 32
-//     neighbouring pairs per warp)
+//     (a burst of 24 requests, one draw of it: 7.26 ms with a warp per pair, 7.09 this way, 8.9 with
+//     32 neighbouring pairs per warp)
 struct PairTile {
     int32_t x[32], y[32];
     int32_t len[32];                 // inclusive sums of the walked lists' lengths
@@ -1093,7 +1093,9 @@ int64_t full_bytes_estimate(const Base &b) { return 38 * b.nnz + 170 * b.n + (16
 // full path: restore a copy of the base graph, apply the removals, rescore; in two halves,
 // because the rescoring's launches are sized by the row classes after the removals.  The server
 // launches other requests while the first half runs: waiting for it in place held the whole
-// queue up (6.3 of the 8.1 ms of a burst of 24 requests on 8 slots were such waits)
+// queue up (6.3 of the 8.1 ms of a burst of 24 requests on 8 slots were such waits; another draw of
+// requests than the one below).  The lists are copied from the request's own, pageable vectors,
+// which may make their copies wait for the restore before them
 int launch_full(rs_server *srv, Slot &sl, const Request &r) {
     Base &b = srv->bases[r.graph];
     cudaStream_t s = sl.s;
@@ -1114,7 +1116,7 @@ int finish_full(rs_server *srv, Slot &sl) {
     rs_graph *g = srv->copies[sl.copy].g;
     // beside other requests the row kernels take turns on the slot's stream: the requests fill the
     // GPU, and a stream per row class for each of them exceeds the device's hardware queues, whose
-    // streams then wait for one another (burst of 24 requests on 8 slots: 7.1 -> 6.8 ms); alone,
+    // streams then wait for one another (one draw of a burst of 24 requests on 8 slots: 7.1 -> 6.8 ms); alone,
     // or with streams chosen for the base graph, as for any graph
     int busy = 0;
     for (auto &o : srv->slots) busy += o.busy;
