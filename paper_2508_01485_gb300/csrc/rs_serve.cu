@@ -1086,7 +1086,7 @@ int launch_incremental(rs_server *srv, Slot &sl, const Request &r) {
 }
 
 // device bytes of a full copy of a base graph (CSR twice, cross lists, G_x slots
-// with both values, per-node records and workspaces: 37 bytes an entry and 153 a node, the rest
+// with both values, per-node records and workspaces: 37 bytes an entry and 152 a node, the rest
 // for hub lists and tables)
 int64_t full_bytes_estimate(const Base &b) { return 38 * b.nnz + 170 * b.n + (16 << 20); }
 
